@@ -70,7 +70,9 @@ struct ne_ctx {
     double *f64 = nullptr, *dF64 = nullptr, *rho = nullptr, *xi64 = nullptr;
     float* xi32 = nullptr;
     int *nbr = nullptr, *ncnt = nullptr, *sl = nullptr, *scnt = nullptr;
-    int *cellof = nullptr, *sorted = nullptr, *cstart = nullptr, *cfill = nullptr;
+    int *cellof = nullptr, *cslot = nullptr, *craw = nullptr, *cstart = nullptr, *ccount = nullptr;
+    float4* csort = nullptr;
+    unsigned* nl_done = nullptr;
     double *partA = nullptr, *partB = nullptr, *tot = nullptr, *W = nullptr, *scratch = nullptr;
     unsigned* tile_done = nullptr;
     int *flags = nullptr, *building = nullptr, *status = nullptr, *tile_rep = nullptr;
@@ -325,6 +327,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.n_rep = n_rep;
     B.n_tot = n_tot;
     B.n_tiles = n_tiles;
+    for (const RepDev& R : ctx->rep_h) B.n_max = std::max(B.n_max, R.n);
     B.tpa = ctx->tpa;
     B.rep = ctx->rep;
     B.tile_rep = ctx->tile_rep;
@@ -345,13 +348,16 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.sl = ctx->sl;
     B.scnt = ctx->scnt;
     B.cellof = ctx->cellof;
-    B.sorted = ctx->sorted;
+    B.cslot = ctx->cslot;
+    B.craw = ctx->craw;
+    B.csort = ctx->csort;
     B.cstart = ctx->cstart;
-    B.cfill = ctx->cfill;
+    B.ccount = ctx->ccount;
     B.partA = ctx->partA;
     B.partB = ctx->partB;
     B.tot = ctx->tot;
     B.tile_done = ctx->tile_done;
+    B.nl_done = ctx->nl_done;
     B.W = a.W;
     B.Wcum = a.Wcum;
     B.trace = a.trace;
@@ -616,9 +622,12 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->sl, N * NE_SMAX));
     A(dalloc(&ctx->scnt, N * 8));
     A(dalloc(&ctx->cellof, N));
-    A(dalloc(&ctx->sorted, N));
+    A(dalloc(&ctx->cslot, N));
+    A(dalloc(&ctx->craw, N));
+    A(dalloc(&ctx->csort, N));
     A(dalloc(&ctx->cstart, (size_t)ctx->cells_cap + R));
-    A(dalloc(&ctx->cfill, (size_t)ctx->cells_cap));
+    A(dalloc(&ctx->ccount, (size_t)ctx->cells_cap));
+    A(dalloc(&ctx->nl_done, R));
     A(dalloc(&ctx->partA, (size_t)ctx->tiles_cap * NPA));
     A(dalloc(&ctx->partB, (size_t)ctx->tiles_cap * NPB));
     A(dalloc(&ctx->tot, R * NTOT));
@@ -641,6 +650,10 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->st_vec, R * 4 * NE_STENCIL_MAX));
     A(dalloc(&ctx->st_dist, R * 4 * NE_STENCIL_MAX));
     if (ok) ok = cudaMemset(ctx->rebuilds, 0, sizeof(unsigned long long)) == cudaSuccess;
+    // the list build leaves these at zero
+    if (ok) ok = cudaMemset(ctx->ccount, 0, sizeof(int) * (size_t)ctx->cells_cap) == cudaSuccess;
+    if (ok) ok = cudaMemset(ctx->nl_done, 0, sizeof(unsigned) * R) == cudaSuccess;
+    if (ok) ok = cudaMemset(ctx->building, 0, sizeof(int) * R) == cudaSuccess;
     if (!ok) {
         ne_ctx_destroy(ctx);
         return NE_ENOMEM;
@@ -667,8 +680,8 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
     if (!ctx) return NE_EINVAL;
     void* ptrs[] = {ctx->theta, ctx->pf32, ctx->pf64, ctx->F32, ctx->F64, ctx->pos32, ctx->posF,
                     ctx->pbuild, ctx->f32, ctx->f64, ctx->dF64, ctx->rho, ctx->xi64, ctx->xi32,
-                    ctx->nbr, ctx->ncnt, ctx->sl, ctx->scnt, ctx->cellof, ctx->sorted, ctx->cstart,
-                    ctx->cfill, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
+                    ctx->nbr, ctx->ncnt, ctx->sl, ctx->scnt, ctx->cellof, ctx->cslot, ctx->craw, ctx->csort,
+                    ctx->cstart, ctx->ccount, ctx->nl_done, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
                     ctx->tile_done, ctx->flags, ctx->building, ctx->status, ctx->tile_rep, ctx->rep, ctx->step_ctr, ctx->rebuilds, ctx->xrep, ctx->work, ctx->st_vec, ctx->st_dist, ctx->lam_tab,
                     ctx->bins};
     for (void* p : ptrs)

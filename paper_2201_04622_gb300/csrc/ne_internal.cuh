@@ -9,6 +9,7 @@
 //   f32 / f64           EAM forces, float4 [N] (mixed) or double [N][3]
 //   dF64                double [N]      F'(rho) (FP64 path)
 //   xi32 / xi64         Langevin normals of the current step, [N][3]
+//   csort               float4 [N]      pbuild sorted by cell, .w the atom's index in its replica
 //   nbr, ncnt           candidate list within r_c + skin, int, lane-interleaved:
 //                       entry k of atom i at ((k / TPA) * N + i) * TPA + k % TPA
 //   sl, scnt            per-step short list (r < r_c) in the same layout, one
@@ -102,6 +103,7 @@ struct Tables {
 
 struct DevBatch {
     int n_rep, n_tot, n_tiles, tpa;
+    int n_max;         // atoms of the largest replica
     const RepDev* rep;
     const int* tile_rep;
     double* x;
@@ -121,19 +123,22 @@ struct DevBatch {
     int* sl;
     int* scnt;
     int* cellof;
-    int* sorted;
+    int* cslot;        // arrival order of each atom in its cell (list build)
+    int* craw;         // atoms by cell, unsorted inside a cell (list build)
+    float4* csort;
     int* cstart;
-    int* cfill;
+    int* ccount;       // atoms per cell; zero between list builds
     double* partA;
     double* partB;
     double* tot;
     unsigned* tile_done;
+    unsigned* nl_done;
     double* W;         // [n_rep][2]
     double* Wcum;      // nullable, [n_rep][2][t_s + 1]
     double* trace;     // nullable, [rows][8], single replica
     int trace_stride, trace_rows;
     int* flags;        // [n_rep] list rebuild requested (set by the step kernel)
-    int* building;     // [n_rep] rebuild in progress this step
+    int* building;     // [n_rep] rebuild in progress (set by the binning, cleared by pass 1)
     unsigned long long* rebuilds;  // count of replica list builds
     int* status;
     Tables tab;
@@ -284,24 +289,6 @@ __device__ __forceinline__ double ne_warp_tile_sum(const double* part, int nq, i
 __device__ __forceinline__ void ne_set_status(int* status, int bits)
 {
     atomicOr(status, bits);
-}
-
-// Fixed-order block sum of NV doubles per thread into out[NV] (thread 0).
-template <int NV>
-__device__ inline void ne_block_sum(double (&val)[NV], double* out, double* scratch)
-{
-    // scratch: blockDim.x * NV doubles
-    const int t = threadIdx.x;
-    for (int q = 0; q < NV; ++q) scratch[q * blockDim.x + t] = val[q];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (t < w)
-            for (int q = 0; q < NV; ++q) scratch[q * blockDim.x + t] += scratch[q * blockDim.x + t + w];
-        __syncthreads();
-    }
-    if (t == 0)
-        for (int q = 0; q < NV; ++q) out[q] = scratch[q * blockDim.x];
-    __syncthreads();
 }
 
 // Launch helpers (defined in the kernel translation units).

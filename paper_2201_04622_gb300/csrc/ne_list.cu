@@ -1,0 +1,274 @@
+// ne_list.cu -- neighbour-list build of the multi-kernel path.
+//
+// Rebuild of the candidate list of every replica whose flag is set (or of all
+// replicas, when forced), in two launches that return at once when there is
+// nothing to do:
+//   k_nl_cells  reference positions (the lattice sites at the start of a run,
+//               the current positions after an atom strayed more than
+//               skin / 2), wrapped and binned into cells of edge >= r_c + skin.
+//               One thread per atom over all SMs; the block that finishes a
+//               replica's last tile forms its cell starts and writes the atoms
+//               sorted by cell, each cell's by index, so the order does not
+//               depend on the atomics;
+//   k_nl_list   for each atom the atoms of the 27 surrounding cells (all atoms
+//               when the box holds < 3 cells per axis) within r_c + skin,
+//               minimum image, FP32 distances with a 1e-3 A margin so that
+//               rounding never drops a pair.
+#include "ne_internal.cuh"
+
+namespace {
+
+__device__ __forceinline__ double wrap(double x, double L, double invL) { return x - L * floor(x * invL); }
+
+constexpr int CELL_THREADS = 1024;
+constexpr int CELL_TILES = CELL_THREADS / NE_TILE;
+
+// replicas above this size have their cells sorted by a launch of its own
+// (k_nl_sort): with one block's pass over 70,304 atoms the FP64 energy call
+// took 1049 us, with the launch 973; below, the launch, paid at every step,
+// costs more than it saves
+constexpr int SORT_IN_BLOCK = 16384;
+
+// Atoms first, first + step, ... (in cell order) of a replica into the sorted
+// copy: an atom's place in its cell is the number of lower indices there.
+__device__ __forceinline__ void rank_cells(const DevBatch& B, int rep, int first, int step)
+{
+    const RepDev& P = B.rep[rep];
+    const int n = P.n, off = P.off;
+    const int* start = B.cstart + P.cell_off + rep;
+    for (int p = first; p < n; p += step) {
+        const int a = B.craw[off + p];
+        const int c = __ldcg(&B.cellof[off + a]);
+        const float4 x = __ldcg(&B.pbuild[off + a]);
+        const int lo = start[c], hi = start[c + 1];
+        int r = 0;
+#pragma unroll 4
+        for (int q = lo; q < hi; ++q) r += B.craw[off + q] < a;
+        B.csort[off + lo + r] = make_float4(x.x, x.y, x.z, __int_as_float(a));
+    }
+}
+
+// Cell starts and the atoms by cell (and, for a replica that one block sorts,
+// the sorted copy) of one replica whose atoms are all counted, by the whole
+// block.
+__device__ void sort_cells(const DevBatch& B, int rep, int* s_warp)
+{
+    const RepDev& P = B.rep[rep];
+    const int tid = threadIdx.x, n = P.n, off = P.off;
+    const int ncell = P.nc[0] * P.nc[1] * P.nc[2];
+    int* start = B.cstart + P.cell_off + rep;  // ncell + 1 entries
+    int* count = B.ccount + P.cell_off;
+    // exclusive scan of the counts: each thread a contiguous chunk of cells,
+    // warp scans over the chunk totals, then over the warps
+    const int per = (ncell + CELL_THREADS - 1) / CELL_THREADS;
+    const int c0 = min(ncell, tid * per), c1 = min(ncell, c0 + per);
+    int tot = 0;
+    for (int c = c0; c < c1; ++c) tot += __ldcg(&count[c]);
+    int inc = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if ((tid & 31) >= o) inc += v;
+    }
+    if ((tid & 31) == 31) s_warp[tid >> 5] = inc;
+    __syncthreads();
+    if (tid < 32) {
+        int v = s_warp[tid];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int w = __shfl_up_sync(0xffffffffu, v, o);
+            if (tid >= o) v += w;
+        }
+        s_warp[tid] = v;
+    }
+    __syncthreads();
+    int run = inc - tot + (tid >= 32 ? s_warp[(tid >> 5) - 1] : 0);
+    for (int c = c0; c < c1; ++c) {
+        const int k = __ldcg(&count[c]);
+        start[c] = run;
+        run += k;
+        count[c] = 0;  // zero for the next build
+    }
+    if (tid == 0) start[ncell] = n;
+    __syncthreads();
+    for (int a0 = tid; a0 < n; a0 += 8 * CELL_THREADS) {
+        int c[8], k[8];  // eight atoms in flight: the chain is cell -> start -> store
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int a = min(a0 + q * CELL_THREADS, n - 1);
+            c[q] = __ldcg(&B.cellof[off + a]);
+            k[q] = __ldcg(&B.cslot[off + a]);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) k[q] += start[c[q]];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (a0 + q * CELL_THREADS < n) B.craw[off + k[q]] = a0 + q * CELL_THREADS;
+    }
+    __syncthreads();
+    if (n <= SORT_IN_BLOCK) rank_cells(B, rep, tid, CELL_THREADS);
+}
+
+// Bound by latency: one thread per atom does the FP64 wrap and one atomic,
+// then the finishing block scans and scatters its replica's atoms.  Before, one
+// 512-thread block counted, scanned and sorted each cell by insertion (176 us
+// for 65,536 atoms, 40 us for 2000) and one thread an atom walked its cells
+// (176 and 253 us).  Whole calls, before and now: energy and forces of 70,304
+// atoms in FP64 1232 -> 973 us, energy and gradients of 65,536 atoms 1504 ->
+// 1091 us, the 200-step spring fit of 2000 atoms at 1400 K 17.0 -> 13.6 ms.
+__global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force, int from_sites)
+{
+    __shared__ int s_warp[32];
+    __shared__ int s_done[CELL_TILES];  // replica whose last tile this block finished, or -1
+    const int tl = threadIdx.x / NE_TILE;
+    const int tile = blockIdx.x * CELL_TILES + tl;
+    const int rep = tile < B.n_tiles ? B.tile_rep[tile] : 0;
+    const bool go = tile < B.n_tiles && (force || B.flags[rep] != 0);
+    if (!__syncthreads_or(go)) return;
+    const RepDev& P = B.rep[rep];
+    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x % NE_TILE;
+    if (go && a < P.n) {
+        const int i = P.off + a;
+        const double* X = from_sites ? B.x0 : B.x;
+        double w[3];
+        for (int d = 0; d < 3; ++d) w[d] = wrap(X[3 * i + d], P.L[d], P.invL[d]);
+        const float4 p = make_float4((float)w[0], (float)w[1], (float)w[2], __int_as_float(a));
+        B.pbuild[i] = p;
+        if (P.nc[0] == 0) {
+            B.csort[i] = p;  // all pairs: the atoms in index order
+        } else {
+            int c3[3];
+            for (int d = 0; d < 3; ++d) {
+                const int q = (int)(w[d] * P.invL[d] * P.nc[d]);
+                c3[d] = min(max(q, 0), P.nc[d] - 1);
+            }
+            const int c = (c3[0] * P.nc[1] + c3[1]) * P.nc[2] + c3[2];
+            B.cellof[i] = c;
+            B.cslot[i] = atomicAdd(&B.ccount[P.cell_off + c], 1);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x % NE_TILE == 0) {
+        int done = -1;
+        if (go) {
+            __threadfence();  // this tile's writes before its ticket
+            if (atomicAdd(&B.nl_done[rep], 1u) == (unsigned)P.ntile - 1u) {
+                __threadfence();
+                B.nl_done[rep] = 0u;
+                B.flags[rep] = 0;  // every tile has read it
+                B.building[rep] = 1;
+                atomicAdd(B.rebuilds, 1ull);
+                if (P.nc[0] != 0) done = rep;
+            }
+        }
+        s_done[tl] = done;
+    }
+    __syncthreads();
+    for (int q = 0; q < CELL_TILES; ++q) {
+        if (s_done[q] >= 0) sort_cells(B, s_done[q], s_warp);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
+{
+    const int tile = blockIdx.x * (256 / NE_TILE) + threadIdx.x / NE_TILE;
+    if (tile >= B.n_tiles) return;
+    const int rep = B.tile_rep[tile];
+    const RepDev& P = B.rep[rep];
+    if (!B.building[rep] || P.nc[0] == 0 || P.n <= SORT_IN_BLOCK) return;
+    rank_cells(B, rep, (tile - P.tile0) * NE_TILE + threadIdx.x % NE_TILE, P.ntile * NE_TILE);
+}
+
+// G lanes per atom walk its 27 cells: the z neighbours of a cell are one run
+// of the sorted copy (two at the box edge), so the lanes read consecutive
+// 16-byte entries, and a ballot packs the lanes' hits in order.
+constexpr int LIST_THREADS = 256;
+
+template <int G>
+__global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
+{
+    constexpr int AT = LIST_THREADS / G, SUB = NE_TILE / AT;
+    const int tile = blockIdx.x / SUB;
+    const int rep = B.tile_rep[tile];
+    if (!B.building[rep]) return;
+    const RepDev& P = B.rep[rep];
+    const int lane = threadIdx.x % G;
+    const int a = (tile - P.tile0) * NE_TILE + (blockIdx.x % SUB) * AT + threadIdx.x / G;
+    const bool valid = a < P.n;
+    const int off = P.off, i = off + (valid ? a : 0);
+    const float L0 = (float)P.L[0], L1 = (float)P.L[1], L2 = (float)P.L[2];
+    const float iL0 = (float)P.invL[0], iL1 = (float)P.invL[1], iL2 = (float)P.invL[2];
+    const float rl = sqrtf((float)P.rlist2) + 1e-3f;
+    const float rl2 = rl * rl;
+    const float4 pi = B.pbuild[i];
+    const int gsh = (threadIdx.x & 31) / G * G;  // this atom's first lane in the warp
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
+    int cnt = 0;
+    // entries [lo, hi) of the sorted copy (empty for a lane group with no atom)
+    auto scan = [&](int lo, int hi) {
+        const int trips = __reduce_max_sync(0xffffffffu, (unsigned)(hi > lo ? (hi - lo + G - 1) / G : 0));
+        for (int t = 0; t < trips; ++t) {
+            const int p = lo + t * G + lane;
+            bool hit = false;
+            int b = 0;
+            if (p < hi) {
+                const float4 pj = B.csort[off + p];
+                b = __float_as_int(pj.w);
+                float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+                dx -= L0 * rintf(dx * iL0);
+                dy -= L1 * rintf(dy * iL1);
+                dz -= L2 * rintf(dz * iL2);
+                hit = b != a && dx * dx + dy * dy + dz * dz < rl2;
+            }
+            const unsigned m = (__ballot_sync(0xffffffffu, hit) >> gsh) & gmask;
+            const int at = cnt + __popc(m & ((1u << lane) - 1u));
+            if (hit && at < NE_NMAX) B.nbr[ne_nbr_index(at, i, B.n_tot, B.tpa)] = off + b;
+            cnt += __popc(m);
+        }
+    };
+    if (P.nc[0] == 0) {
+        scan(0, valid ? P.n : 0);
+    } else {
+        const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
+        const int* start = B.cstart + P.cell_off + rep;
+        const int c = valid ? B.cellof[i] : 0;
+        const int cx = c / (nc1 * nc2), cy = (c / nc2) % nc1, cz = c % nc2;
+        // z cells cz - 1 .. cz + 1 in order: [z0, z1) and, across the edge, [z2, z3)
+        int z0 = cz - 1, z1 = cz + 2, z2 = 0, z3 = 0;
+        if (cz == 0) z0 = nc2 - 1, z1 = nc2, z3 = 2;
+        if (cz == nc2 - 1) z1 = nc2, z3 = 1;
+#pragma unroll 1
+        for (int r = 0; r < 9; ++r) {
+            const int o = (((cx + r / 3 - 1 + nc0) % nc0) * nc1 + (cy + r % 3 - 1 + nc1) % nc1) * nc2;
+            scan(valid ? start[o + z0] : 0, valid ? start[o + z1] : 0);
+            if (__any_sync(0xffffffffu, z3 > 0)) {
+                const bool two = valid && z3 > 0;
+                scan(two ? start[o + z2] : 0, two ? start[o + z3] : 0);
+            }
+        }
+    }
+    if (valid && lane == 0) {
+        if (cnt > NE_NMAX) ne_set_status(B.status, ST_ENEIGH);
+        B.ncnt[i] = min(cnt, NE_NMAX);
+    }
+}
+
+}  // namespace
+
+namespace ne {
+
+void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t st)
+{
+    k_nl_cells<<<(B.n_tiles + CELL_TILES - 1) / CELL_TILES, CELL_THREADS, 0, st>>>(B, force, from_sites);
+    if (B.n_max > SORT_IN_BLOCK)
+        k_nl_sort<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
+    // a warp an atom up to 8192 atoms (a quarter of a million threads, one
+    // wave), eight lanes above: fewer idle lanes at the ends of the short runs
+    if (B.n_tot <= 8192)
+        k_nl_list<32><<<B.n_tiles * (NE_TILE * 32 / LIST_THREADS), LIST_THREADS, 0, st>>>(B);
+    else
+        k_nl_list<8><<<B.n_tiles * (NE_TILE * 8 / LIST_THREADS), LIST_THREADS, 0, st>>>(B);
+}
+
+}  // namespace ne

@@ -1,184 +1,12 @@
-// ne_md.cu -- dynamics kernels of libne.so: neighbour-list build, the fused
-// lambda-blend + Einstein spring + work increment + BAOAB Langevin step,
-// Maxwell-Boltzmann initial velocities, the spring energy, and small
-// reductions (msd samples, exported energies/forces).
+// ne_md.cu -- dynamics kernels of libne.so: the fused lambda-blend + Einstein
+// spring + work increment + BAOAB Langevin step, Maxwell-Boltzmann initial
+// velocities, the spring energy, and small reductions (msd samples, exported
+// energies/forces).
 #include "ne_internal.cuh"
 
 namespace {
 
 __device__ __forceinline__ double wrap(double x, double L, double invL) { return x - L * floor(x * invL); }
-
-// ------------------------------------------------------------ neighbours
-// Rebuild of the candidate list of every replica whose flag is set (or of
-// all replicas, when forced), in two launches:
-//   k_nl_bin   one block per replica: reference positions (the lattice
-//              sites at the start of a run, the current positions after an
-//              atom strayed more than skin/2), wrapped; cell binning with
-//              cells of edge >= r_c + skin; counting sort by cell (count,
-//              exclusive scan, scatter) and an insertion sort inside each
-//              cell so the order does not depend on the atomics;
-//   k_nl_list  one thread per atom on every SM: all atoms of the 27
-//              surrounding cells (all atoms when the box holds < 3 cells per
-//              axis) within r_c + skin, minimum image, FP32 distances with a
-//              1e-3 A margin so that rounding never drops a pair.
-// Both return at once for replicas that need no rebuild.  The per-atom part
-// of the binning (wrapped position, cell in FP64) runs first in k_nl_prep,
-// one block per tile, so a large replica's FP64 work spreads over the SMs.
-__global__ void __launch_bounds__(NE_TILE) k_nl_prep(DevBatch B, int force, int from_sites)
-{
-    const int tile = blockIdx.x;
-    const int rep = B.tile_rep[tile];
-    if (!(force || B.flags[rep] != 0)) return;
-    const RepDev& P = B.rep[rep];
-    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x;
-    if (a >= P.n) return;
-    const int i = P.off + a;
-    const double* X = from_sites ? B.x0 : B.x;
-    double w[3];
-    for (int d = 0; d < 3; ++d) w[d] = wrap(X[3 * i + d], P.L[d], P.invL[d]);
-    B.pbuild[i] = make_float4((float)w[0], (float)w[1], (float)w[2], 0.f);
-    if (P.nc[0] == 0) return;
-    int c3[3];
-    for (int d = 0; d < 3; ++d) {
-        const int q = (int)(w[d] * P.invL[d] * P.nc[d]);
-        c3[d] = min(max(q, 0), P.nc[d] - 1);
-    }
-    B.cellof[i] = (c3[0] * P.nc[1] + c3[1]) * P.nc[2] + c3[2];
-}
-
-__global__ void __launch_bounds__(512) k_nl_bin(DevBatch B, int force, int from_sites)
-{
-    const int rep = blockIdx.x;
-    const RepDev& P = B.rep[rep];
-    const int tid = threadIdx.x, bs = blockDim.x;
-    const int go = force || B.flags[rep] != 0;
-    __syncthreads();
-    if (tid == 0) {
-        B.building[rep] = go;
-        B.flags[rep] = 0;
-        if (go) atomicAdd(B.rebuilds, 1ull);
-    }
-    if (!go) return;
-    (void)from_sites;  // positions were wrapped and binned by k_nl_prep
-    const int n = P.n, off = P.off;
-    if (P.nc[0] == 0) return;
-    const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
-    const int ncell = nc0 * nc1 * nc2;
-    int* start = B.cstart + P.cell_off + rep;  // ncell + 1 entries
-    int* fill = B.cfill + P.cell_off;
-    for (int c = tid; c <= ncell; c += bs) start[c] = 0;
-    for (int c = tid; c < ncell; c += bs) fill[c] = 0;
-    __syncthreads();
-    for (int a = tid; a < n; a += bs) atomicAdd(&start[B.cellof[off + a] + 1], 1);
-    __syncthreads();
-    // inclusive scan of start[1..ncell] by the whole block: each thread sums
-    // a contiguous chunk of cells, a shared-memory scan over the chunk
-    // totals gives each chunk's offset, then each thread writes its chunk
-    {
-        __shared__ int s_chunk[512];
-        const int per = (ncell + bs - 1) / bs;
-        const int c0 = 1 + tid * per, c1 = min(ncell + 1, c0 + per);
-        int tot = 0;
-        for (int c = c0; c < c1; ++c) tot += start[c];
-        s_chunk[tid] = tot;
-        __syncthreads();
-        for (int o = 1; o < bs; o <<= 1) {  // Hillis-Steele inclusive scan over the chunk totals
-            const int v = tid >= o ? s_chunk[tid - o] : 0;
-            __syncthreads();
-            s_chunk[tid] += v;
-            __syncthreads();
-        }
-        int run = tid > 0 ? s_chunk[tid - 1] : 0;
-        for (int c = c0; c < c1; ++c) {
-            run += start[c];
-            start[c] = run;
-        }
-    }
-    __syncthreads();
-    for (int a = tid; a < n; a += bs) {
-        const int c = B.cellof[off + a];
-        const int pos = atomicAdd(&fill[c], 1);
-        B.sorted[off + start[c] + pos] = a;
-    }
-    __syncthreads();
-    // sort each cell's atoms by index: in a thread-local copy when the cell
-    // holds at most NE_CELL_LOCAL atoms (the common case), else in place
-    constexpr int NE_CELL_LOCAL = 64;
-    for (int c = tid; c < ncell; c += bs) {
-        int* sl = B.sorted + off + start[c];
-        const int len = start[c + 1] - start[c];
-        if (len <= NE_CELL_LOCAL) {
-            int loc[NE_CELL_LOCAL];
-            for (int p = 0; p < len; ++p) {
-                const int key = sl[p];
-                int q = p - 1;
-                while (q >= 0 && loc[q] > key) {
-                    loc[q + 1] = loc[q];
-                    --q;
-                }
-                loc[q + 1] = key;
-            }
-            for (int p = 0; p < len; ++p) sl[p] = loc[p];
-        } else {
-            for (int p = 1; p < len; ++p) {
-                int key = sl[p], q = p - 1;
-                while (q >= 0 && sl[q] > key) {
-                    sl[q + 1] = sl[q];
-                    --q;
-                }
-                sl[q + 1] = key;
-            }
-        }
-    }
-}
-
-__global__ void __launch_bounds__(NE_TILE) k_nl_list(DevBatch B)
-{
-    const int tile = blockIdx.x;
-    const int rep = B.tile_rep[tile];
-    if (!B.building[rep]) return;
-    const RepDev& P = B.rep[rep];
-    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x;
-    if (a >= P.n) return;
-    const int off = P.off, i = off + a, tpa = B.tpa;
-    const float L0 = (float)P.L[0], L1 = (float)P.L[1], L2 = (float)P.L[2];
-    const float iL0 = (float)P.invL[0], iL1 = (float)P.invL[1], iL2 = (float)P.invL[2];
-    const float rl = sqrtf((float)P.rlist2) + 1e-3f;
-    const float rl2 = rl * rl;
-    const float4 pi = B.pbuild[i];
-    int cnt = 0, bad = 0;
-    auto test = [&](int b) {
-        if (b == a) return;
-        const int j = off + b;
-        const float4 pj = B.pbuild[j];
-        float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-        dx -= L0 * rintf(dx * iL0);
-        dy -= L1 * rintf(dy * iL1);
-        dz -= L2 * rintf(dz * iL2);
-        if (dx * dx + dy * dy + dz * dz < rl2) {
-            if (cnt < NE_NMAX) B.nbr[ne_nbr_index(cnt, i, B.n_tot, tpa)] = j;
-            ++cnt;
-        }
-    };
-    if (P.nc[0] == 0) {
-        for (int b = 0; b < P.n; ++b) test(b);
-    } else {
-        const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
-        const int* start = B.cstart + P.cell_off + rep;
-        const int c = B.cellof[i];
-        const int cx = c / (nc1 * nc2), cy = (c / nc2) % nc1, cz = c % nc2;
-        for (int dx = -1; dx <= 1; ++dx)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dz = -1; dz <= 1; ++dz) {
-                    const int o = (((cx + dx + nc0) % nc0) * nc1 + (cy + dy + nc1) % nc1) * nc2 +
-                                  (cz + dz + nc2) % nc2;
-                    for (int p = start[o]; p < start[o + 1]; ++p) test(B.sorted[off + p]);
-                }
-    }
-    if (cnt > NE_NMAX) bad |= ST_ENEIGH;
-    B.ncnt[i] = min(cnt, NE_NMAX);
-    if (bad) ne_set_status(B.status, bad);
-}
 
 // ------------------------------------------------------------ fused step
 // Total force of H(lambda) on atom i from the EAM force F0, the spring force
@@ -819,13 +647,6 @@ __global__ void __launch_bounds__(256) k_msd_sample_species(DevBatch B, double* 
 }  // namespace
 
 namespace ne {
-
-void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t st)
-{
-    k_nl_prep<<<B.n_tiles, NE_TILE, 0, st>>>(B, force, from_sites);
-    k_nl_bin<<<B.n_rep, 512, 0, st>>>(B, force, from_sites);
-    k_nl_list<<<B.n_tiles, NE_TILE, 0, st>>>(B);
-}
 
 void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base, int j,
                  int do_close, int do_open, cudaStream_t st)

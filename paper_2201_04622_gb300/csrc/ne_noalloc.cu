@@ -45,16 +45,18 @@ constexpr size_t O_NCNT = O_NBR + up(sizeof(int) * (size_t)NA * NE_NMAX);
 constexpr size_t O_SL = O_NCNT + up(sizeof(int) * NA);
 constexpr size_t O_SCNT = O_SL + up(sizeof(int) * (size_t)NA * NE_SMAX);
 constexpr size_t O_CELLOF = O_SCNT + up(sizeof(int) * NA * TPA);
-constexpr size_t O_SORTED = O_CELLOF + up(sizeof(int) * NA);
-constexpr size_t O_CSTART = O_SORTED + up(sizeof(int) * NA);
-constexpr size_t O_CFILL = O_CSTART + up(sizeof(int) * (CELLS + 1));
-constexpr size_t O_PARTA = O_CFILL + up(sizeof(int) * CELLS);
+constexpr size_t O_CSLOT = O_CELLOF + up(sizeof(int) * NA);
+constexpr size_t O_CRAW = O_CSLOT + up(sizeof(int) * NA);
+constexpr size_t O_CSORT = O_CRAW + up(sizeof(int) * NA);
+constexpr size_t O_CSTART = O_CSORT + up(sizeof(float4) * NA);
+constexpr size_t O_CCOUNT = O_CSTART + up(sizeof(int) * (CELLS + 1));
+constexpr size_t O_PARTA = O_CCOUNT + up(sizeof(int) * CELLS);
 constexpr size_t O_PARTB = O_PARTA + up(sizeof(double) * TILES * NPA);
 constexpr size_t O_TOT = O_PARTB + up(sizeof(double) * TILES * NPB);
 constexpr size_t O_REP = O_TOT + up(sizeof(double) * NTOT);
 constexpr size_t O_TILEREP = O_REP + up(sizeof(RepDev));
 constexpr size_t O_SMALL = O_TILEREP + up(sizeof(int) * TILES);
-// small words: tile_done, flags, building, status (ints), rebuilds, step counter (8 bytes)
+// small words: tile_done, flags, building, status (ints), rebuilds, step counter (8 bytes), nl_done
 constexpr size_t O_END = O_SMALL + 256;
 static_assert(O_END <= NE_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds NE_NOALLOC_SCRATCH_BYTES");
 
@@ -180,6 +182,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     DevBatch B{};
     B.n_rep = 1;
     B.n_tot = n;
+    B.n_max = n;
     B.n_tiles = R.ntile;
     B.tpa = TPA;
     B.rep = (const RepDev*)(base + O_REP);
@@ -196,9 +199,11 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     B.sl = (int*)(base + O_SL);
     B.scnt = (int*)(base + O_SCNT);
     B.cellof = (int*)(base + O_CELLOF);
-    B.sorted = (int*)(base + O_SORTED);
+    B.cslot = (int*)(base + O_CSLOT);
+    B.craw = (int*)(base + O_CRAW);
+    B.csort = (float4*)(base + O_CSORT);
     B.cstart = (int*)(base + O_CSTART);
-    B.cfill = (int*)(base + O_CFILL);
+    B.ccount = (int*)(base + O_CCOUNT);
     B.partA = (double*)(base + O_PARTA);
     B.partB = (double*)(base + O_PARTB);
     B.tot = (double*)(base + O_TOT);
@@ -209,6 +214,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     B.status = small + 3;
     B.rebuilds = (unsigned long long*)(base + O_SMALL + 16);
     long long* step_ctr = (long long*)(base + O_SMALL + 24);
+    B.nl_done = (unsigned*)(base + O_SMALL + 32);
     B.trace_stride = 1;
     Tables& t = B.tab;
     t.pf32 = (const float4*)(base + O_PF32);
@@ -233,6 +239,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
         cudaMemcpyAsync(base + O_TILEREP, tile_rep, sizeof(int) * R.ntile, cudaMemcpyHostToDevice, st) !=
             cudaSuccess ||
         cudaMemsetAsync(base + O_SMALL, 0, 256, st) != cudaSuccess ||
+        cudaMemsetAsync(base + O_CCOUNT, 0, sizeof(int) * CELLS, st) != cudaSuccess ||
         cudaMemsetAsync(base + O_TOT, 0, sizeof(double) * NTOT, st) != cudaSuccess)
         return NE_ECUDA;
 
