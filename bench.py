@@ -269,7 +269,8 @@ def run_ours(args):
         m.replica = rid
     n_rep, n_atoms = len(mds), int(offs[-1])
     ctx = ne.ne_ctx_create(ne.eam_params(**W.EAM_FE_LIKE), n_atoms, n_rep)
-    ne.ne_ctx_set_tuning(ctx, args.tpa)
+    if args.tpa:
+        ne.ne_ctx_set_tuning(ctx, args.tpa)
     x0 = torch.tensor(x0_np, dtype=torch.float64, device=dev)
     x = x0.clone()
     v = torch.zeros_like(x)
@@ -629,7 +630,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=200)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--prec", default="mixed", choices=["mixed", "fp64"])
-    ap.add_argument("--tpa", type=int, default=4)
+    ap.add_argument("--tpa", type=int, default=0, help="threads per atom of the multi-kernel path (0: by the batch's size)")
     ap.add_argument("--path", default="auto", choices=["auto", "crystal", "general"],
                     help="crystal: persistent cluster runner (mixed); general: multi-kernel path")
     ap.add_argument("--cpu-steps", type=int, default=80)

@@ -150,7 +150,8 @@ ne_status ne_ctx_set_theta(ne_ctx* ctx, const double* theta_dev, void* stream);
 /* Copy the current knot parameters to theta_dev (same layout). */
 ne_status ne_ctx_get_theta(ne_ctx* ctx, double* theta_dev, void* stream);
 
-/* Tuning of the pair kernels: threads per atom (1, 2, 4 or 8). */
+/* Tuning of the pair kernels: threads per atom (1, 2, 4 or 8).  Without this
+ * call they are chosen by the batch's size (8 to 32). */
 ne_status ne_ctx_set_tuning(ne_ctx* ctx, int threads_per_atom);
 
 /* CTAs per thread-block cluster of ne_crystal_run_segment (a scheduling

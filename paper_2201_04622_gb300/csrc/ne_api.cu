@@ -57,7 +57,9 @@ struct CrPlan {
 
 struct ne_ctx {
     ne_eam_params eam{};
-    int max_atoms = 0, max_rep = 0, tiles_cap = 0, cells_cap = 0, tpa = 4;
+    int max_atoms = 0, max_rep = 0, tiles_cap = 0, cells_cap = 0;
+    int sms = 0;        // SMs of the context's device
+    int tpa = 0;        // threads per atom of the pair passes (0: by the batch's size)
     int cluster_c = 0;  // crystal runner: CTAs per cluster (0: chosen per batch)
     int last_nrep = 0;  // replicas of the last multi-kernel run (ne_ctx_boxes)
     int last_nrep_cr = 0;  // replicas of the last crystal-runner call (ne_ctx_replica_status)
@@ -67,7 +69,8 @@ struct ne_ctx {
     float4* F32 = nullptr;
     ned4* F64 = nullptr;
     float4 *pos32 = nullptr, *posF = nullptr, *pbuild = nullptr, *f32 = nullptr;
-    double *f64 = nullptr, *dF64 = nullptr, *rho = nullptr, *xi64 = nullptr;
+    double *f64 = nullptr, *gs = nullptr, *rho = nullptr, *xi64 = nullptr;
+    ned4* pos64 = nullptr;
     float* xi32 = nullptr;
     int *nbr = nullptr, *ncnt = nullptr, *sl = nullptr, *scnt = nullptr;
     int *cellof = nullptr, *cslot = nullptr, *craw = nullptr, *cstart = nullptr, *ccount = nullptr;
@@ -196,6 +199,8 @@ void fill_tables(ne_ctx* ctx)
     t.rc2f = (float)(p.r_c * p.r_c);
     t.rmin2f = (float)(NE_RMIN * NE_RMIN);
     t.inv_h_rhof = (float)t.inv_h_rho;
+    t.rho_maxf = (float)p.rho_max;
+    t.ihr_lo = (float)(t.inv_h_rho - (double)t.inv_h_rhof);
 }
 
 // ------------------------------------------------------------ batches
@@ -268,6 +273,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
             if (geometry && !(R.L[d] > 2.0 * rl))
                 return fail(ctx, NE_EINVAL, "box edge must exceed 2 (r_c + skin)");
             R.invL[d] = 1.0 / R.L[d];
+            R.Lf[d] = (float)R.L[d];
+            R.iLf[d] = (float)R.invL[d];
             R.nc[d] = geometry ? (int)std::min(std::floor(shrink * R.L[d] / rl), 1024.0) : 0;
         }
         // cells of edge >= r_c + skin; fewer (larger) cells when the box is
@@ -328,7 +335,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.n_tot = n_tot;
     B.n_tiles = n_tiles;
     for (const RepDev& R : ctx->rep_h) B.n_max = std::max(B.n_max, R.n);
-    B.tpa = ctx->tpa;
+    B.sms = ctx->sms;
+    B.g = ctx->tpa > 0 ? ctx->tpa : ne::lanes_per_atom(n_tot);
     B.rep = ctx->rep;
     B.tile_rep = ctx->tile_rep;
     B.x = a.x;
@@ -339,7 +347,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.pbuild = ctx->pbuild;
     B.f32 = ctx->f32;
     B.f64 = ctx->f64;
-    B.dF64 = ctx->dF64;
+    if (md[0].prec != NE_MIXED) B.pos64 = ctx->pos64;
+    B.gs = ctx->gs;
     B.rho = a.rho;
     B.xi32 = ctx->xi32;
     B.xi64 = ctx->xi64;
@@ -392,13 +401,12 @@ ne_status finish(ne_ctx* ctx, cudaStream_t st)
 }
 
 // Forces at the current x of every replica: list (re)build when flagged,
-// pass 1, pass 2 (with the noise of step s when want_noise).
-void force_eval(const DevBatch& B, const Sched& S, bool mixed, const long long* ctr, int j,
-                int want_noise, int force_build, cudaStream_t st)
+// pass 1, pass 2.
+void force_eval(const DevBatch& B, bool mixed, cudaStream_t st)
 {
-    ne::launch_nl_build(B, force_build, 0, st);
-    ne::launch_density(B, mixed, ctr, j, st);
-    ne::launch_force(B, S, mixed, ctr, j, want_noise, st);
+    ne::launch_nl_build(B, 0, 0, st);
+    ne::launch_pass1(B, mixed, st);
+    ne::launch_pass2(B, mixed, st);
 }
 
 // One fused step of the schedule (device step = *ctr + j).
@@ -414,14 +422,14 @@ struct GradAcc {
 
 void grad_at(const DevBatch& B, bool mixed, const GradAcc* ga, const long long* ctr, int j, cudaStream_t st)
 {
-    if (ga) ne::launch_backward(B, mixed, 0.0, nullptr, ga->gtheta, ga->bins, ga->nbb, true, st, ga->w, ctr, j,
+    if (ga) ne::launch_backward(B, mixed, 0.0, ga->gtheta, ga->bins, ga->nbb, true, st, ga->w, ctr, j,
                                 ga->s_off, false);
 }
 
 void one_step(const DevBatch& B, const Sched& S, bool mixed, const long long* ctr, int j, int first,
               cudaStream_t st, const GradAcc* ga = nullptr)
 {
-    force_eval(B, S, mixed, ctr, j, 1, 0, st);
+    force_eval(B, mixed, st);
     grad_at(B, mixed, ga, ctr, j, st);
     ne::launch_step(B, S, mixed, ctr, j, first ? 0 : 1, 1, st);
     if (B.npt_any) ne::launch_npt_box(B, S, ctr, j, st);
@@ -496,7 +504,7 @@ ne_status run_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, 
             ne::launch_msd_sample(B, msd_acc, st);
     }
     // closing half kick of the last step
-    force_eval(B, S, mixed, ctr, 0, 0, 0, st);
+    force_eval(B, mixed, st);
     grad_at(B, mixed, ga, ctr, 0, st);
     ne::launch_step(B, S, mixed, ctr, 0, 1, 0, st);
     NE_CU(cudaGetLastError());
@@ -522,17 +530,17 @@ ne_status profile_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mix
         ne::launch_nl_build(B, 0, 0, st);
         NE_CU(cudaEventRecord(e[1], st));
         NE_CU(cudaEventRecord(e[2], st));
-        ne::launch_density(B, mixed, ctr, 0, st);
+        ne::launch_pass1(B, mixed, st);
         NE_CU(cudaEventRecord(e[3], st));
         NE_CU(cudaEventRecord(e[4], st));
-        ne::launch_force(B, S, mixed, ctr, 0, 1, st);
+        ne::launch_pass2(B, mixed, st);
         NE_CU(cudaEventRecord(e[5], st));
         NE_CU(cudaEventRecord(e[6], st));
         ne::launch_step(B, S, mixed, ctr, 0, s == 0 ? 0 : 1, 1, st);
         NE_CU(cudaEventRecord(e[7], st));
         ne::launch_advance(ctr, 1, st);
     }
-    force_eval(B, S, mixed, ctr, 0, 0, 0, st);
+    force_eval(B, mixed, st);
     ne::launch_step(B, S, mixed, ctr, 0, 1, 0, st);
     NE_CU(cudaStreamSynchronize(st));
     for (int k = 0; k < 4; ++k) {
@@ -603,6 +611,9 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     const size_t N = (size_t)max_atoms, R = (size_t)max_replicas, nk = (size_t)eam->n_knots;
     bool ok = true;
     auto A = [&](cudaError_t e) { ok = ok && e == cudaSuccess; };
+    int dev = 0;
+    A(cudaGetDevice(&dev));
+    A(cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev));
     A(dalloc(&ctx->theta, 6 * nk));
     A(dalloc(&ctx->pf32, 2 * nk));
     A(dalloc(&ctx->pf64, 2 * nk));
@@ -613,14 +624,15 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->pbuild, N));
     A(dalloc(&ctx->f32, N));
     A(dalloc(&ctx->f64, 3 * N));
-    A(dalloc(&ctx->dF64, N));
+    A(dalloc(&ctx->pos64, N));
+    A(dalloc(&ctx->gs, N * NE_SMAX));
     A(dalloc(&ctx->rho, N));
     A(dalloc(&ctx->xi64, 3 * N));
     A(dalloc(&ctx->xi32, 3 * N));
     A(dalloc(&ctx->nbr, N * NE_NMAX));
     A(dalloc(&ctx->ncnt, N));
-    A(dalloc(&ctx->sl, N * NE_SMAX));
-    A(dalloc(&ctx->scnt, N * 8));
+    A(dalloc(&ctx->sl, 2 * N * NE_SMAX));
+    A(dalloc(&ctx->scnt, N));
     A(dalloc(&ctx->cellof, N));
     A(dalloc(&ctx->cslot, N));
     A(dalloc(&ctx->craw, N));
@@ -628,7 +640,7 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->cstart, (size_t)ctx->cells_cap + R));
     A(dalloc(&ctx->ccount, (size_t)ctx->cells_cap));
     A(dalloc(&ctx->nl_done, R));
-    A(dalloc(&ctx->partA, (size_t)ctx->tiles_cap * NPA));
+    A(dalloc(&ctx->partA, (size_t)ctx->tiles_cap * NE_PAIR_SUB * NPA));
     A(dalloc(&ctx->partB, (size_t)ctx->tiles_cap * NPB));
     A(dalloc(&ctx->tot, R * NTOT));
     A(dalloc(&ctx->W, 2 * R));
@@ -679,7 +691,7 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
 {
     if (!ctx) return NE_EINVAL;
     void* ptrs[] = {ctx->theta, ctx->pf32, ctx->pf64, ctx->F32, ctx->F64, ctx->pos32, ctx->posF,
-                    ctx->pbuild, ctx->f32, ctx->f64, ctx->dF64, ctx->rho, ctx->xi64, ctx->xi32,
+                    ctx->pbuild, ctx->f32, ctx->f64, ctx->pos64, ctx->gs, ctx->rho, ctx->xi64, ctx->xi32,
                     ctx->nbr, ctx->ncnt, ctx->sl, ctx->scnt, ctx->cellof, ctx->cslot, ctx->craw, ctx->csort,
                     ctx->cstart, ctx->ccount, ctx->nl_done, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
                     ctx->tile_done, ctx->flags, ctx->building, ctx->status, ctx->tile_rep, ctx->rep, ctx->step_ctr, ctx->rebuilds, ctx->xrep, ctx->work, ctx->st_vec, ctx->st_dist, ctx->lam_tab,
@@ -939,12 +951,9 @@ ne_status ne_eam_energy_forces(ne_ctx* ctx, ne_precision prec, const double* x_d
     ne_status s = setup_batch(ctx, 1, off, box, &m, 0, 0.0, B, a, st);
     if (s) return s;
     const bool mixed = prec == NE_MIXED;
-    Sched S{};
-    S.kind = SCHED_FIXED;
     ne::launch_nl_build(B, 1, 0, st);
-    if (mixed) ne::launch_wrap32(B, st);
-    ne::launch_density(B, mixed, ctx->step_ctr, 0, st);
-    ne::launch_force(B, S, mixed, ctx->step_ctr, 0, 0, st);
+    ne::launch_pass1(B, mixed, st);
+    ne::launch_pass2(B, mixed, st);
     ne::launch_export(B, mixed, f_dev, e_dev, st);
     return finish(ctx, st);
 }
@@ -965,8 +974,10 @@ ne_status ne_eam_virial(ne_ctx* ctx, const double* x_dev, int n, const double bo
     DevBatch B;
     ne_status s = setup_batch(ctx, 1, off, box, &m, 0, 0.0, B, a, st);
     if (s) return s;
+    B.npt_any = 1;  // sum the virial
     ne::launch_nl_build(B, 1, 0, st);
-    ne::launch_density(B, false, ctx->step_ctr, 0, st);
+    ne::launch_pass1(B, false, st);
+    ne::launch_pass2(B, false, st);
     ne::launch_virial(B, w_dev, st);
     return finish(ctx, st);
 }
@@ -988,6 +999,7 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
     m.dt = 1e-3;
     m.T = 1.0;
     m.mass = 1.0;
+    m.prec = prec;
     int off[2] = {0, n};
     RunArgs a{};
     a.x = const_cast<double*>(x_dev);
@@ -996,12 +1008,9 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
     ne_status s = setup_batch(ctx, 1, off, box, &m, 0, 0.0, B, a, st);
     if (s) return s;
     const bool mixed = prec == NE_MIXED;
-    Sched S{};
-    S.kind = SCHED_FIXED;
     ne::launch_nl_build(B, 1, 0, st);
-    if (mixed) ne::launch_wrap32(B, st);
-    ne::launch_density(B, mixed, ctx->step_ctr, 0, st);
-    ne::launch_force(B, S, mixed, ctx->step_ctr, 0, 0, st);
+    ne::launch_pass1(B, mixed, st);
+    ne::launch_pass2(B, mixed, st);
     if (gx_dev) ne::launch_export(B, mixed, gx_dev, nullptr, st);
     if (mixed && !ne::backward_fits(ctx->eam.n_knots))
         return fail(ctx, NE_EINVAL, "mixed backward: n_knots too large for one block's shared-memory bins");
@@ -1013,7 +1022,7 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
         NE_CU(cudaMalloc((void**)&ctx->bins, ne::backward_bins_bytes(ctx->eam.n_knots, nbb)));
         ctx->bins_blocks = nbb;
     }
-    ne::launch_backward(B, mixed, gE, gx_dev, gtheta_dev, ctx->bins, nbb, accumulate, st);
+    ne::launch_backward(B, mixed, gE, gtheta_dev, ctx->bins, nbb, accumulate, st);
     if (gx_dev) ne::launch_scale(gx_dev, 3 * n, -gE, st);  // dU/dx = -F times gE
     return finish(ctx, st);
 }

@@ -3,21 +3,26 @@
 //
 // Data layout in HBM (all replicas of a batch concatenated, atom-major):
 //   x, v, x0            double [N][3]   caller-owned, unwrapped positions
-//   pos32               float4 [N]      FP32 copy of x wrapped into the box
-//   posF                float4 [N]      (x, y, z, F'(rho)) written by pass 1
 //   pbuild              float4 [N]      wrapped positions at the last list build
+//   pos32               float4 [N]      FP32 copy of x wrapped into the box; .w (int bits) the code
+//                                       9 a + 3 b + c of the box lengths it lies from the image
+//                                       nearest pbuild, which the list's images refer to
+//   posF                float4 [N]      (x, y, z, F'(rho)) written by pass 1 (mixed)
+//   pos64               ned4 [N]        wrapped positions (x, y, z) and F'(rho) (FP64 path)
+//   csort               float4 [N]      the same sorted by cell, .w the atom's index in its replica
 //   f32 / f64           EAM forces, float4 [N] (mixed) or double [N][3]
-//   dF64                double [N]      F'(rho) (FP64 path)
-//   xi32 / xi64         Langevin normals of the current step, [N][3]
-//   csort               float4 [N]      pbuild sorted by cell, .w the atom's index in its replica
-//   nbr, ncnt           candidate list within r_c + skin, int, lane-interleaved:
-//                       entry k of atom i at ((k / TPA) * N + i) * TPA + k % TPA
-//   sl, scnt            per-step short list (r < r_c) in the same layout, one
-//                       count per (atom, lane)
-//   partA / partB       per-tile FP64 partial sums (pass 1+2 / step kernel)
-//   tot                 per-replica totals formed by the last tile of pass 2
+//   xi32 / xi64         Langevin normals of the coming step, [N][3]
+//   nbr, ncnt           candidate list within r_c + skin: int [N][NE_NMAX] (neighbour and its
+//                       image), count [N]
+//   sl, gs, scnt        the step's pairs inside r_c: neighbour and its image, and f'(r)/r of
+//                       each -- (int, float bits) pairs [N][NE_SMAX] in sl (mixed), int
+//                       [N][NE_SMAX] in sl and double [N][NE_SMAX] in gs (FP64); count [N]
+//   partA / partB       partial sums of the pair blocks (pass 1 and 2) and of the
+//                       step kernel's tiles, quantity-major
+//   tot                 per-replica totals formed by the last block of pass 2
 // A tile is NE_TILE consecutive atoms of one replica; tiles never straddle
-// replicas, so every per-replica sum is a fixed-order sum of tile partials.
+// replicas, and a pair block takes a whole fraction of a tile, so every
+// per-replica sum is a fixed-order sum of partials.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -28,6 +33,11 @@ struct __align__(32) ned4 {
 };
 
 #define NE_TILE 64
+#define NE_PAIR_SUB 8   // most pair blocks per tile (32 lanes per atom)
+// list entry: neighbour in the low 27 bits, above them the code 9 (a + 1) + 3 (b + 1) + c + 1 of the
+// shift (a, b, c), each in {-1, 0, 1}, in box lengths, that is added to r_j - r_i
+#define NE_IMG_SHIFT 27
+#define NE_IMG_NONE 13
 #define NE_MAX_SPECIES_DEV 8  // species per replica (NE_MAX_SPECIES of the public header)
 #define NE_NMAX 256   // candidate neighbours per atom (r < r_c + skin)
 #define NE_SMAX 128   // neighbours per atom inside r_c
@@ -39,17 +49,17 @@ enum { ST_ERANGE = 1, ST_ENEIGH = 2, ST_ENAN = 4, ST_ETIMEOUT = 8, ST_EINVAL = 1
 // Philox stream ids (low 4 bits of the 4th counter word)
 enum { STREAM_FL = 0, STREAM_INITV = 1, STREAM_RS = 2, STREAM_MSD = 3, STREAM_STEP = 4, STREAM_BARO = 5 };
 
-// tile partials of pass 1 / pass 2 (at x_k)
-enum { PA_UEMB = 0, PA_UPAIR, PA_F0X, PA_F0Y, PA_F0Z, PA_XIX, PA_XIY, PA_XIZ, PA_VIR, PA_VXX, PA_VYY, PA_VZZ, NPA };
-// tile partials of the step kernel (at x_{k+1}; KE of the completed velocity)
-enum { PB_UE = 0, PB_UX, PB_UY, PB_UZ, PB_U2, PB_KE, NPB };
+// partials of pass 1 (energies, the pair part of the virial) and pass 2 (forces, its embedding part), at x_k
+enum { PA_UEMB = 0, PA_UPAIR, PA_F0X, PA_F0Y, PA_F0Z, PA_VXX, PA_VYY, PA_VZZ, PA_WXX, PA_WYY, PA_WZZ, NPA };
+// tile partials of the step kernel (at x_{k+1}; KE of the completed velocity; the normals of step k+1)
+enum { PB_UE = 0, PB_UX, PB_UY, PB_UZ, PB_U2, PB_KE, PB_XIX, PB_XIY, PB_XIZ, NPB };
 // per-replica totals
-enum { TOT_UEMB = 0, TOT_UPAIR, TOT_F0X, TOT_F0Y, TOT_F0Z, TOT_XIX, TOT_XIY, TOT_XIZ, TOT_VIR,
-       TOT_VXX, TOT_VYY, TOT_VZZ, TOT_UE, TOT_UX, TOT_UY, TOT_UZ, TOT_U2, TOT_KE, NTOT };
-static_assert((int)TOT_VIR == (int)PA_VIR && (int)TOT_UE == (int)NPA, "totals: pass-2 partials first, then the step's");
+enum { TOT_UEMB = 0, TOT_UPAIR, TOT_F0X, TOT_F0Y, TOT_F0Z, TOT_VXX, TOT_VYY, TOT_VZZ, TOT_UE, TOT_UX, TOT_UY, TOT_UZ,
+       TOT_XIX, TOT_XIY, TOT_XIZ, NTOT };
 
 struct RepDev {
     double L[3], invL[3];
+    float Lf[3], iLf[3];  // the same in FP32 (a conversion costs an FP64 slot)
     double k;        // Einstein spring
     double c1, c2;   // Ornstein-Uhlenbeck coefficients
     double hdt_m;    // dt / (2 m)
@@ -69,8 +79,8 @@ struct RepDev {
     // nsp >= 2 -- atom a has species sp[a] (validated on the host) with mass
     // ms, spring ks, noise amplitude c2s and half-step factor hdts of its
     // species; M is the replica's total mass.  With species tables the
-    // step kernel's sum PB_UX.. holds sum_j k_j u_j and pass 2's PA_XIX..
-    // holds sum_j m_j c2_j xi_j: the sums the mass-weighted centre-of-mass
+    // step kernel's sum PB_UX.. holds sum_j k_j u_j and its PB_XIX.. holds
+    // sum_j m_j c2_j xi_j: the sums the mass-weighted centre-of-mass
     // constraint needs.
     int nsp;
     const unsigned char* sp;
@@ -99,11 +109,14 @@ struct Tables {
     double h_r, inv_h_r, h_rho, inv_h_rho;
     double r_c, rho_max;
     float inv_h_rf, rcf, rc2f, rmin2f, inv_h_rhof;
+    float rho_maxf, ihr_lo;  // inv_h_rho = inv_h_rhof + ihr_lo to double-float precision
 };
 
 struct DevBatch {
-    int n_rep, n_tot, n_tiles, tpa;
+    int n_rep, n_tot, n_tiles;
     int n_max;         // atoms of the largest replica
+    int g;             // lanes per atom in the pair passes
+    int sms;           // SMs of the device
     const RepDev* rep;
     const int* tile_rep;
     double* x;
@@ -111,25 +124,26 @@ struct DevBatch {
     const double* x0;
     float4* pos32;
     float4* posF;
+    ned4* pos64;
     float4* pbuild;
+    float4* csort;
     float4* f32;
     double* f64;
-    double* dF64;
     double* rho;       // nullable: per-atom density output
     float* xi32;
     double* xi64;
     int* nbr;
     int* ncnt;
     int* sl;
+    double* gs;        // FP64 path: [N][NE_SMAX]
     int* scnt;
     int* cellof;
     int* cslot;        // arrival order of each atom in its cell (list build)
     int* craw;         // atoms by cell, unsorted inside a cell (list build)
-    float4* csort;
     int* cstart;
     int* ccount;       // atoms per cell; zero between list builds
-    double* partA;
-    double* partB;
+    double* partA;     // [NPA][pair blocks]
+    double* partB;     // [NPB][n_tiles]
     double* tot;
     unsigned* tile_done;
     unsigned* nl_done;
@@ -142,7 +156,7 @@ struct DevBatch {
     unsigned long long* rebuilds;  // count of replica list builds
     int* status;
     Tables tab;
-    int npt_any;       // some replica has the barostat on
+    int npt_any;       // some replica has the barostat on (or the call wants the virial)
     int species_any;   // every replica has species tables (msd sampling per species)
 };
 
@@ -243,11 +257,6 @@ __device__ __forceinline__ void ne_normals32(uint4 w, float z[3])
 }
 
 // ------------------------------------------------------------------ misc
-__device__ __forceinline__ int ne_nbr_index(int k, int i, int n_tot, int tpa)
-{
-    return ((k / tpa) * n_tot + i) * tpa + (k % tpa);
-}
-
 // double-float (hi + lo, |lo| <= ulp(hi) / 2) sum of two such numbers from
 // FP32 operations (TwoSum of the high parts, the low parts added to its error)
 struct dff {
@@ -272,18 +281,22 @@ __device__ __forceinline__ dff dff_warp_sum(dff v)
     return v;
 }
 
-// Sum of quantity q over tiles [t0, t0 + nt) of a tile-partials array (nq
-// values a tile), by one warp: lane l adds tiles t0 + l, t0 + l + 32, ...
-// in order, then a fixed xor-shuffle tree; every lane returns the total, and
-// the order depends only on nt, never on scheduling.  Called by all 32 lanes.
-__device__ __forceinline__ double ne_warp_tile_sum(const double* part, int nq, int q, int t0, int nt)
+// Sum of nt consecutive partials, by one warp: lane l adds entries l, l + 32,
+// ... in four interleaved chains (a serial FP64 chain's latency was the cost
+// on a 65,536-atom replica), then a fixed xor-shuffle tree; every lane returns
+// the total, and the order depends only on nt, never on scheduling.  Called by
+// all 32 lanes.
+__device__ __forceinline__ double ne_warp_part_sum(const double* part, int nt)
 {
-    const int l = threadIdx.x & 31;
-    double acc = 0.0;
-    for (int t = l; t < nt; t += 32) acc += __ldcg(&part[(size_t)(t0 + t) * nq + q]);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int t = threadIdx.x & 31; t < nt; t += 128)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return acc;
+        for (int c = 0; c < 4; ++c)
+            if (t + 32 * c < nt) acc[c] += __ldcg(&part[t + 32 * c]);
+    double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
 }
 
 __device__ __forceinline__ void ne_set_status(int* status, int bits)
@@ -295,17 +308,18 @@ __device__ __forceinline__ void ne_set_status(int* status, int bits)
 namespace ne {
 void launch_tables(const double* theta, int nk, double r_c, double rho_max, float4* pf32,
                    ned4* pf64, float4* F32, ned4* F64, cudaStream_t st);
+// list build of the flagged (or, forced, all) replicas around the sites (the
+// step kernel then writes the positions for the pair passes) or the positions
+// (written here)
 void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t st);
-void launch_density(const DevBatch& B, bool mixed, const long long* step_base, int j,
-                    cudaStream_t st);
-void launch_force(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
-                  int j, int want_noise, cudaStream_t st);
+int lanes_per_atom(int n_tot);  // the pair passes' lanes per atom for a batch of n_tot atoms
+void launch_pass1(const DevBatch& B, bool mixed, cudaStream_t st);
+void launch_pass2(const DevBatch& B, bool mixed, cudaStream_t st);
 void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
                  int j, int do_close, int do_open, cudaStream_t st);
 void launch_prep(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
                  cudaStream_t st);
 void launch_advance(long long* step_base, long long by, cudaStream_t st);
-void launch_wrap32(const DevBatch& B, cudaStream_t st);
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,
                   double* z, cudaStream_t st);
 void launch_scale(double* p, int n, double s, cudaStream_t st);
@@ -320,7 +334,7 @@ void launch_msd_sample(const DevBatch& B, double* acc, cudaStream_t st);
 size_t backward_block_bytes(int nk);  // one mixed backward block's bins (device and shared memory)
 size_t backward_bins_bytes(int nk, int n_blocks);  // the whole bins buffer: F's (zeroed once), then the blocks'
 bool backward_fits(int nk);           // those bins fit one block's shared memory
-void launch_backward(const DevBatch& B, bool mixed, double gE, double* gx, double* gtheta,
+void launch_backward(const DevBatch& B, bool mixed, double gE, double* gtheta,
                      float* bins, int n_bin_blocks, bool accumulate, cudaStream_t st,
                      const double* gw = nullptr, const long long* ctr = nullptr, int j = 0,
                      long long s_off = 0, bool set_attr = true);

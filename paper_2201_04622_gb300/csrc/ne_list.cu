@@ -134,6 +134,10 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
         for (int d = 0; d < 3; ++d) w[d] = wrap(X[3 * i + d], P.L[d], P.invL[d]);
         const float4 p = make_float4((float)w[0], (float)w[1], (float)w[2], __int_as_float(a));
         B.pbuild[i] = p;
+        if (!from_sites) {  // what the pair passes read
+            B.pos32[i] = make_float4(p.x, p.y, p.z, __int_as_float(0));
+            if (B.pos64) B.pos64[i] = ned4{w[0], w[1], w[2], 0.0};
+        }
         if (P.nc[0] == 0) {
             B.csort[i] = p;  // all pairs: the atoms in index order
         } else {
@@ -186,22 +190,23 @@ __global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
 constexpr int LIST_THREADS = 256;
 
 template <int G>
-__global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
+__device__ void list_block(const DevBatch& B, int blk)
 {
     constexpr int AT = LIST_THREADS / G, SUB = NE_TILE / AT;
-    const int tile = blockIdx.x / SUB;
+    const int tile = blk / SUB;
     const int rep = B.tile_rep[tile];
     if (!B.building[rep]) return;
     const RepDev& P = B.rep[rep];
     const int lane = threadIdx.x % G;
-    const int a = (tile - P.tile0) * NE_TILE + (blockIdx.x % SUB) * AT + threadIdx.x / G;
+    const int a = (tile - P.tile0) * NE_TILE + (blk % SUB) * AT + threadIdx.x / G;
     const bool valid = a < P.n;
     const int off = P.off, i = off + (valid ? a : 0);
-    const float L0 = (float)P.L[0], L1 = (float)P.L[1], L2 = (float)P.L[2];
-    const float iL0 = (float)P.invL[0], iL1 = (float)P.invL[1], iL2 = (float)P.invL[2];
+    const float L0 = P.Lf[0], L1 = P.Lf[1], L2 = P.Lf[2];
+    const float iL0 = P.iLf[0], iL1 = P.iLf[1], iL2 = P.iLf[2];
     const float rl = sqrtf((float)P.rlist2) + 1e-3f;
     const float rl2 = rl * rl;
     const float4 pi = B.pbuild[i];
+    int* const row = B.nbr + (size_t)i * NE_NMAX;
     const int gsh = (threadIdx.x & 31) / G * G;  // this atom's first lane in the warp
     const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     int cnt = 0;
@@ -211,19 +216,21 @@ __global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
         for (int t = 0; t < trips; ++t) {
             const int p = lo + t * G + lane;
             bool hit = false;
-            int b = 0;
+            int b = 0, code = 0;
             if (p < hi) {
                 const float4 pj = B.csort[off + p];
                 b = __float_as_int(pj.w);
                 float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-                dx -= L0 * rintf(dx * iL0);
-                dy -= L1 * rintf(dy * iL1);
-                dz -= L2 * rintf(dz * iL2);
+                const float n0 = rintf(dx * iL0), n1 = rintf(dy * iL1), n2 = rintf(dz * iL2);
+                dx -= L0 * n0;
+                dy -= L1 * n1;
+                dz -= L2 * n2;
+                code = NE_IMG_NONE - (int)(9.f * n0 + 3.f * n1 + n2);
                 hit = b != a && dx * dx + dy * dy + dz * dz < rl2;
             }
             const unsigned m = (__ballot_sync(0xffffffffu, hit) >> gsh) & gmask;
             const int at = cnt + __popc(m & ((1u << lane) - 1u));
-            if (hit && at < NE_NMAX) B.nbr[ne_nbr_index(at, i, B.n_tot, B.tpa)] = off + b;
+            if (hit && at < NE_NMAX) row[at] = (off + b) | (int)((unsigned)code << NE_IMG_SHIFT);
             cnt += __popc(m);
         }
     };
@@ -254,6 +261,14 @@ __global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
     }
 }
 
+// a few blocks an SM take the atoms in turn: a launch with nothing to build is
+// over sooner than with a block for every 8 or 32 atoms
+template <int G>
+__global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
+{
+    for (int blk = blockIdx.x; blk < B.n_tiles * (NE_TILE * G / LIST_THREADS); blk += gridDim.x) list_block<G>(B, blk);
+}
+
 }  // namespace
 
 namespace ne {
@@ -261,14 +276,15 @@ namespace ne {
 void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t st)
 {
     k_nl_cells<<<(B.n_tiles + CELL_TILES - 1) / CELL_TILES, CELL_THREADS, 0, st>>>(B, force, from_sites);
+    const auto grid = [&](int want) { return want < 6 * B.sms ? want : 6 * B.sms; };
     if (B.n_max > SORT_IN_BLOCK)
         k_nl_sort<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
     // a warp an atom up to 8192 atoms (a quarter of a million threads, one
     // wave), eight lanes above: fewer idle lanes at the ends of the short runs
     if (B.n_tot <= 8192)
-        k_nl_list<32><<<B.n_tiles * (NE_TILE * 32 / LIST_THREADS), LIST_THREADS, 0, st>>>(B);
+        k_nl_list<32><<<grid(B.n_tiles * (NE_TILE * 32 / LIST_THREADS)), LIST_THREADS, 0, st>>>(B);
     else
-        k_nl_list<8><<<B.n_tiles * (NE_TILE * 8 / LIST_THREADS), LIST_THREADS, 0, st>>>(B);
+        k_nl_list<8><<<grid(B.n_tiles * (NE_TILE * 8 / LIST_THREADS)), LIST_THREADS, 0, st>>>(B);
 }
 
 }  // namespace ne

@@ -6,8 +6,6 @@
 
 namespace {
 
-__device__ __forceinline__ double wrap(double x, double L, double invL) { return x - L * floor(x * invL); }
-
 // ------------------------------------------------------------ fused step
 // Total force of H(lambda) on atom i from the EAM force F0, the spring force
 // F_E = -k u and, with the centre of mass fixed, their replica means:
@@ -25,8 +23,11 @@ __device__ __forceinline__ double blend(int path, double lam, double F0, double 
 //             v += dt/2m F(x_s; Lambda(s+1));  x += dt/2 v;
 //             v = c1 v + c2 (xi - mean xi);    x += dt/2 v
 // then the tile partials at the resulting x (U_E, sum u, sum |u|^2) and the
-// kinetic energy of the completed velocity v_s, the FP32 wrapped copy of x
-// and the displacement check against the list-build positions.
+// kinetic energy of the completed velocity v_s, the copies of x for
+// the pair passes, the
+// displacement check against the list-build positions, and the normals of the
+// next step with their sums (counter-based, so drawn one step ahead, one
+// thread an atom; the prep launch draws the first step's).
 //
 // With the barostat (RepDev.npt), after the second drift ln V takes one
 // Euler-Maruyama step of the overdamped Langevin equation whose stationary
@@ -59,7 +60,8 @@ __device__ inline void npt_scale(const RepDev& P, const double* T, double lam, l
         }
         return;
     }
-    const double drive = (P.dof * P.kT + lam * T[TOT_VIR]) / (3.0 * V) - P.P0;
+    const double W = T[TOT_VXX] + T[TOT_VYY] + T[TOT_VZZ];
+    const double drive = (P.dof * P.kT + lam * W) / (3.0 * V) - P.P0;
     const double deps = P.mp * drive * dt + noise * z[0];
     mu[0] = mu[1] = mu[2] = exp(deps / 3.0);
 }
@@ -106,7 +108,6 @@ __device__ void step_work(const DevBatch& B, const Sched& S, const double* T, in
     }
 }
 
-template <bool MIXED>
 __global__ void __launch_bounds__(NE_TILE)
     k_step(DevBatch B, Sched S, const long long* __restrict__ step_base, int j, int do_close, int do_open)
 {
@@ -122,7 +123,8 @@ __global__ void __launch_bounds__(NE_TILE)
     const double lam_s = ne_sched_lambda(S, s);
     const double lam_n = ne_sched_lambda(S, s + 1);
     const double invN = 1.0 / P.n;
-    double part[NPB] = {0, 0, 0, 0, 0, 0};
+    const bool draw = do_open || !do_close;  // a step follows: its normals
+    double part[NPB] = {};
     int bad = 0;
     if (valid) {
         double x[3], v[3], u[3], F0[3], mF0[3], mFE[3];
@@ -132,16 +134,7 @@ __global__ void __launch_bounds__(NE_TILE)
             v[c] = B.v[3 * i + c];
             u[c] = x[c] - B.x0[3 * i + c];
         }
-        if constexpr (MIXED) {
-            float4 f = B.f32[i];
-            F0[0] = f.x;
-            F0[1] = f.y;
-            F0[2] = f.z;
-        } else {
-            F0[0] = B.f64[3 * i];
-            F0[1] = B.f64[3 * i + 1];
-            F0[2] = B.f64[3 * i + 2];
-        }
+        for (int c = 0; c < 3; ++c) F0[c] = B.f64[3 * i + c];
         // this atom's mass, spring, noise amplitude and half-step factor
         // (one species, or its species' entries)
         const int q = P.nsp ? (int)P.sp[a] : 0;
@@ -166,7 +159,7 @@ __global__ void __launch_bounds__(NE_TILE)
             // species; c2_i xi_i - sum_j m_j c2_j xi_j / M with species tables
             double dv[3];
             for (int c = 0; c < 3; ++c) {
-                const double xi = MIXED ? (double)B.xi32[3 * i + c] : B.xi64[3 * i + c];
+                const double xi = B.xi64[3 * i + c];
                 if (P.nsp) dv[c] = c2i * xi - (S.fix_cm ? T[TOT_XIX + c] / P.M : 0.0);
                 else dv[c] = P.c2 * (S.fix_cm ? xi - T[TOT_XIX + c] * invN : xi);
             }
@@ -194,17 +187,40 @@ __global__ void __launch_bounds__(NE_TILE)
         }
         part[PB_U2] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         part[PB_UE] = 0.5 * ki * part[PB_U2];
-        // FP32 wrapped copy and displacement since the list build
-        float w[3];
-        for (int c = 0; c < 3; ++c) w[c] = (float)wrap(x[c], Lb[c], 1.0 / Lb[c]);
-        if constexpr (MIXED) B.pos32[i] = make_float4(w[0], w[1], w[2], 0.f);
-        float4 pb = B.pbuild[i];
-        float d0 = w[0] - pb.x, d1 = w[1] - pb.y, d2 = w[2] - pb.z;
-        const float L0 = (float)Lb[0], L1 = (float)Lb[1], L2 = (float)Lb[2];
-        d0 -= L0 * rintf(d0 / L0);
-        d1 -= L1 * rintf(d1 / L1);
-        d2 -= L2 * rintf(d2 / L2);
-        if (d0 * d0 + d1 * d1 + d2 * d2 > P.half_skin2) B.flags[rep] = 1;
+        // x wrapped, its image against the list build's and the displacement
+        // from there (image indices in FP32: exact integers)
+        const float4 pb = B.pbuild[i];
+        const float pbx[3] = {pb.x, pb.y, pb.z};
+        double w64[3];
+        float w[3], d2 = 0.f;
+        int code = 0;
+        for (int c = 0; c < 3; ++c) {
+            const float Lf = (float)Lb[c], iLf = 1.f / Lf;
+            w64[c] = x[c];
+            w[c] = (float)x[c];
+            const float n = floorf(w[c] * iLf);
+            if (n != 0.f) {
+                w64[c] = x[c] - Lb[c] * (double)n;
+                w[c] = (float)w64[c];
+            }
+            const float nb = rintf((w[c] - pbx[c]) * iLf), d = fmaf(-Lf, nb, w[c] - pbx[c]);
+            code = 3 * code + (int)nb;
+            d2 = fmaf(d, d, d2);
+        }
+        B.pos32[i] = make_float4(w[0], w[1], w[2], __int_as_float(code));
+        B.pos64[i] = ned4{w64[0], w64[1], w64[2], 0.0};
+        if (d2 > P.half_skin2) B.flags[rep] = 1;
+        if (draw) {
+            double z[3];
+            ne_normals64(ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
+                                         (unsigned long long)(do_open ? s + 1 : s)),
+                         z);
+            const double wq = P.nsp ? mi * c2i : 1.0;  // the velocity increments' momentum: sum m_j c2_j xi_j
+            for (int c = 0; c < 3; ++c) {
+                B.xi64[3 * i + c] = z[c];
+                part[PB_XIX + c] = wq * z[c];
+            }
+        }
     }
     if (bad) ne_set_status(B.status, bad);
     if (do_open && valid && a == 0) step_work(B, S, T, rep, s, lam_s, lam_n);
@@ -216,8 +232,7 @@ __global__ void __launch_bounds__(NE_TILE)
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        double* pb = B.partB + (size_t)tile * NPB;
-        for (int q = 0; q < NPB; ++q) pb[q] = red[q][0];
+        for (int q = 0; q < NPB; ++q) B.partB[(size_t)q * B.n_tiles + tile] = red[q][0];
     }
 }
 
@@ -292,7 +307,8 @@ __global__ void __launch_bounds__(NE_TILE)
     __syncthreads();
     const double lam_s = s_lam[0], lam_n = s_lam[1];
     const float ls = (float)lam_s, ln = (float)lam_n;
-    float part[NPB] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const bool draw = do_open || !do_close;  // a step follows: its normals
+    float part[NPB] = {};
     int bad = 0;
     if (valid) {
         double x[3];
@@ -341,22 +357,33 @@ __global__ void __launch_bounds__(NE_TILE)
         }
         part[PB_U2] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         part[PB_UE] = 0.5f * ki * part[PB_U2];
-        // FP32 wrapped copy and displacement since the list build: the image
-        // index in FP32, the shift (only for an atom outside the box) in FP64
-        float w[3];
+        // x wrapped (image index in FP32, the shift, only for an atom outside
+        // the box, in FP64), its image against the list build's and the
+        // displacement from there
+        const float4 pb = B.pbuild[i];
+        const float pbx[3] = {pb.x, pb.y, pb.z};
+        float w[3], d2 = 0.f;
+        int code = 0;
         for (int c = 0; c < 3; ++c) {
             w[c] = (float)x[c];
             const float n = floorf(w[c] * s_box[3 + c]);
             if (n != 0.f) w[c] = (float)(x[c] - s_mu[c] * P.L[c] * (double)n);
+            const float nb = rintf((w[c] - pbx[c]) * s_box[3 + c]), d = fmaf(-s_box[c], nb, w[c] - pbx[c]);
+            code = 3 * code + (int)nb;
+            d2 = fmaf(d, d, d2);
         }
-        B.pos32[i] = make_float4(w[0], w[1], w[2], 0.f);
-        const float4 pb = B.pbuild[i];
-        float d[3] = {w[0] - pb.x, w[1] - pb.y, w[2] - pb.z}, d2 = 0.f;
-        for (int c = 0; c < 3; ++c) {
-            d[c] = fmaf(-s_box[c], rintf(d[c] * s_box[3 + c]), d[c]);
-            d2 = fmaf(d[c], d[c], d2);
-        }
+        B.pos32[i] = make_float4(w[0], w[1], w[2], __int_as_float(code));
         if (d2 > s_box[7]) B.flags[rep] = 1;
+        if (draw) {
+            float z[3];
+            ne_normals32(ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
+                                         (unsigned long long)(do_open ? s + 1 : s)),
+                         z);
+            for (int c = 0; c < 3; ++c) {
+                B.xi32[3 * i + c] = z[c];
+                part[PB_XIX + c] = P.nsp ? mi * c2i * z[c] : z[c];
+            }
+        }
     }
     if (bad) ne_set_status(B.status, bad);
     if (do_open && valid && a == 0) step_work(B, S, T, rep, s, lam_s, lam_n);
@@ -371,7 +398,7 @@ __global__ void __launch_bounds__(NE_TILE)
     if (threadIdx.x < NPB) {
         dff t = {0.f, 0.f};
         for (int w2 = 0; w2 < NE_TILE / 32; ++w2) t = dff_add(t, {s_w[threadIdx.x][w2].x, s_w[threadIdx.x][w2].y});
-        B.partB[(size_t)tile * NPB + threadIdx.x] = (double)t.hi + (double)t.lo;
+        B.partB[(size_t)threadIdx.x * B.n_tiles + tile] = (double)t.hi + (double)t.lo;
     }
 }
 
@@ -382,7 +409,7 @@ __global__ void k_trace_T(DevBatch B, const long long* __restrict__ step_base, i
     const long long s = *step_base + j;
     if (!B.trace || s % B.trace_stride != 0 || s / B.trace_stride >= B.trace_rows) return;
     const RepDev& P = B.rep[0];
-    const double ke = ne_warp_tile_sum(B.partB, NPB, PB_KE, P.tile0, P.ntile);
+    const double ke = ne_warp_part_sum(B.partB + (size_t)PB_KE * B.n_tiles + P.tile0, P.ntile);
     const double kB = 8.617333262e-5;
     if (threadIdx.x == 0) B.trace[8 * (s / B.trace_stride) + 5] = 2.0 * ke / (P.dof * kB);
 }
@@ -413,6 +440,8 @@ __global__ void k_npt_box(DevBatch B, Sched S, const long long* __restrict__ ste
     for (int c = 0; c < 3; ++c) {
         P.L[c] *= mu[c];
         P.invL[c] = 1.0 / P.L[c];
+        P.Lf[c] = (float)P.L[c];
+        P.iLf[c] = (float)P.invL[c];
     }
 }
 
@@ -431,20 +460,6 @@ __global__ void k_noise(unsigned long long seed, unsigned replica, int stream, l
             for (int c = 0; c < 3; ++c) z[3 * a + c] = d[c];
         }
     }
-}
-
-// FP32 copy of the positions wrapped into the box (pass-1/2 input of the
-// mixed path when no step kernel has produced it).
-__global__ void k_wrap32(DevBatch B)
-{
-    const int tile = blockIdx.x;
-    const RepDev& P = B.rep[B.tile_rep[tile]];
-    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x;
-    if (a >= P.n) return;
-    const int i = P.off + a;
-    B.pos32[i] = make_float4((float)wrap(B.x[3 * i], P.L[0], P.invL[0]),
-                             (float)wrap(B.x[3 * i + 1], P.L[1], P.invL[1]),
-                             (float)wrap(B.x[3 * i + 2], P.L[2], P.invL[2]), 0.f);
 }
 
 // ------------------------------------------------------------ velocities
@@ -492,7 +507,7 @@ __global__ void __launch_bounds__(NE_TILE) k_init_v_draw(DevBatch B)
     }
     for (int c = 0; c < 3; ++c) {
         const double t = tile_sum64(sum[c], red);
-        if (threadIdx.x == 0) B.partA[(size_t)tile * NPA + c] = t;
+        if (threadIdx.x == 0) B.partA[(size_t)c * B.n_tiles + tile] = t;
     }
 }
 
@@ -504,7 +519,7 @@ __global__ void __launch_bounds__(NE_TILE) k_init_v_center(DevBatch B, int fix_c
     const RepDev& P = B.rep[B.tile_rep[tile]];
     if (threadIdx.x < 32)
         for (int c = 0; c < 3; ++c) {
-            const double t = ne_warp_tile_sum(B.partA, NPA, c, P.tile0, P.ntile);
+            const double t = ne_warp_part_sum(B.partA + (size_t)c * B.n_tiles + P.tile0, P.ntile);
             if (threadIdx.x == 0) s_mean[c] = fix_cm ? (P.nsp ? t : t / P.n) : 0.0;
         }
     __syncthreads();
@@ -517,7 +532,7 @@ __global__ void __launch_bounds__(NE_TILE) k_init_v_center(DevBatch B, int fix_c
             ke += 0.5 * init_mass(P, a) * (*vv) * (*vv);
         }
     const double t = tile_sum64(ke, red);
-    if (threadIdx.x == 0) B.partA[(size_t)tile * NPA + 3] = t;
+    if (threadIdx.x == 0) B.partA[(size_t)3 * B.n_tiles + tile] = t;
 }
 
 __global__ void __launch_bounds__(NE_TILE) k_init_v_scale(DevBatch B)
@@ -526,7 +541,7 @@ __global__ void __launch_bounds__(NE_TILE) k_init_v_scale(DevBatch B)
     const int tile = blockIdx.x;
     const RepDev& P = B.rep[B.tile_rep[tile]];
     if (threadIdx.x < 32) {
-        const double ke = ne_warp_tile_sum(B.partA, NPA, 3, P.tile0, P.ntile);
+        const double ke = ne_warp_part_sum(B.partA + (size_t)3 * B.n_tiles + P.tile0, P.ntile);
         const double kB = 8.617333262e-5;
         if (threadIdx.x == 0) s_sc = sqrt((P.kT / kB) / (2.0 * ke / (P.dof * kB)));
     }
@@ -587,10 +602,10 @@ __global__ void k_msd_sample(DevBatch B, double* acc)
     const int rep = blockIdx.x;
     const RepDev& P = B.rep[rep];
     double s[4];
-    s[0] = ne_warp_tile_sum(B.partB, NPB, PB_UX, P.tile0, P.ntile);
-    s[1] = ne_warp_tile_sum(B.partB, NPB, PB_UY, P.tile0, P.ntile);
-    s[2] = ne_warp_tile_sum(B.partB, NPB, PB_UZ, P.tile0, P.ntile);
-    s[3] = ne_warp_tile_sum(B.partB, NPB, PB_U2, P.tile0, P.ntile);
+    s[0] = ne_warp_part_sum(B.partB + (size_t)PB_UX * B.n_tiles + P.tile0, P.ntile);
+    s[1] = ne_warp_part_sum(B.partB + (size_t)PB_UY * B.n_tiles + P.tile0, P.ntile);
+    s[2] = ne_warp_part_sum(B.partB + (size_t)PB_UZ * B.n_tiles + P.tile0, P.ntile);
+    s[3] = ne_warp_part_sum(B.partB + (size_t)PB_U2 * B.n_tiles + P.tile0, P.ntile);
     if (threadIdx.x != 0) return;
     const double invN = 1.0 / P.n;
     acc[rep] += s[3] * invN - (s[0] * s[0] + s[1] * s[1] + s[2] * s[2]) * invN * invN;
@@ -654,7 +669,7 @@ void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long*
     if (mixed)
         k_step_mixed<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, j, do_close, do_open);
     else
-        k_step<false><<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, j, do_close, do_open);
+        k_step<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, j, do_close, do_open);
     if (B.trace) k_trace_T<<<1, 32, 0, st>>>(B, step_base, j);
 }
 
@@ -664,17 +679,12 @@ void launch_prep(const DevBatch& B, const Sched& S, bool mixed, const long long*
     if (mixed)
         k_step_mixed<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, 0, 0, 0);
     else
-        k_step<false><<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, 0, 0, 0);
+        k_step<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, 0, 0, 0);
 }
 
 void launch_npt_box(const DevBatch& B, const Sched& S, const long long* step_base, int j, cudaStream_t st)
 {
     k_npt_box<<<B.n_rep, 32, 0, st>>>(B, S, step_base, j);
-}
-
-void launch_wrap32(const DevBatch& B, cudaStream_t st)
-{
-    k_wrap32<<<B.n_tiles, NE_TILE, 0, st>>>(B);
 }
 
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,

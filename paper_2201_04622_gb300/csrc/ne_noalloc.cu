@@ -22,7 +22,6 @@ namespace {
 
 constexpr int NA = NE_NOALLOC_MAX_ATOMS;
 constexpr int NK = NE_NOALLOC_MAX_KNOTS;
-constexpr int TPA = 4;
 constexpr int TILES = (NA + NE_TILE - 1) / NE_TILE;
 constexpr int CELLS = 2 * NA + 27;
 
@@ -39,24 +38,28 @@ constexpr size_t O_POSF = O_POS32 + up(sizeof(float4) * NA);
 constexpr size_t O_PBUILD = O_POSF + up(sizeof(float4) * NA);
 constexpr size_t O_FORCE32 = O_PBUILD + up(sizeof(float4) * NA);
 constexpr size_t O_FORCE64 = O_FORCE32 + up(sizeof(float4) * NA);
-constexpr size_t O_DF64 = O_FORCE64 + up(sizeof(double) * 3 * NA);
-constexpr size_t O_NBR = O_DF64 + up(sizeof(double) * NA);
+constexpr size_t O_POS64 = O_FORCE64 + up(sizeof(double) * 3 * NA);
+// the candidate rows and, over them, the pairs' f'(r)/r (mixed: neighbour and
+// f'(r)/r): an atom's lanes have read its row (NE_NMAX ints) before they write
+// its NE_SMAX 8-byte entries
+constexpr size_t O_NBR = O_POS64 + up(sizeof(ned4) * NA);
+static_assert(sizeof(int) * NE_NMAX >= sizeof(double) * NE_SMAX, "one row holds the other");
 constexpr size_t O_NCNT = O_NBR + up(sizeof(int) * (size_t)NA * NE_NMAX);
 constexpr size_t O_SL = O_NCNT + up(sizeof(int) * NA);
 constexpr size_t O_SCNT = O_SL + up(sizeof(int) * (size_t)NA * NE_SMAX);
-constexpr size_t O_CELLOF = O_SCNT + up(sizeof(int) * NA * TPA);
+constexpr size_t O_CELLOF = O_SCNT + up(sizeof(int) * NA);
 constexpr size_t O_CSLOT = O_CELLOF + up(sizeof(int) * NA);
 constexpr size_t O_CRAW = O_CSLOT + up(sizeof(int) * NA);
 constexpr size_t O_CSORT = O_CRAW + up(sizeof(int) * NA);
 constexpr size_t O_CSTART = O_CSORT + up(sizeof(float4) * NA);
 constexpr size_t O_CCOUNT = O_CSTART + up(sizeof(int) * (CELLS + 1));
 constexpr size_t O_PARTA = O_CCOUNT + up(sizeof(int) * CELLS);
-constexpr size_t O_PARTB = O_PARTA + up(sizeof(double) * TILES * NPA);
+constexpr size_t O_PARTB = O_PARTA + up(sizeof(double) * TILES * NE_PAIR_SUB * NPA);
 constexpr size_t O_TOT = O_PARTB + up(sizeof(double) * TILES * NPB);
 constexpr size_t O_REP = O_TOT + up(sizeof(double) * NTOT);
 constexpr size_t O_TILEREP = O_REP + up(sizeof(RepDev));
 constexpr size_t O_SMALL = O_TILEREP + up(sizeof(int) * TILES);
-// small words: tile_done, flags, building, status (ints), rebuilds, step counter (8 bytes), nl_done
+// small words: tile_done, flags, building, status (ints), rebuilds (8 bytes), nl_done
 constexpr size_t O_END = O_SMALL + 256;
 static_assert(O_END <= NE_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds NE_NOALLOC_SCRATCH_BYTES");
 
@@ -159,6 +162,8 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     for (int d = 0; d < 3; ++d) {
         R.L[d] = box[d];
         R.invL[d] = 1.0 / box[d];
+        R.Lf[d] = (float)R.L[d];
+        R.iLf[d] = (float)R.invL[d];
         R.nc[d] = (int)std::min(std::floor(box[d] / rc), 1024.0);
     }
     while ((long long)R.nc[0] * R.nc[1] * R.nc[2] > 2ll * n + 27) {
@@ -184,7 +189,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     B.n_tot = n;
     B.n_max = n;
     B.n_tiles = R.ntile;
-    B.tpa = TPA;
+    B.g = ne::lanes_per_atom(n);
     B.rep = (const RepDev*)(base + O_REP);
     B.tile_rep = (const int*)(base + O_TILEREP);
     B.x = const_cast<double*>(x_dev);
@@ -193,10 +198,12 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     B.pbuild = (float4*)(base + O_PBUILD);
     B.f32 = (float4*)(base + O_FORCE32);
     B.f64 = (double*)(base + O_FORCE64);
-    B.dF64 = (double*)(base + O_DF64);
+    if (prec == NE_FP64) B.pos64 = (ned4*)(base + O_POS64);
+    B.sms = TILES * NE_PAIR_SUB;  // bounds the list kernel's grid only, at this size
+    B.gs = (double*)(base + O_NBR);
     B.nbr = (int*)(base + O_NBR);
     B.ncnt = (int*)(base + O_NCNT);
-    B.sl = (int*)(base + O_SL);
+    B.sl = (int*)(base + (prec == NE_FP64 ? O_SL : O_NBR));
     B.scnt = (int*)(base + O_SCNT);
     B.cellof = (int*)(base + O_CELLOF);
     B.cslot = (int*)(base + O_CSLOT);
@@ -213,8 +220,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     B.building = small + 2;
     B.status = small + 3;
     B.rebuilds = (unsigned long long*)(base + O_SMALL + 16);
-    long long* step_ctr = (long long*)(base + O_SMALL + 24);
-    B.nl_done = (unsigned*)(base + O_SMALL + 32);
+    B.nl_done = (unsigned*)(base + O_SMALL + 24);
     B.trace_stride = 1;
     Tables& t = B.tab;
     t.pf32 = (const float4*)(base + O_PF32);
@@ -233,6 +239,8 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     t.rc2f = (float)(rc * rc);
     t.rmin2f = (float)(NE_RMIN * NE_RMIN);
     t.inv_h_rhof = (float)t.inv_h_rho;
+    t.rho_maxf = (float)eam->rho_max;
+    t.ihr_lo = (float)(t.inv_h_rho - (double)t.inv_h_rhof);
 
     // ---- what must start at zero (the scratch keeps the previous call's contents)
     if (cudaMemcpyAsync(base + O_REP, &R, sizeof(RepDev), cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -249,12 +257,9 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     ne::launch_tables(theta, nk, rc, eam->rho_max, (float4*)(base + O_PF32), (ned4*)(base + O_PF64),
                       (float4*)(base + O_F32), (ned4*)(base + O_F64), st);
     const bool mixed = prec == NE_MIXED;
-    Sched S{};
-    S.kind = SCHED_FIXED;
     ne::launch_nl_build(B, 1, 0, st);
-    if (mixed) ne::launch_wrap32(B, st);
-    ne::launch_density(B, mixed, step_ctr, 0, st);
-    ne::launch_force(B, S, mixed, step_ctr, 0, 0, st);
+    ne::launch_pass1(B, mixed, st);
+    ne::launch_pass2(B, mixed, st);
     ne::launch_export(B, mixed, f_dev, e_dev, st);
     if (cudaGetLastError() != cudaSuccess) return NE_ECUDA;
     int bits = 0;
