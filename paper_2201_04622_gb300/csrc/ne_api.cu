@@ -88,6 +88,8 @@ struct ne_ctx {
     XRep* xrep = nullptr;
     double* lam_tab = nullptr;  // lambda of each step of the crystal runner's schedule
     long long lam_cap = 0;
+    double* run_lam = nullptr;  // lambda of the steps of the current multi-kernel run
+    long long run_lam_cap = 0;
     Sched lam_sched{};          // the schedule lam_tab holds
     bool lam_valid = false;
     CrPlan plan;                // launch plan of the last crystal-runner batch
@@ -234,6 +236,7 @@ ne_status species_tables(ne_ctx* ctx, const ne_md_params& m, int n, double c1, R
         M += m.mass_s[sp[a]];
     }
     R.nsp = m.n_species;
+    R.inv_w = 1.0 / M;
     R.sp = m.species_dev;
     R.M = M;
     for (int q = 0; q < m.n_species; ++q) {
@@ -289,6 +292,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
         if (!(m.mass > 0)) return fail(ctx, NE_EINVAL, "mass must be positive");
         const double gamma = m.damp > 0 ? 1.0 / m.damp : 0.0;
         R.c1 = std::exp(-gamma * m.dt);
+        R.c1f = (float)R.c1;
         R.c2 = std::sqrt((1.0 - R.c1 * R.c1) * kB * m.T / m.mass);
         R.hdt_m = 0.5 * m.dt / m.mass;
         R.kT = kB * m.T;
@@ -302,6 +306,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
         R.cell_off = cells;
         cells += R.nc[0] * R.nc[1] * R.nc[2];
         R.dof = m.fix_cm ? 3 * n - 3 : 3 * n;
+        R.inv_w = 1.0 / n;
         R.seed = m.seed;
         R.replica = m.replica;
         if (m.replica >= (1u << 28)) return fail(ctx, NE_EINVAL, "replica id must be < 2^28");
@@ -432,29 +437,48 @@ void one_step(const DevBatch& B, const Sched& S, bool mixed, const long long* ct
     force_eval(B, mixed, st);
     grad_at(B, mixed, ga, ctr, j, st);
     ne::launch_step(B, S, mixed, ctr, j, first ? 0 : 1, 1, st);
-    if (B.npt_any) ne::launch_npt_box(B, S, ctr, j, st);
+}
+
+// lambda of the run's steps [s_begin, s_begin + n_steps + 1], formed once per
+// run (FP64) and read by the step kernel
+ne_status run_lambda(ne_ctx* ctx, DevBatch& B, const Sched& S, long long s_begin, long long n_steps, cudaStream_t st)
+{
+    const long long need = n_steps + 2;
+    if (need > ctx->run_lam_cap) {
+        // every earlier run ended with a synchronisation of its stream
+        if (ctx->run_lam) cudaFree(ctx->run_lam);
+        ctx->run_lam = nullptr;
+        ctx->run_lam_cap = 0;
+        NE_CU(cudaMalloc((void**)&ctx->run_lam, sizeof(double) * (size_t)need));
+        ctx->run_lam_cap = need;
+    }
+    NE_CU(ne::launch_lambda_table(S, s_begin, need, ctx->run_lam, st));
+    B.lam = ctx->run_lam;
+    B.lam_s0 = s_begin;
+    return NE_OK;
 }
 
 // Run steps [0, n_steps) of schedule S from the state held in B, then the
 // closing half kick.  Chunks of G steps are captured once into a CUDA graph
 // and replayed; the step index lives in device memory, so one graph serves
 // every chunk.
-ne_status run_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, long long s_begin,
+ne_status run_steps(ne_ctx* ctx, DevBatch& B, const Sched& S, bool mixed, long long s_begin,
                     long long n_steps, cudaStream_t st, double* msd_acc = nullptr,
                     long long msd_from = 0, int msd_stride = 0, const GradAcc* ga = nullptr)
 {
     long long* ctr = ctx->step_ctr;
     NE_CU(cudaMemcpyAsync(ctr, &s_begin, sizeof(long long), cudaMemcpyHostToDevice, st));
     NE_CU(cudaStreamSynchronize(st));
+    ne_status ls = run_lambda(ctx, B, S, s_begin, n_steps, st);
+    if (ls) return ls;
     // list from the lattice sites (from the positions when a barostat may
     // have changed the box since the sites were made)
     ne::launch_nl_build(B, 1, B.npt_any ? 0 : 1, st);
-    ne::launch_prep(B, S, mixed, ctr, st);
-    long long s = 0;
+    ne::launch_step(B, S, mixed, ctr, 0, 0, 0, st);
+    long long s = 0, s_ctr = 0;  // steps done, and those the counter has been advanced by
     // first step: no closing kick
     if (n_steps > 0) {
         one_step(B, S, mixed, ctr, 0, 1, st, ga);
-        ne::launch_advance(ctr, 1, st);
         s = 1;
         if (msd_acc && msd_stride > 0 && s > msd_from && (s - msd_from) % msd_stride == 0)
             ne::launch_msd_sample(B, msd_acc, st);
@@ -471,7 +495,7 @@ ne_status run_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, 
         NE_CU(cudaEventRecord(ev, st));
         NE_CU(cudaStreamWaitEvent(cs, ev, 0));
         NE_CU(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        for (int j = 0; j < G; ++j) one_step(B, S, mixed, ctr, j, 0, cs, ga);
+        for (int j = 0; j < G; ++j) one_step(B, S, mixed, ctr, j + 1, 0, cs, ga);
         ne::launch_advance(ctr, G, cs);
         cudaError_t ce = cudaStreamEndCapture(cs, &graph);
         if (ce != cudaSuccess) {
@@ -492,21 +516,26 @@ ne_status run_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, 
             if (ce != cudaSuccess) break;
         }
         s += reps * G;
+        s_ctr = reps * G;
         cudaGraphExecDestroy(exec);
         cudaStreamDestroy(cs);
         cudaEventDestroy(ev);
         if (ce != cudaSuccess) return fail(ctx, NE_ECUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
     }
     for (; s < n_steps; ++s) {
-        one_step(B, S, mixed, ctr, 0, 0, st, ga);
-        ne::launch_advance(ctr, 1, st);
+        // (the counter moves on only where the offset would leave its type)
+        if (s - s_ctr >= (1 << 30)) {
+            ne::launch_advance(ctr, s - s_ctr, st);
+            s_ctr = s;
+        }
+        one_step(B, S, mixed, ctr, (int)(s - s_ctr), 0, st, ga);
         if (msd_acc && msd_stride > 0 && s + 1 > msd_from && (s + 1 - msd_from) % msd_stride == 0)
             ne::launch_msd_sample(B, msd_acc, st);
     }
     // closing half kick of the last step
     force_eval(B, mixed, st);
-    grad_at(B, mixed, ga, ctr, 0, st);
-    ne::launch_step(B, S, mixed, ctr, 0, 1, 0, st);
+    grad_at(B, mixed, ga, ctr, (int)(s - s_ctr), st);
+    ne::launch_step(B, S, mixed, ctr, (int)(s - s_ctr), 1, 0, st);
     NE_CU(cudaGetLastError());
     return NE_OK;
 }
@@ -514,14 +543,16 @@ ne_status run_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, 
 // Per-kernel timing: the same steps launched one by one with CUDA events
 // around each kernel on the launching stream.  kinds: 0 list build,
 // 1 pass 1 (density), 2 pass 2 (forces), 3 fused step.
-ne_status profile_steps(ne_ctx* ctx, const DevBatch& B, const Sched& S, bool mixed, long long s_begin,
+ne_status profile_steps(ne_ctx* ctx, DevBatch& B, const Sched& S, bool mixed, long long s_begin,
                         long long n_steps, double* ms, long long* counts, cudaStream_t st)
 {
     long long* ctr = ctx->step_ctr;
     NE_CU(cudaMemcpyAsync(ctr, &s_begin, sizeof(long long), cudaMemcpyHostToDevice, st));
     NE_CU(cudaStreamSynchronize(st));
+    ne_status ls = run_lambda(ctx, B, S, s_begin, n_steps, st);
+    if (ls) return ls;
     ne::launch_nl_build(B, 1, 1, st);
-    ne::launch_prep(B, S, mixed, ctr, st);
+    ne::launch_step(B, S, mixed, ctr, 0, 0, 0, st);
     std::vector<cudaEvent_t> ev(2 * 4 * (size_t)n_steps);
     for (auto& e : ev) NE_CU(cudaEventCreate(&e));
     for (long long s = 0; s < n_steps; ++s) {
@@ -566,6 +597,7 @@ Sched make_sched(const ne_md_params& m)
     S.t_s = m.t_s;
     S.lambda_f = m.lambda_f;
     S.dt = m.dt;
+    S.hdtf = 0.5f * (float)m.dt;
     S.path = m.path;
     S.fn = m.lambda_fn;
     S.stream = m.path == NE_PATH_FL ? STREAM_FL : STREAM_RS;
@@ -694,7 +726,7 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
                     ctx->pbuild, ctx->f32, ctx->f64, ctx->pos64, ctx->gs, ctx->rho, ctx->xi64, ctx->xi32,
                     ctx->nbr, ctx->ncnt, ctx->sl, ctx->scnt, ctx->cellof, ctx->cslot, ctx->craw, ctx->csort,
                     ctx->cstart, ctx->ccount, ctx->nl_done, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
-                    ctx->tile_done, ctx->flags, ctx->building, ctx->status, ctx->tile_rep, ctx->rep, ctx->step_ctr, ctx->rebuilds, ctx->xrep, ctx->work, ctx->st_vec, ctx->st_dist, ctx->lam_tab,
+                    ctx->tile_done, ctx->flags, ctx->building, ctx->status, ctx->tile_rep, ctx->rep, ctx->step_ctr, ctx->rebuilds, ctx->xrep, ctx->work, ctx->st_vec, ctx->st_dist, ctx->lam_tab, ctx->run_lam,
                     ctx->bins};
     for (void* p : ptrs)
         if (p) cudaFree(p);

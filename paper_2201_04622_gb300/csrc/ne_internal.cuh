@@ -61,6 +61,7 @@ struct RepDev {
     double L[3], invL[3];
     float Lf[3], iLf[3];  // the same in FP32 (a conversion costs an FP64 slot)
     double k;        // Einstein spring
+    float c1f;       // c1 in FP32
     double c1, c2;   // Ornstein-Uhlenbeck coefficients
     double hdt_m;    // dt / (2 m)
     double kT;
@@ -85,6 +86,7 @@ struct RepDev {
     int nsp;
     const unsigned char* sp;
     double M;
+    double inv_w;    // 1 / n, or 1 / M with species tables
     double ms[NE_MAX_SPECIES_DEV], ks[NE_MAX_SPECIES_DEV], c2s[NE_MAX_SPECIES_DEV], hdts[NE_MAX_SPECIES_DEV];
 };
 
@@ -96,6 +98,7 @@ struct Sched {
     double lam_a, lam_b;   // SCHED_FIXED: lambda before / after the jump
     long long s0;          // SCHED_FIXED: step of the jump
     double dt;
+    float hdtf;            // dt / 2 in FP32
     int kind, path, fn, stream, fix_cm;
 };
 
@@ -147,6 +150,8 @@ struct DevBatch {
     double* tot;
     unsigned* tile_done;
     unsigned* nl_done;
+    const double* lam; // lambda of the run's steps from lam_s0 on
+    long long lam_s0;
     double* W;         // [n_rep][2]
     double* Wcum;      // nullable, [n_rep][2][t_s + 1]
     double* trace;     // nullable, [rows][8], single replica
@@ -256,6 +261,23 @@ __device__ __forceinline__ void ne_normals32(uint4 w, float z[3])
     z[2] = r1 * c3;
 }
 
+// Component c of those normals alone, for one thread per component.
+__device__ __forceinline__ double ne_normal64(uint4 w, int c)
+{
+    const double s = 2.3283064365386963e-10;  // 2^-32
+    const double u0 = ((double)(c < 2 ? w.x : w.z) + 0.5) * s, u1 = ((double)(c < 2 ? w.y : w.w) + 0.5) * s;
+    return sqrt(-2.0 * log(u0)) * (c == 1 ? sinpi(2.0 * u1) : cospi(2.0 * u1));
+}
+
+__device__ __forceinline__ float ne_normal32(uint4 w, int c)
+{
+    const float s = 5.9604644775390625e-8f;  // 2^-24
+    const float u0 = ((float)((c < 2 ? w.x : w.z) >> 8) + 0.5f) * s, u1 = ((float)((c < 2 ? w.y : w.w) >> 8) + 0.5f) * s;
+    float sn, cs;
+    sincospif(2.0f * u1, &sn, &cs);
+    return sqrtf(-2.0f * logf(u0)) * (c == 1 ? sn : cs);
+}
+
 // ------------------------------------------------------------------ misc
 // double-float (hi + lo, |lo| <= ulp(hi) / 2) sum of two such numbers from
 // FP32 operations (TwoSum of the high parts, the low parts added to its error)
@@ -315,10 +337,9 @@ void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t 
 int lanes_per_atom(int n_tot);  // the pair passes' lanes per atom for a batch of n_tot atoms
 void launch_pass1(const DevBatch& B, bool mixed, cudaStream_t st);
 void launch_pass2(const DevBatch& B, bool mixed, cudaStream_t st);
+// (0, 0): no kick and no step, the copies, sums and normals of the first step
 void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
                  int j, int do_close, int do_open, cudaStream_t st);
-void launch_prep(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
-                 cudaStream_t st);
 void launch_advance(long long* step_base, long long by, cudaStream_t st);
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,
                   double* z, cudaStream_t st);
@@ -341,5 +362,4 @@ void launch_backward(const DevBatch& B, bool mixed, double gE, double* gtheta,
 int backward_bin_blocks(const DevBatch& B);
 cudaError_t prepare_backward(const DevBatch& B);  // the mixed backward kernel's shared-memory attribute
 void launch_virial(const DevBatch& B, double* out, cudaStream_t st);
-void launch_npt_box(const DevBatch& B, const Sched& S, const long long* step_base, int j, cudaStream_t st);
 }  // namespace ne

@@ -2,6 +2,8 @@
 // spring + work increment + BAOAB Langevin step, Maxwell-Boltzmann initial
 // velocities, the spring energy, and small reductions (msd samples, exported
 // energies/forces).
+#include <type_traits>
+
 #include "ne_internal.cuh"
 
 namespace {
@@ -11,12 +13,8 @@ namespace {
 // F_E = -k u and, with the centre of mass fixed, their replica means:
 //   Frenkel-Ladd (eq. interp): (1 - lambda) F0 + lambda F_E
 //   reversible scaling (eq. H_rs): lambda F0
-__device__ __forceinline__ double blend(int path, double lam, double F0, double FE)
-{
-    return path == 0 ? (1.0 - lam) * F0 + lam * FE : lam * F0;
-}
-
-// One thread per atom.  With s the global step and Lambda(s) the schedule:
+//
+// With s the global step and Lambda(s) the schedule:
 //   do_close: v += dt/2m F(x_s; Lambda(s))      (second half kick of step s-1)
 //   do_open:  W += (Lambda(s+1) - Lambda(s)) dH/dlambda(x_s)   (first thread
 //             of the replica; the discrete work sum of Sec. II.A)
@@ -37,8 +35,8 @@ __device__ __forceinline__ double blend(int path, double lam, double F0, double 
 //   d ln V = m [(dof kT + lambda W)/(3V) - P0] dt + sqrt(2 kT m dt / V) eta,
 // W the virial at x_s (replica totals of pass 2 of this step), eta the first
 // normal of Philox stream 5 at (atom 0, step s).  Every block computes the
-// same factor; positions scale about the origin here, the box in k_npt_box
-// after this kernel.
+// same factor and scales its positions about the origin; the replica's last
+// block then scales the box.
 //
 // Per axis (RepDev.npt = 2, for non-cubic cells such as hcp, whose c/a the
 // isotropic form cannot change): each eps_a = ln L_a takes the same kind of
@@ -108,297 +106,246 @@ __device__ void step_work(const DevBatch& B, const Sched& S, const double* T, in
     }
 }
 
-__global__ void __launch_bounds__(NE_TILE)
+// One thread per atom and component: warp w of a tile's block has component
+// w / 2 of 32 atoms.  GB300 issues an FP64 instruction of a warp every ~64
+// cycles, so a step's time at small sizes is the number of them in one warp: with
+// one thread an atom the FP64 step took 17 us at 128 atoms, now 11 (33 and 34
+// at 40,480, where the FP64 Box-Muller, twice the rest, sets it), the mixed one
+// 7.7 us at 2000 atoms, now 6.6.
+// What every atom of the block shares (lambda, the centre-of-mass means, the
+// barostat's factors, the box) is formed once, a lane each, from the schedule's
+// table and the replica's totals.  Mixed precision: velocities, kicks and
+// thermostat in FP32, each drift added to the FP64 position once, tile sums in
+// double-float -- the crystal runner's precision.
+constexpr int STEP_THREADS = 3 * NE_TILE;
+
+template <bool MIXED>
+__global__ void __launch_bounds__(STEP_THREADS)
     k_step(DevBatch B, Sched S, const long long* __restrict__ step_base, int j, int do_close, int do_open)
 {
-    __shared__ double red[NPB][NE_TILE];
+    using R = typename std::conditional<MIXED, float, double>::type;
+    __shared__ double s_lam[2], s_mu[3], s_L[3];
+    __shared__ R s_mean[9];             // mean F0, spring and noise terms (see below)
+    __shared__ float s_Lf[3], s_iLf[3]; // box and 1 / box after this step's scaling
+    __shared__ R s_tab[4][NE_MAX_SPECIES_DEV + 1];  // m, k, c2, dt / 2m: species 0.., the replica's last
+    __shared__ float s_w[3][NE_TILE], s_d2[3][NE_TILE];
+    __shared__ int s_code[3][NE_TILE];
+    __shared__ double s_x64[MIXED ? 1 : 3][NE_TILE];
+    __shared__ double s_red[MIXED ? 1 : 5][3][NE_TILE + 1];
+    __shared__ float2 s_dff[MIXED ? 5 : 1][6];
     const int tile = blockIdx.x;
     const int rep = B.tile_rep[tile];
     const RepDev& P = B.rep[rep];
-    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x;
+    const int c = threadIdx.x / NE_TILE, al = threadIdx.x % NE_TILE;  // component (warp-uniform), atom of the tile
+    const int a = (tile - P.tile0) * NE_TILE + al;
     const bool valid = a < P.n;
-    const int i = P.off + (valid ? a : 0);
+    const size_t e = 3 * (size_t)(P.off + (valid ? a : 0)) + c;
     const long long s = *step_base + j;
     const double* T = B.tot + (size_t)rep * NTOT;
-    const double lam_s = ne_sched_lambda(S, s);
-    const double lam_n = ne_sched_lambda(S, s + 1);
-    const double invN = 1.0 / P.n;
     const bool draw = do_open || !do_close;  // a step follows: its normals
-    double part[NPB] = {};
-    int bad = 0;
-    if (valid) {
-        double x[3], v[3], u[3], F0[3], mF0[3], mFE[3];
-        double Lb[3] = {P.L[0], P.L[1], P.L[2]};  // box after this step (the barostat scales it)
-        for (int c = 0; c < 3; ++c) {
-            x[c] = B.x[3 * i + c];
-            v[c] = B.v[3 * i + c];
-            u[c] = x[c] - B.x0[3 * i + c];
-        }
-        for (int c = 0; c < 3; ++c) F0[c] = B.f64[3 * i + c];
-        // this atom's mass, spring, noise amplitude and half-step factor
-        // (one species, or its species' entries)
-        const int q = P.nsp ? (int)P.sp[a] : 0;
-        const double mi = P.nsp ? P.ms[q] : P.m, ki = P.nsp ? P.ks[q] : P.k;
-        const double c2i = P.nsp ? P.c2s[q] : P.c2, hdti = P.nsp ? P.hdts[q] : P.hdt_m;
-        for (int c = 0; c < 3; ++c) {
-            if (P.nsp) {  // mass-weighted constraint: F_i -= m_i sum_j F_j / M
-                mF0[c] = S.fix_cm ? mi * T[TOT_F0X + c] / P.M : 0.0;
-                mFE[c] = S.fix_cm ? -mi * T[TOT_UX + c] / P.M : 0.0;  // TOT_UX: sum_j k_j u_j
-            } else {
-                mF0[c] = S.fix_cm ? T[TOT_F0X + c] * invN : 0.0;
-                mFE[c] = S.fix_cm ? -P.k * T[TOT_UX + c] * invN : 0.0;
-            }
-        }
-        if (do_close) {
-            for (int c = 0; c < 3; ++c)
-                v[c] += hdti * blend(S.path, lam_s, F0[c] - mF0[c], -ki * u[c] - mFE[c]);
-        }
-        part[PB_KE] = 0.5 * mi * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-        if (do_open) {
-            // velocity increments of the thermostat: c2 (xi - mean xi) for one
-            // species; c2_i xi_i - sum_j m_j c2_j xi_j / M with species tables
-            double dv[3];
-            for (int c = 0; c < 3; ++c) {
-                const double xi = B.xi64[3 * i + c];
-                if (P.nsp) dv[c] = c2i * xi - (S.fix_cm ? T[TOT_XIX + c] / P.M : 0.0);
-                else dv[c] = P.c2 * (S.fix_cm ? xi - T[TOT_XIX + c] * invN : xi);
-            }
-            for (int c = 0; c < 3; ++c) {
-                v[c] += hdti * blend(S.path, lam_n, F0[c] - mF0[c], -ki * u[c] - mFE[c]);
-                x[c] += 0.5 * S.dt * v[c];
-                v[c] = P.c1 * v[c] + dv[c];
-                x[c] += 0.5 * S.dt * v[c];
-            }
-            if (P.npt) {
-                double mu[3];
-                npt_scale(P, T, lam_n, s, S.dt, mu);
-                for (int c = 0; c < 3; ++c) {
-                    x[c] *= mu[c];
-                    Lb[c] = mu[c] * P.L[c];
-                }
-            }
-            for (int c = 0; c < 3; ++c) u[c] = x[c] - B.x0[3 * i + c];
-        }
-        for (int c = 0; c < 3; ++c) {
-            if (!isfinite(x[c]) || !isfinite(v[c])) bad |= ST_ENAN;
-            B.x[3 * i + c] = x[c];
-            B.v[3 * i + c] = v[c];
-            part[PB_UX + c] = P.nsp ? ki * u[c] : u[c];
-        }
-        part[PB_U2] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        part[PB_UE] = 0.5 * ki * part[PB_U2];
-        // x wrapped, its image against the list build's and the displacement
-        // from there (image indices in FP32: exact integers)
-        const float4 pb = B.pbuild[i];
-        const float pbx[3] = {pb.x, pb.y, pb.z};
-        double w64[3];
-        float w[3], d2 = 0.f;
-        int code = 0;
-        for (int c = 0; c < 3; ++c) {
-            const float Lf = (float)Lb[c], iLf = 1.f / Lf;
-            w64[c] = x[c];
-            w[c] = (float)x[c];
-            const float n = floorf(w[c] * iLf);
-            if (n != 0.f) {
-                w64[c] = x[c] - Lb[c] * (double)n;
-                w[c] = (float)w64[c];
-            }
-            const float nb = rintf((w[c] - pbx[c]) * iLf), d = fmaf(-Lf, nb, w[c] - pbx[c]);
-            code = 3 * code + (int)nb;
-            d2 = fmaf(d, d, d2);
-        }
-        B.pos32[i] = make_float4(w[0], w[1], w[2], __int_as_float(code));
-        B.pos64[i] = ned4{w64[0], w64[1], w64[2], 0.0};
-        if (d2 > P.half_skin2) B.flags[rep] = 1;
-        if (draw) {
-            double z[3];
-            ne_normals64(ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
-                                         (unsigned long long)(do_open ? s + 1 : s)),
-                         z);
-            const double wq = P.nsp ? mi * c2i : 1.0;  // the velocity increments' momentum: sum m_j c2_j xi_j
-            for (int c = 0; c < 3; ++c) {
-                B.xi64[3 * i + c] = z[c];
-                part[PB_XIX + c] = wq * z[c];
-            }
-        }
-    }
-    if (bad) ne_set_status(B.status, bad);
-    if (do_open && valid && a == 0) step_work(B, S, T, rep, s, lam_s, lam_n);
-    for (int q = 0; q < NPB; ++q) red[q][threadIdx.x] = part[q];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int q = 0; q < NPB; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < NPB; ++q) B.partB[(size_t)q * B.n_tiles + tile] = red[q][0];
-    }
-}
-
-// The mixed-precision step: the same steps as k_step, with the velocity
-// arithmetic (kicks, thermostat) in FP32, each drift added to the FP64
-// position once, and the tile sums in double-float -- the crystal runner's
-// precision, keeping GB300's FP64 pipe (1/64 of FP32) to a few conversions
-// an atom.  Thread 0 forms the block's replica scalars (lambda at s and s + 1,
-// the centre-of-mass means, the barostat's factors, the box after it) in FP64
-// once and the second warp the FP32 mass, spring and thermostat tables.
-__global__ void __launch_bounds__(NE_TILE)
-    k_step_mixed(DevBatch B, Sched S, const long long* __restrict__ step_base, int j, int do_close, int do_open)
-{
-    __shared__ double s_lam[2], s_mu[3];
-    __shared__ float s_mean[9];  // mean F0, spring and noise terms (see below)
-    __shared__ float s_box[8];   // box and 1 / box after this step's scaling, c1, (skin / 2)^2
-    __shared__ float s_tab[4][NE_MAX_SPECIES_DEV + 1];  // m, k, c2, dt / 2m: species 0.., the replica's last
-    __shared__ float2 s_w[NPB][NE_TILE / 32];
-    const int tile = blockIdx.x;
-    const int rep = B.tile_rep[tile];
-    const RepDev& P = B.rep[rep];
-    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x;
-    const bool valid = a < P.n;
-    const int i = P.off + (valid ? a : 0);
-    const long long s = *step_base + j;
-    const double* T = B.tot + (size_t)rep * NTOT;
     if (threadIdx.x < 32) {
-        // the replica scalars, one a lane, the lanes running the same
-        // instructions (GB300 issues an FP64 warp instruction at the same cost
-        // for one lane as for 32, so a serial chain on one thread held the
-        // whole block): lambda at s and s + 1 in lanes of each parity; the
-        // barostat's factors (lane 0); one division for the centre-of-mass
-        // means (lanes 0-8: mean F0, the spring's mean and the noise mean,
-        // per unit mass with species tables, mass-weighted) and 1 / box
-        // (lanes 9-11); the box (lanes 12-14), c1 and (skin / 2)^2
-        const int l = threadIdx.x, c = l % 3;
-        const double lam = ne_sched_lambda(S, s + (l & 1));
-        if (l < 2) s_lam[l] = lam;
+        // lanes 0-8: mean F0, the spring's mean and the noise mean (per unit
+        // mass with species tables: the mass-weighted constraint); 9-11 the
+        // box after the barostat's step; 12, 13 lambda at s and s + 1
+        const int l = threadIdx.x, d = l % 3;
+        const double* lam = B.lam + (s - B.lam_s0);
         double mu[3] = {1.0, 1.0, 1.0};
         if (do_open && P.npt) {
-            const double lam_n1 = __shfl_sync(0xffffffffu, lam, 1);
-            if (l == 0) npt_scale(P, T, lam_n1, s, S.dt, mu);
+            if (l == 0) npt_scale(P, T, lam[1], s, S.dt, mu);
             for (int q = 0; q < 3; ++q) mu[q] = __shfl_sync(0xffffffffu, mu[q], 0);
         }
-        const double muc = c == 0 ? mu[0] : (c == 1 ? mu[1] : mu[2]);
-        double num, den = P.nsp ? P.M : (double)P.n;
-        if (l < 3) num = T[TOT_F0X + c];
-        else if (l < 6) num = -(P.nsp ? 1.0 : P.k) * T[TOT_UX + c];
-        else if (l < 9) num = T[TOT_XIX + c];
-        else {
-            num = P.invL[c];
-            den = muc;
+        const double muc = d == 0 ? mu[0] : (d == 1 ? mu[1] : mu[2]);
+        if (l < 9) {
+            double v = T[l < 3 ? TOT_F0X + d : (l < 6 ? TOT_UX + d : TOT_XIX + d)];
+            if (l >= 3 && l < 6) v *= P.nsp ? -1.0 : -P.k;
+            s_mean[l] = S.fix_cm ? (R)(v * P.inv_w) : (R)0;
+        } else if (l < 12) {
+            const double L = P.npt ? muc * P.L[d] : P.L[d];
+            s_mu[d] = muc;
+            s_L[d] = L;
+            s_Lf[d] = P.npt ? (float)L : P.Lf[d];
+            s_iLf[d] = P.npt ? 1.f / (float)L : P.iLf[d];
+        } else if (l < 14) {
+            s_lam[l - 12] = lam[l - 12];
         }
-        const double quo = num / den;
-        if (l < 9) s_mean[l] = S.fix_cm ? (float)quo : 0.f;
-        else if (l < 12) s_box[3 + c] = (float)quo;
-        else if (l < 15) s_box[c] = (float)(muc * P.L[c]);
-        else if (l == 15) s_box[6] = (float)P.c1;
-        else if (l == 16) s_box[7] = (float)P.half_skin2;
-        if (l < 3) s_mu[l] = muc;
-    } else if (threadIdx.x >= 32 && threadIdx.x < 33 + NE_MAX_SPECIES_DEV) {
+    } else if (threadIdx.x < 33 + NE_MAX_SPECIES_DEV) {
         const int t = threadIdx.x - 32;
         const bool r1 = t == NE_MAX_SPECIES_DEV;  // the replica's single-species values
         const int ts = r1 ? 0 : t;
         if (r1 || t < P.nsp) {
-            s_tab[0][t] = (float)(r1 ? P.m : P.ms[ts]);
-            s_tab[1][t] = (float)(r1 ? P.k : P.ks[ts]);
-            s_tab[2][t] = (float)(r1 ? P.c2 : P.c2s[ts]);
-            s_tab[3][t] = (float)(r1 ? P.hdt_m : P.hdts[ts]);
+            s_tab[0][t] = (R)(r1 ? P.m : P.ms[ts]);
+            s_tab[1][t] = (R)(r1 ? P.k : P.ks[ts]);
+            s_tab[2][t] = (R)(r1 ? P.c2 : P.c2s[ts]);
+            s_tab[3][t] = (R)(r1 ? P.hdt_m : P.hdts[ts]);
         }
     }
+    // this component's state, while the shared values form
+    double x = 0.0, x0 = 0.0, vd = 0.0;
+    R F0 = 0, xi = 0;
+    int q = NE_MAX_SPECIES_DEV;
+    float pb = 0.f;
+    if (valid) {
+        x = B.x[e];
+        vd = B.v[e];
+        x0 = B.x0[e];
+        if (do_close || do_open) F0 = MIXED ? (R)((const float*)B.f32)[4 * (size_t)(P.off + a) + c] : (R)B.f64[e];
+        if (do_open) xi = MIXED ? (R)B.xi32[e] : (R)B.xi64[e];
+        if (P.nsp) q = P.sp[a];
+        pb = ((const float*)B.pbuild)[4 * (size_t)(P.off + a) + c];
+    }
     __syncthreads();
-    const double lam_s = s_lam[0], lam_n = s_lam[1];
-    const float ls = (float)lam_s, ln = (float)lam_n;
-    const bool draw = do_open || !do_close;  // a step follows: its normals
-    float part[NPB] = {};
+    const R ls = (R)s_lam[0], ln = (R)s_lam[1];
+    const R mi = s_tab[0][q], ki = s_tab[1][q], c2i = s_tab[2][q], hdti = s_tab[3][q];
+    R v = (R)vd, p_ke = 0, p_ux = 0, p_u2 = 0, p_xi = 0;
     int bad = 0;
     if (valid) {
-        double x[3];
-        float v[3], u[3], F0[3], mF0[3], mFE[3];
-        const float4 f = B.f32[i];
-        F0[0] = f.x;
-        F0[1] = f.y;
-        F0[2] = f.z;
-        for (int c = 0; c < 3; ++c) {
-            x[c] = B.x[3 * i + c];
-            v[c] = (float)B.v[3 * i + c];
-            u[c] = (float)(x[c] - B.x0[3 * i + c]);
-        }
-        const int q = P.nsp ? (int)P.sp[a] : NE_MAX_SPECIES_DEV;
-        const float mi = s_tab[0][q], ki = s_tab[1][q], c2i = s_tab[2][q], hdti = s_tab[3][q];
-        const float wm = P.nsp ? mi : 1.f;  // F_i -= m_i sum_j F_j / M with species tables
-        for (int c = 0; c < 3; ++c) {
-            mF0[c] = wm * s_mean[c];
-            mFE[c] = wm * s_mean[3 + c];
-        }
-        auto blendf = [&](float lam, float a0, float ae) { return S.path == 0 ? (1.f - lam) * a0 + lam * ae : lam * a0; };
-        if (do_close)
-            for (int c = 0; c < 3; ++c) v[c] += hdti * blendf(ls, F0[c] - mF0[c], -ki * u[c] - mFE[c]);
-        part[PB_KE] = 0.5f * mi * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        R u = (R)(x - x0);
+        // with species tables F_i -= m_i sum_j F_j / M
+        const R wm = P.nsp ? mi : (R)1;
+        const R f0 = F0 - wm * s_mean[c], fe = -ki * u - wm * s_mean[3 + c];
+        const auto blend = [&](R lam) { return S.path == 0 ? ((R)1 - lam) * f0 + lam * fe : lam * f0; };
+        if (do_close) v += hdti * blend(ls);
+        if (B.trace) p_ke = (R)0.5 * mi * v * v;
         if (do_open) {
-            for (int c = 0; c < 3; ++c) {
-                const float xi = B.xi32[3 * i + c];
-                const float dv = P.nsp ? c2i * xi - s_mean[6 + c] : c2i * (xi - s_mean[6 + c]);
-                v[c] += hdti * blendf(ln, F0[c] - mF0[c], -ki * u[c] - mFE[c]);
-                const float v1 = v[c];
-                v[c] = s_box[6] * v[c] + dv;
-                const float dx = 0.5f * (float)S.dt * (v1 + v[c]);
+            // velocity increments of the thermostat: c2 (xi - mean xi) for one
+            // species; c2_i xi_i - sum_j m_j c2_j xi_j / M with species tables
+            const R dv = P.nsp ? c2i * xi - s_mean[6 + c] : c2i * (xi - s_mean[6 + c]);
+            v += hdti * blend(ln);
+            const R v1 = v;
+            v = (MIXED ? (R)P.c1f : (R)P.c1) * v + dv;
+            if constexpr (MIXED) {
+                const float dx = S.hdtf * (v1 + v);
                 if (!isfinite(dx)) bad |= ST_ENAN;
-                x[c] += (double)dx;
+                x += (double)dx;
+            } else {
+                x = fma(0.5 * S.dt, v1, x);
+                x = fma(0.5 * S.dt, v, x);
             }
-            if (P.npt)
-                for (int c = 0; c < 3; ++c) x[c] *= s_mu[c];
+            if (P.npt) x *= s_mu[c];
             // from x itself, so that a run resumed from (x, v) forms the same totals
-            for (int c = 0; c < 3; ++c) u[c] = (float)(x[c] - B.x0[3 * i + c]);
+            u = (R)(x - x0);
+            B.x[e] = x;
         }
-        for (int c = 0; c < 3; ++c) {
-            if (!isfinite(v[c])) bad |= ST_ENAN;
-            B.x[3 * i + c] = x[c];
-            B.v[3 * i + c] = (double)v[c];
-            part[PB_UX + c] = P.nsp ? ki * u[c] : u[c];
-        }
-        part[PB_U2] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        part[PB_UE] = 0.5f * ki * part[PB_U2];
+        if (!isfinite(x) || !isfinite(v)) bad |= ST_ENAN;
+        if (do_close || do_open) B.v[e] = (double)v;
+        p_ux = P.nsp ? ki * u : u;
+        p_u2 = u * u;
         // x wrapped (image index in FP32, the shift, only for an atom outside
         // the box, in FP64), its image against the list build's and the
         // displacement from there
-        const float4 pb = B.pbuild[i];
-        const float pbx[3] = {pb.x, pb.y, pb.z};
-        float w[3], d2 = 0.f;
-        int code = 0;
-        for (int c = 0; c < 3; ++c) {
-            w[c] = (float)x[c];
-            const float n = floorf(w[c] * s_box[3 + c]);
-            if (n != 0.f) w[c] = (float)(x[c] - s_mu[c] * P.L[c] * (double)n);
-            const float nb = rintf((w[c] - pbx[c]) * s_box[3 + c]), d = fmaf(-s_box[c], nb, w[c] - pbx[c]);
-            code = 3 * code + (int)nb;
-            d2 = fmaf(d, d, d2);
+        float w = (float)x;
+        const float n = floorf(w * s_iLf[c]);
+        if constexpr (!MIXED) s_x64[c][al] = x;
+        if (n != 0.f) {
+            const double xw = x - s_L[c] * (double)n;
+            w = (float)xw;
+            if constexpr (!MIXED) s_x64[c][al] = xw;
         }
-        B.pos32[i] = make_float4(w[0], w[1], w[2], __int_as_float(code));
-        if (d2 > s_box[7]) B.flags[rep] = 1;
+        const float nb = rintf((w - pb) * s_iLf[c]), d = fmaf(-s_Lf[c], nb, w - pb);
+        s_w[c][al] = w;
+        s_d2[c][al] = d * d;
+        s_code[c][al] = (int)nb;
         if (draw) {
-            float z[3];
-            ne_normals32(ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
-                                         (unsigned long long)(do_open ? s + 1 : s)),
-                         z);
-            for (int c = 0; c < 3; ++c) {
-                B.xi32[3 * i + c] = z[c];
-                part[PB_XIX + c] = P.nsp ? mi * c2i * z[c] : z[c];
-            }
+            const uint4 ph = ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
+                                             (unsigned long long)(do_open ? s + 1 : s));
+            const R z = MIXED ? (R)ne_normal32(ph, c) : (R)ne_normal64(ph, c);
+            if constexpr (MIXED) B.xi32[e] = z;
+            else B.xi64[e] = z;
+            p_xi = P.nsp ? mi * c2i * z : z;
         }
     }
     if (bad) ne_set_status(B.status, bad);
-    if (do_open && valid && a == 0) step_work(B, S, T, rep, s, lam_s, lam_n);
-    // the tile's partials in double-float: a fixed tree in each warp, then
-    // the two warps in order
-    const int wp = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int q = 0; q < NPB; ++q) {
-        const dff t = dff_warp_sum({part[q], 0.f});
-        if (l == 0) s_w[q][wp] = make_float2(t.hi, t.lo);
+    if (do_open && threadIdx.x == STEP_THREADS - 32 && tile == P.tile0)
+        step_work(B, S, T, rep, s, s_lam[0], s_lam[1]);
+    // the tile's partials: UX.. and the normals per component, U2, U_E and KE
+    // over the components.  Mixed: double-float, a fixed tree in each warp, then
+    // the warps in order; FP64: rows of 64 in shared memory, eight threads a row
+    const R p_ue = P.nsp ? (R)0.5 * ki * p_u2 : (R)0;  // one species: U_E is k/2 times the sum of u^2
+    const int nq = P.nsp || B.trace ? 5 : 3;
+    const R pq[5] = {p_ux, p_u2, p_xi, p_ue, p_ke};
+    if constexpr (MIXED) {
+        const int wp = threadIdx.x >> 5;
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (k < nq) {
+                const dff t = dff_warp_sum({pq[k], 0.f});
+                if ((threadIdx.x & 31) == 0) s_dff[k][wp] = make_float2(t.hi, t.lo);
+            }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (k < nq) s_red[k][c][al] = pq[k];
     }
     __syncthreads();
-    if (threadIdx.x < NPB) {
-        dff t = {0.f, 0.f};
-        for (int w2 = 0; w2 < NE_TILE / 32; ++w2) t = dff_add(t, {s_w[threadIdx.x][w2].x, s_w[threadIdx.x][w2].y});
-        B.partB[(size_t)threadIdx.x * B.n_tiles + tile] = (double)t.hi + (double)t.lo;
+    double* const pbt = B.partB + tile;
+    const size_t np = B.n_tiles;
+    if constexpr (MIXED) {
+        if (threadIdx.x < 15 && threadIdx.x / 3 < nq) {
+            const int k = threadIdx.x / 3, d = threadIdx.x % 3;
+            dff t = dff_add({s_dff[k][2 * d].x, s_dff[k][2 * d].y}, {s_dff[k][2 * d + 1].x, s_dff[k][2 * d + 1].y});
+            if (k == 0 || k == 2) {
+                pbt[((k == 0 ? PB_UX : PB_XIX) + d) * np] = (double)t.hi + (double)t.lo;
+            } else if (d == 0 && (k != 3 || P.nsp)) {
+                for (int w2 = 2; w2 < 6; ++w2) t = dff_add(t, {s_dff[k][w2].x, s_dff[k][w2].y});
+                const double tot = (double)t.hi + (double)t.lo;
+                pbt[(k == 1 ? PB_U2 : (k == 3 ? PB_UE : PB_KE)) * np] = tot;
+                if (k == 1 && !P.nsp) pbt[PB_UE * np] = 0.5 * P.k * tot;
+            }
+        }
+    } else if (threadIdx.x < 128) {
+        const int row = threadIdx.x >> 3, sg = threadIdx.x & 7, k = row / 3, d = row % 3;
+        const bool on = k < nq;
+        const double* r = s_red[on ? k : 0][d] + sg * 8;
+        double t = r[0];
+#pragma unroll
+        for (int z = 1; z < 8; ++z) t += r[z];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (on && sg == 0) {
+            if (k == 0 || k == 2) pbt[((k == 0 ? PB_UX : PB_XIX) + d) * np] = t;
+            else s_red[k][d][NE_TILE] = t;  // the pad column
+        }
+    }
+    // the atom's copies for the pair passes, from its three components
+    if (threadIdx.x < NE_TILE && valid) {
+        const int i = P.off + a;
+        B.pos32[i] = make_float4(s_w[0][al], s_w[1][al], s_w[2][al],
+                                 __int_as_float(9 * s_code[0][al] + 3 * s_code[1][al] + s_code[2][al]));
+        if constexpr (!MIXED) B.pos64[i] = ned4{s_x64[0][al], s_x64[1][al], s_x64[2][al], 0.0};
+        if (s_d2[0][al] + s_d2[1][al] + s_d2[2][al] > P.half_skin2) B.flags[rep] = 1;
+    }
+    if constexpr (!MIXED) {
+        __syncthreads();
+        // U2; U_E with species tables; KE with a trace
+        if (threadIdx.x == 0 || (threadIdx.x == 1 && P.nsp) || (threadIdx.x == 2 && nq == 5)) {
+            const int k = threadIdx.x == 0 ? 1 : 2 + threadIdx.x;
+            const double t = s_red[k][0][NE_TILE] + s_red[k][1][NE_TILE] + s_red[k][2][NE_TILE];
+            pbt[(k == 1 ? PB_U2 : (k == 3 ? PB_UE : PB_KE)) * np] = t;
+            if (k == 1 && !P.nsp) pbt[PB_UE * np] = 0.5 * P.k * t;
+        }
+    }
+    // the box of a barostatted replica, by its last block (every block has
+    // read the box).  A box whose cells became shorter than r_c + skin, or whose
+    // edge fell below 2 (r_c + skin), is reported (NE_ERANGE) and left unchanged.
+    if (do_open && P.npt && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&B.tile_done[rep], 1u) == (unsigned)P.ntile - 1u) {
+            __threadfence();
+            B.tile_done[rep] = 0u;
+            RepDev& Pw = const_cast<RepDev*>(B.rep)[rep];
+            const double rl = sqrt(P.rlist2);
+            bool ok = true;
+            for (int d = 0; d < 3; ++d)
+                ok = ok && s_L[d] > 2.0 * rl && (P.nc[d] == 0 || s_L[d] / P.nc[d] >= rl);
+            if (!ok) ne_set_status(B.status, ST_ERANGE);
+            else
+                for (int d = 0; d < 3; ++d) {
+                    Pw.L[d] = s_L[d];
+                    Pw.invL[d] = 1.0 / s_L[d];
+                    Pw.Lf[d] = (float)Pw.L[d];
+                    Pw.iLf[d] = (float)Pw.invL[d];
+                }
+        }
     }
 }
 
@@ -415,35 +362,6 @@ __global__ void k_trace_T(DevBatch B, const long long* __restrict__ step_base, i
 }
 
 __global__ void k_advance(long long* step_base, long long by) { *step_base += by; }
-
-// Box of every barostatted replica after the step kernel of step s (same
-// scale factor as that kernel).  A box whose cells became shorter than
-// r_c + skin, or whose edge fell below 2 (r_c + skin), is reported
-// (NE_ERANGE) and left unchanged.
-__global__ void k_npt_box(DevBatch B, Sched S, const long long* __restrict__ step_base, int j)
-{
-    const int rep = blockIdx.x;
-    if (rep >= B.n_rep || threadIdx.x != 0) return;
-    RepDev& P = const_cast<RepDev*>(B.rep)[rep];
-    if (!P.npt) return;
-    const long long s = *step_base + j;
-    double mu[3];
-    npt_scale(P, B.tot + (size_t)rep * NTOT, ne_sched_lambda(S, s + 1), s, S.dt, mu);
-    const double rl = sqrt(P.rlist2);
-    for (int c = 0; c < 3; ++c) {
-        const double L = mu[c] * P.L[c];
-        if (!(L > 2.0 * rl) || (P.nc[c] > 0 && !(L / P.nc[c] >= rl))) {
-            ne_set_status(B.status, ST_ERANGE);
-            return;
-        }
-    }
-    for (int c = 0; c < 3; ++c) {
-        P.L[c] *= mu[c];
-        P.invL[c] = 1.0 / P.L[c];
-        P.Lf[c] = (float)P.L[c];
-        P.iLf[c] = (float)P.invL[c];
-    }
-}
 
 __global__ void k_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n,
                         int mixed, double* z)
@@ -667,24 +585,10 @@ void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long*
                  int do_close, int do_open, cudaStream_t st)
 {
     if (mixed)
-        k_step_mixed<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, j, do_close, do_open);
+        k_step<true><<<B.n_tiles, STEP_THREADS, 0, st>>>(B, S, step_base, j, do_close, do_open);
     else
-        k_step<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, j, do_close, do_open);
-    if (B.trace) k_trace_T<<<1, 32, 0, st>>>(B, step_base, j);
-}
-
-void launch_prep(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
-                 cudaStream_t st)
-{
-    if (mixed)
-        k_step_mixed<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, 0, 0, 0);
-    else
-        k_step<<<B.n_tiles, NE_TILE, 0, st>>>(B, S, step_base, 0, 0, 0);
-}
-
-void launch_npt_box(const DevBatch& B, const Sched& S, const long long* step_base, int j, cudaStream_t st)
-{
-    k_npt_box<<<B.n_rep, 32, 0, st>>>(B, S, step_base, j);
+        k_step<false><<<B.n_tiles, STEP_THREADS, 0, st>>>(B, S, step_base, j, do_close, do_open);
+    if (B.trace && do_open) k_trace_T<<<1, 32, 0, st>>>(B, step_base, j);
 }
 
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,
