@@ -737,7 +737,7 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
         if (ctx->gev[g]) cudaEventDestroy(ctx->gev[g]);
     for (int g = 0; g < 2; ++g)
         if (ctx->ev_run[g]) cudaEventDestroy(ctx->ev_run[g]);
-    void* bptrs[] = {ctx->bb.u4, ctx->bb.fp, ctx->bb.part, ctx->bb.vir, ctx->bb.bar, ctx->bb.abortf, ctx->cta_rep,
+    void* bptrs[] = {ctx->bb.u4, ctx->bb.part, ctx->bb.vir, ctx->bb.bar, ctx->bb.abortf, ctx->cta_rep,
                      ctx->cr_boxes};
     for (void* p : bptrs)
         if (p) cudaFree(p);
@@ -1562,7 +1562,10 @@ static ne_status build_plan(ne_ctx* ctx, const ne_md_params* md, const ne_crysta
             const size_t base = (ne::brick_smem_bytes(tpa, gnb, glut, P.npt) + 15) & ~(size_t)15;
             if (base > (size_t)smem_max) continue;
             const long long fit = ((long long)smem_max - (long long)base) / (2 * (long long)sizeof(float4));
-            const int n_int = (int)std::min<long long>(nk - 1, fit);
+            // intervals from 1 A up (shorter pairs read the global table): what
+            // shared memory does not take is L1 for the neighbours' u
+            const long long from1 = (long long)std::ceil((nk - 1) * (1.0 - 1.0 / std::max(rc, 1.0)));
+            const int n_int = (int)std::min<long long>(std::max<long long>(from1, 1), fit);
             const size_t smem = std::max(base + (size_t)n_int * 2 * sizeof(float4), smem_floor);
             if (smem > (size_t)smem_max) continue;
             const int per = ne::brick_atoms_per_cta(tpa);
@@ -1596,8 +1599,7 @@ static ne_status build_plan(ne_ctx* ctx, const ne_md_params* md, const ne_crysta
         if (!ctx->bb.u4) {
             const size_t N = (size_t)ctx->max_atoms;
             NE_CU(cudaMalloc((void**)&ctx->bb.u4, sizeof(float4) * 2 * N));
-            NE_CU(cudaMalloc((void**)&ctx->bb.fp, sizeof(float) * N));
-            NE_CU(cudaMalloc((void**)&ctx->bb.bar, sizeof(unsigned) * 2));
+            NE_CU(cudaMalloc((void**)&ctx->bb.bar, sizeof(unsigned) * NE_BAR_STRIDE * (size_t)ctx->max_rep));
             NE_CU(cudaMalloc((void**)&ctx->bb.abortf, sizeof(int)));
         }
         if (P.n_cta > ctx->bb_ctas) {
@@ -1776,7 +1778,7 @@ static ne_status crystal_segment_impl(ne_ctx* ctx, const ne_md_params* md, const
             for (const XRep& X : P.xs) t = std::max<long long>(t, (long long)X.off + X.n);
             return t;
         }();
-        NE_CU(ne::launch_brick(P.tpa, ctx->xrep, ctx->cta_rep, P.n_cta, P.smem, ctx->st_vec, ctx->st_dist, x_dev,
+        NE_CU(ne::launch_brick(P.tpa, ctx->xrep, n_rep, ctx->cta_rep, P.n_cta, P.smem, ctx->st_vec, ctx->st_dist, x_dev,
                                v_dev, W_dev, ctx->status, S, step_begin, n_steps, ctx->tab, ctx->work, P.k_lo,
                                ctx->lam_tab + step_begin, Wcum_dev, ctx->bb, n_tot, st, P.npt, ctx->cr_boxes));
         ++ctx->cr_launches;

@@ -3,7 +3,7 @@
 // every CTA owns a block of consecutive cells of one replica and the CTAs of
 // a replica exchange what the cluster runner keeps in distributed shared
 // memory -- the displacements u_j = x_j - r0_j and F'(rho_j) -- through global
-// memory (L2) between grid barriers.
+// memory (L2) between barriers of the replica's CTAs.
 //
 // The arithmetic of a step is that of the cluster runner (ne_cluster.cu):
 // the same lattice stencil and scan bound, rho as a double-float, positions
@@ -12,24 +12,32 @@
 // rounding of its replica sums (which depend on how the atoms are split over
 // CTAs).  Per step:
 //   replica sums of step s from the CTA partials written at the end of s-1
-//   pass 1: rho, pair forces and energy, f'(r)/r of every visit to tensor memory (u_j from L2);
-//           F'(rho) of the owned atoms to global memory
-//   [grid barrier]
-//   pass 2: embedding forces over the visits inside r_c (u_j, F'_j from L2)
+//   pass 1: rho, pair forces and energy, f'(r)/r of every visit to tensor memory;
+//           F'(rho) of the owned atoms beside their u
+//   [barrier of the replica's CTAs]
+//   pass 2: embedding forces over the visits inside r_c
 //   fused step of the owned atoms; u of step s+1 to the other parity buffer;
 //           CTA partials for step s+1
-//   [grid barrier]
-// Two grid barriers a step; u is double-buffered by step parity, so no CTA
+//   [barrier of the replica's CTAs]
+// Two barriers a step; u is double-buffered by step parity, so no CTA
 // overwrites a u another still reads.  With the barostat (reading A23, the
 // cluster runner's arithmetic) pass 2 also sums the diagonal virial; the
-// CTA sums go to global memory behind a third grid barrier, after which
-// every CTA of the replica forms the same scale factors (the same sums in
-// the same order, the same Philox normal) before its integration.  The barrier is an arrival counter and
-// a generation word in global memory; every CTA of the launch is resident at
-// once (cooperative launch), and every wait is bounded: after BAR_SPIN_LIMIT
-// polls a CTA records NE_ETIMEOUT, raises the abort word and leaves, and the
-// others leave at their next barrier.  Loads of data other CTAs wrote use
-// ld.global.cg (L2, never a stale L1 line).
+// CTA sums go to global memory behind a third barrier, after which every CTA of
+// the replica forms the same scale factors (the same sums in the same order,
+// the same Philox normal) before its integration.  A barrier is an arrival count
+// in global memory; every CTA of the launch is resident at once (cooperative
+// launch), and every wait is bounded: after BAR_SPIN_LIMIT polls a CTA records
+// NE_ETIMEOUT, raises the abort word and leaves, and the others leave at the
+// barrier they wait at.
+//
+// The neighbours' (u, F') are plain loads through L1: a barrier's acquire orders
+// them after the other CTAs' writes (and drops the SM's L1 lines), and a CTA's
+// atoms share most of their ~2000 neighbours, so all but the first read of each
+// hit L1.  The spline window in shared memory starts at 1 A, which leaves L1
+// room for them.  Four bcc 16^3, a step: 29.4 us with every neighbour from L2
+// (long-scoreboard and barrier stalls 5.2 and 5.1 an issue), u and F' apart and
+// barriers of the whole launch; 23.7 us now (2.7 and 3.8).  bcc 32^3: 69.7 and
+// 59.4 us.
 //
 // Threads: TPA threads per atom (8, 4, 3, 2 or 1, the largest at which the
 // batch's CTAs fit the device at one CTA per SM); thread t works on slot
@@ -63,7 +71,7 @@ constexpr int NSV = 2 * ND_ + NF_;  // floats of the sums: (hi, lo) per energy, 
 constexpr int NPART = NSV + 1;      // and max |u|
 constexpr int T_UX = 2 * ND_ + (P_UX - ND_), T_XX = 2 * ND_ + (P_XX - ND_);
 constexpr int NRED = (int)NP_ + 1;
-constexpr unsigned BAR_SPIN_LIMIT = 1u << 22;  // polls, each >= 64 ns: a few seconds at most
+constexpr unsigned BAR_SPIN_LIMIT = 1u << 22;  // polls, each an L2 round trip: a few seconds at most
 constexpr double XSCALE = 4294967296.0;        // fixed point: 2^32 per Angstrom
 
 struct dfl {
@@ -103,35 +111,33 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
     return v;
 }
 
-// Barrier over every CTA of the launch.  Returns false when a wait gave up
-// (here or, through the abort word, in another CTA): the caller leaves.
-__device__ bool grid_barrier(unsigned* bar, unsigned n_cta, unsigned& gen, int* status, int* abortf, int* s_flag)
+// Barrier over the CTAs of one replica (n of them): every CTA adds one to the
+// replica's word and waits until all n have for this time round (target; the
+// difference is taken modulo 2^32).  One release and the polls, no reset; a
+// barrier over the whole launch, with a reset and a generation word, cost every
+// replica the slowest one's time and two more L2 round trips.  Returns false
+// when a wait gave up, here or, as the abort word says, in another CTA: the
+// caller leaves.
+__device__ bool replica_barrier(unsigned* bar, unsigned n, unsigned& target, int* status, int widx, int* abortf,
+                                int* s_flag)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
+        target += n;
         __threadfence();  // this CTA's global writes before its arrival
-        const unsigned g = gen;
-        if (atomicAdd(&bar[0], 1u) == n_cta - 1) {
-            atomicExch(&bar[0], 0u);
-            __threadfence();
-            atomicExch(&bar[1], g + 1u);
-        } else {
-            unsigned spins = 0;
-            while (ld_acquire(&bar[1]) == g) {
-                if (++spins > BAR_SPIN_LIMIT || ld_acquire((const unsigned*)abortf) != 0u) {
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        unsigned spins = 0;
+        while ((int)(ld_acquire(bar) - target) < 0) {
+            ++spins;
+            if (spins > BAR_SPIN_LIMIT || ((spins & 63u) == 0u && ld_acquire((const unsigned*)abortf) != 0u)) {
+                ok = 0;
+                ne_set_status(status, ST_ETIMEOUT);
+                ne_set_status(status + 1 + widx, ST_ETIMEOUT);
+                atomicExch(abortf, 1);
+                break;
             }
         }
-        if (!ok || ld_acquire((const unsigned*)abortf) != 0u) {
-            ok = 0;
-            ne_set_status(status, ST_ETIMEOUT);
-            atomicExch(abortf, 1);
-        }
-        gen = g + 1u;
         __threadfence();
         *s_flag = ok;
     }
@@ -167,6 +173,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     const XRep& R_ = reps[rep];
     const int C = R_.ncta, rank = (int)blockIdx.x - R_.cta0;
     const unsigned n_cta = gridDim.x;
+    unsigned* const bar = bb.bar + (size_t)R_.widx * NE_BAR_STRIDE;
     const int n = R_.n, nb = R_.nb, nx = R_.nx, ny = R_.ny, nz = R_.nz;
     const int nst = R_.st_cnt, M = R_.st_margin;
     const int A_c = brick_cta_atoms(n, C, nb);
@@ -384,8 +391,8 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         }
         cta_partials(pd, pf, um, (int)(s_begin & 1));
     }
-    unsigned gen = 0;
-    bool alive = grid_barrier(bb.bar, n_cta, gen, status, bb.abortf, s_flag);
+    unsigned target = 0;
+    bool alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);
 
     unsigned n_cand = 0, n_pair = 0;
     const float rc2 = tab.rc2f, rmin2 = tab.rmin2f, inv_h = tab.inv_h_rf;
@@ -464,7 +471,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         }
 
         // ---- pass 1: density, pair forces and energy, f'(r)/r of every visit to TMEM
-        const float4 ui = dead ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcg(&u_cur[sui]);
+        const float4 ui = dead ? make_float4(0.f, 0.f, 0.f, 0.f) : u_cur[sui];
         int m = 0, nq = 0;  // pairs inside r_c; the warp's visits
         float fx = 0.f, fy = 0.f, fz = 0.f, ep = 0.f;
         float vxx = 0.f, vyy = 0.f, vzz = 0.f;  // diagonal virial (barostat only)
@@ -486,7 +493,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             // f'(r)/r inside r_c, else 0
             auto visit = [&](float4 e, int j, int qv) -> float {
                 float fr = 0.f;
-                const float4 uj = __ldcg(&u_cur[j]);
+                const float4 uj = u_cur[j];
                 if constexpr (NPT) {
                     e.x *= muf[0];
                     e.y *= muf[1];
@@ -599,16 +606,15 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             const float4 c = __ldg(&tab.F32[kk]);
             emb = c.x + w * (c.y + w * (c.z + w * c.w));
             const float dF = (c.y + w * (2.f * c.z + 3.f * w * c.w)) * tab.inv_h_rhof;
-            bb.fp[gofs + tsu] = dF;
+            ((float*)&u_cur[tsu])[3] = dF;
             if (!isfinite(emb)) bad |= ST_ENAN;
         }
-        alive = grid_barrier(bb.bar, n_cta, gen, status, bb.abortf, s_flag);  // F' visible everywhere
+        alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // F' visible everywhere
         if (!alive) break;
 
         // ---- pass 2: embedding forces over the visits of pass 1, f'(r)/r from TMEM
         if (!dead) {
-            const float dFi = __ldcg(&bb.fp[gofs + sui]);
-            const float* fp_r = bb.fp + gofs;
+            const float dFi = u_cur[sui].w;
             const int nqt = min(nq, QF);
 #pragma unroll 1
             for (int q0 = 0; q0 < nqt; q0 += FRB) {
@@ -625,15 +631,14 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                         float4 e = s_sv[stb + k];
                         const int code = __float_as_int(e.w);
                         const int j = s_lxy[sxy + (code & 0xffff)] + s_lz[sz + ((unsigned)code >> 16)];
-                        const float4 uj = __ldcg(&u_cur[j]);
-                        const float dFj = __ldcg(&fp_r[j]);
+                        const float4 uj = u_cur[j];
                         if constexpr (NPT) {
                             e.x *= muf[0];
                             e.y *= muf[1];
                             e.z *= muf[2];
                         }
                         const float dx = e.x + uj.x - ui.x, dy = e.y + uj.y - ui.y, dz = e.z + uj.z - ui.z;
-                        const float sc = (dFi + dFj) * frv[uq];
+                        const float sc = (dFi + uj.w) * frv[uq];
                         fx += sc * dx;
                         fy += sc * dy;
                         fz += sc * dz;
@@ -651,7 +656,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                 float4 e = s_sv[stb + k];
                 const int code = __float_as_int(e.w);
                 const int j = s_lxy[sxy + (code & 0xffff)] + s_lz[sz + ((unsigned)code >> 16)];
-                const float4 uj = __ldcg(&u_cur[j]);
+                const float4 uj = u_cur[j];
                 if constexpr (NPT) {
                     e.x *= muf[0];
                     e.y *= muf[1];
@@ -660,13 +665,12 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                 const float dx = e.x + uj.x - ui.x, dy = e.y + uj.y - ui.y, dz = e.z + uj.z - ui.z;
                 const float r2 = dx * dx + dy * dy + dz * dz;
                 if (!(r2 < rc2)) continue;
-                const float dFj = __ldcg(&fp_r[j]);
                 const float irh = rsqrtf(r2) * inv_h;
                 const float t = r2 * irh;
                 const int kk = min((int)t, nk - 2);
                 const float w = t - (float)kk;
                 const float4 g = kk >= k_lo ? s_tabF[kk - k_lo] : __ldg(&tab.pf32[2 * kk + 1]);
-                const float sc = (dFi + dFj) * ((g.y + w * (2.f * g.z + 3.f * w * g.w)) * irh);
+                const float sc = (dFi + uj.w) * ((g.y + w * (2.f * g.z + 3.f * w * g.w)) * irh);
                 fx += sc * dx;
                 fy += sc * dy;
                 fz += sc * dz;
@@ -722,7 +726,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                             bb.vir[(size_t)blockIdx.x * 6 + 2 * a3 + 1] = t[a3].lo;
                         }
                 }
-                alive = grid_barrier(bb.bar, n_cta, gen, status, bb.abortf, s_flag);  // virials visible
+                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // virials visible
                 if (!alive) break;
                 if (w == 0) {
                     dfl t[3] = {};
@@ -848,7 +852,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             }
             if (!fin) {
                 cta_partials(pd, pf, dead ? 1e30f : un, p ^ 1);
-                alive = grid_barrier(bb.bar, n_cta, gen, status, bb.abortf, s_flag);  // u of s + 1 visible
+                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // u of s + 1 visible
             }
         }
     }
@@ -867,12 +871,12 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             atomicAdd(&work[1], (unsigned long long)n_pair);
         }
     }
-    if (!alive) return;  // a wait gave up: the call reports NE_ETIMEOUT and writes nothing back
+    if (!alive) return;  // a wait gave up: the call reports NE_ETIMEOUT
     // every CTA's error bits for its replica are in the status word after
     // this barrier; a replica that raised none writes its state back
-    alive = grid_barrier(bb.bar, n_cta, gen, status, bb.abortf, s_flag);
+    alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);
     if (!alive) return;
-    if (threadIdx.x == 0) s_flag[1] = atomicOr(status + 1 + R_.widx, 0);
+    if (threadIdx.x == 0) s_flag[1] = atomicOr(status + 1 + R_.widx, 0) | (int)ld_acquire((const unsigned*)bb.abortf);
     __syncthreads();
     if (s_flag[1] == 0) {
         if (own)
@@ -967,14 +971,14 @@ int brick_max_ctas(int tpa, size_t smem, bool npt)
     return per * sms;
 }
 
-cudaError_t launch_brick(int tpa, const XRep* reps, const int* cta_rep, int n_cta, size_t smem, const float4* st_vec,
+cudaError_t launch_brick(int tpa, const XRep* reps, int n_rep, const int* cta_rep, int n_cta, size_t smem, const float4* st_vec,
                          const float* st_dist, double* x, double* v, double* W, int* status, const Sched& S,
                          long long s_begin, long long n_steps, const Tables& tab, unsigned long long* work,
                          int k_lo, const double* lam_tab, double* wcum, const BrickBufs& bb, long long n_tot,
                          cudaStream_t st, bool npt, double* boxes_out)
 {
     if (npt && !bb.vir) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(bb.bar, 0, 2 * sizeof(unsigned), st);
+    cudaError_t e = cudaMemsetAsync(bb.bar, 0, sizeof(unsigned) * NE_BAR_STRIDE * (size_t)n_rep, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(bb.abortf, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -983,7 +987,7 @@ cudaError_t launch_brick(int tpa, const XRep* reps, const int* cta_rep, int n_ct
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;  // every CTA resident at once: the grid barrier needs it
+    attr[0].id = cudaLaunchAttributeCooperative;  // every CTA resident at once: the barriers need it
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
