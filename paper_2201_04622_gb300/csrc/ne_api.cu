@@ -1361,6 +1361,9 @@ static bool same_sched(const Sched& a, const Sched& b)
            a.fn == b.fn && a.stream == b.stream && a.fix_cm == b.fix_cm;
 }
 
+// SMs that a brick launch leaves free where its atoms do not need them
+constexpr int BRICK_FREE_SMS = 8;
+
 // Build the launch plan of a batch (stencils, replica table, cluster size,
 // size classes and their shared memory) and upload its device part.  Runs
 // on a call whose key differs from the cached plan's; later calls with the
@@ -1579,6 +1582,23 @@ static ne_status build_plan(ne_ctx* ctx, const ne_md_params* md, const ne_crysta
             }
             const int cap = ne::brick_max_ctas(tpa, smem, P.npt);
             if (total > cap) continue;
+            // where a quarter of the SMs or more would stay idle: more CTAs than
+            // the atoms need, down to 32 atoms each, while one more makes the
+            // fullest replica's CTAs smaller (a step is as long as its fullest
+            // SM).  A few SMs stay free for another stream's kernels
+            // (a replica on the multi-kernel path alongside)
+            auto cta_atoms = [&](int r, int C) { return (((xr[r].n + C - 1) / C) + xr[r].nb - 1) / xr[r].nb * xr[r].nb; };
+            const bool spread = 4 * total <= 3 * cap;
+            while (spread && total < cap - BRICK_FREE_SMS) {
+                int big = 0;
+                for (int r = 1; r < n_rep; ++r)
+                    if (cta_atoms(r, cr_[r]) > cta_atoms(big, cr_[big])) big = r;
+                int C = cr_[big] + 1;
+                while (total - cr_[big] + C <= cap - BRICK_FREE_SMS && cta_atoms(big, C) == cta_atoms(big, cr_[big])) ++C;
+                if (total - cr_[big] + C > cap - BRICK_FREE_SMS || cta_atoms(big, C) < 32) break;
+                total += C - cr_[big];
+                cr_[big] = C;
+            }
             P.brick = true;
             P.tpa = tpa;
             P.n_cta = total;
