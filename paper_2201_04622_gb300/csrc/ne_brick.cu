@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     float* s_red = (float*)(s_rho + (TPA - 1) * SLOTS);           // [NWARP][NRED][2]
     int* s_flag = (int*)(s_red + NWARP * NRED * 2);               // [4]
     unsigned* s_tm = (unsigned*)(s_flag + 4);                     // [4] TMEM base address
-    unsigned char* s_end = (unsigned char*)(s_tm + 4);
+    double* s_work = (double*)(s_tm + 4);                         // [4] the work thread's W and U_E
+    unsigned char* s_end = (unsigned char*)(s_work + 4);
     float4* s_vir = nullptr;  // barostat: [TPA - 1][SLOTS] pair-lane virials
     float* s_vred = nullptr;  // [NWARP][6] warp sums of the virial
     double* s_mu = nullptr;   // [3] the step's scale factors
@@ -402,12 +403,10 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     const float rho_maxf = (float)tab.rho_max;
     const float ihr_hi = (float)tab.inv_h_rho, ihr_lo = (float)(tab.inv_h_rho - (double)ihr_hi);
     const bool wthread = rank == 0 && threadIdx.x == BTHREADS - 1;
-    double Wacc[2] = {0.0, 0.0};
     if (wthread) {
-        Wacc[0] = Wg[2 * R_.widx];
-        Wacc[1] = Wg[2 * R_.widx + 1];
+        s_work[0] = Wg[2 * R_.widx];
+        s_work[1] = Wg[2 * R_.widx + 1];
     }
-    double UE_prev = 0.0;
     bool dead = false;  // the replica left the stencil range: its CTAs keep to the barriers only
     // barostat: the box and the sites scale by mu_tot per axis from the
     // call's start (the same values in every CTA of the replica); stencil
@@ -772,21 +771,21 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             const double U0 = (double)s_tot[2 * P_U0] + (double)s_tot[2 * P_U0 + 1];
             if (it > 0) {
                 const long long sp = s - 1;
-                const double gw = S.path == 0 ? U0 - UE_prev : U0;
+                const double gw = S.path == 0 ? U0 - s_work[2] : U0;
                 int wslot = -1;
                 if (sp >= S.t_eq && sp < S.t_eq + S.t_s) wslot = 0;
                 else if (sp >= 2 * S.t_eq + S.t_s && sp < 2 * S.t_eq + 2 * S.t_s) wslot = 1;
                 if (wslot >= 0) {
-                    Wacc[wslot] += (lam_tab[it] - lam_tab[it - 1]) * gw;
+                    s_work[wslot] += (lam_tab[it] - lam_tab[it - 1]) * gw;
                     if (wcum) {
                         const long long k = wslot == 0 ? sp - S.t_eq : sp - (2 * S.t_eq + S.t_s);
                         double* wc = wcum + (size_t)(2 * R_.widx + wslot) * (size_t)(S.t_s + 1);
                         if (k == 0) wc[0] = 0.0;
-                        wc[k + 1] = Wacc[wslot];
+                        wc[k + 1] = s_work[wslot];
                     }
                 }
             }
-            UE_prev = (double)s_tot[2 * P_UE] + (double)s_tot[2 * P_UE + 1];
+            s_work[2] = (double)s_tot[2 * P_UE] + (double)s_tot[2 * P_UE + 1];
         }
         {
             dfl pd[ND_] = {};
@@ -887,8 +886,8 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                 vg[gi + c] = (double)v[c];
             }
         if (wthread) {
-            Wg[2 * R_.widx] = Wacc[0];
-            Wg[2 * R_.widx + 1] = Wacc[1];
+            Wg[2 * R_.widx] = s_work[0];
+            Wg[2 * R_.widx + 1] = s_work[1];
             if (NPT && boxes_out)
                 for (int c = 0; c < 3; ++c) boxes_out[3 * R_.widx + c] = mu_tot[c] * R_.box0[c];
         }
@@ -936,7 +935,7 @@ size_t brick_smem_bytes(int tpa, int nb_nst_max, int lut_max, bool npt)
     b += sizeof(float) * NSV;
     b = (b + 15) & ~(size_t)15;
     b += (sizeof(float4) + sizeof(float2)) * (size_t)(tpa - 1) * slots + sizeof(float) * NWARP * NRED * 2 +
-         sizeof(int) * 4 + sizeof(unsigned) * 4;
+         sizeof(int) * 4 + sizeof(unsigned) * 4 + sizeof(double) * 4;
     if (npt) {  // pair-lane virials, warp sums, scale factors
         b = (b + 15) & ~(size_t)15;
         b += sizeof(float4) * (size_t)(tpa - 1) * slots + sizeof(float) * NWARP * 6;

@@ -253,10 +253,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     float* s_slotM = (float*)(s_rho + SLOTS);                     // [2][16] max |u| per CTA
     float* s_red = s_slotM + 32;                                  // [NWARP][NRED][2]
     unsigned* s_tm = (unsigned*)(s_red + NWARP * NRED * 2);       // [4] TMEM base address
+    double* s_work = (double*)(s_tm + 4);                         // [4] the work thread's W and U_E
     // barostat: the diagonal virial of the second pair lane of each slot, the
     // warps' double-float partials, every CTA's partial (written by the CTA
     // into all CTAs of the cluster) and the step's scale factors
-    float4* s_vir = (float4*)(((size_t)(s_tm + 4) + 15) & ~(size_t)15);  // [SLOTS] (NPT)
+    float4* s_vir = (float4*)(((size_t)(s_work + 4) + 15) & ~(size_t)15);  // [SLOTS] (NPT)
     float* s_vred = (float*)(s_vir + (NPT ? SLOTS : 0));          // [NWARP][6] (NPT)
     float* s_vcta = s_vred + (NPT ? NWARP * 6 : 0);               // [16][6] (NPT)
     double* s_mu = (double*)(((size_t)(s_vcta + (NPT ? 16 * 6 : 0)) + 7) & ~(size_t)7);  // [4] (NPT)
@@ -437,17 +438,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     const float dt = (float)S.dt;
     const float rho_maxf = (float)tab.rho_max;
     const float ihr_hi = (float)tab.inv_h_rho, ihr_lo = (float)(tab.inv_h_rho - (double)ihr_hi);
-    // rank 0, thread SLOTS (owns no atom) keeps the replica's two works in
-    // registers and writes them back at the end, only if the replica
-    // completed the range; likewise x and v below, so a replica that raised
+    // rank 0, thread SLOTS (owns no atom) keeps the replica's two works and
+    // U_E at the positions of the previous step in shared memory (registers
+    // would cost every thread six) and writes the works back at the end, only
+    // if the replica completed the range; likewise x and v below, so a replica that raised
     // an error keeps its state of step s_begin and can be rerun from there
     const bool wthread = rank == 0 && threadIdx.x == SLOTS;
-    double Wacc[2] = {0.0, 0.0};
     if (wthread) {
-        Wacc[0] = Wg[2 * reps[rep].widx];
-        Wacc[1] = Wg[2 * reps[rep].widx + 1];
+        s_work[0] = Wg[2 * reps[rep].widx];
+        s_work[1] = Wg[2 * reps[rep].widx + 1];
     }
-    double UE_prev = 0.0;  // the work thread: U_E at the positions of the previous step
     // barostat: the box and the lattice sites scale by mu_tot per axis from
     // the call's start (every thread holds the same values: they come from
     // the same sums); stencil vectors are multiplied by it
@@ -778,21 +778,21 @@ __global__ void __launch_bounds__(THREADS, 1)
             const double U0 = (double)s_tot[2 * P_U0] + (double)s_tot[2 * P_U0 + 1];
             if (it > 0) {
                 const long long sp = s - 1;
-                const double g = S.path == 0 ? U0 - UE_prev : U0;
+                const double g = S.path == 0 ? U0 - s_work[2] : U0;
                 int wslot = -1;
                 if (sp >= S.t_eq && sp < S.t_eq + S.t_s) wslot = 0;
                 else if (sp >= 2 * S.t_eq + S.t_s && sp < 2 * S.t_eq + 2 * S.t_s) wslot = 1;
                 if (wslot >= 0) {
-                    Wacc[wslot] += (lam_tab[it] - lam_tab[it - 1]) * g;
+                    s_work[wslot] += (lam_tab[it] - lam_tab[it - 1]) * g;
                     if (wcum) {  // cumulative work of the switch: [0] = 0, [k + 1] after its step k
                         const long long k = wslot == 0 ? sp - S.t_eq : sp - (2 * S.t_eq + S.t_s);
                         double* wc = wcum + (size_t)(2 * reps[rep].widx + wslot) * (size_t)(S.t_s + 1);
                         if (k == 0) wc[0] = 0.0;
-                        wc[k + 1] = Wacc[wslot];
+                        wc[k + 1] = s_work[wslot];
                     }
                 }
             }
-            UE_prev = (double)s_tot[2 * P_UE] + (double)s_tot[2 * P_UE + 1];
+            s_work[2] = (double)s_tot[2 * P_UE] + (double)s_tot[2 * P_UE + 1];
         }
         {
             dfl pd[ND_] = {};
@@ -938,8 +938,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 vg[gi + c] = (double)v[c];
             }
         if (wthread) {
-            Wg[2 * reps[rep].widx] = Wacc[0];
-            Wg[2 * reps[rep].widx + 1] = Wacc[1];
+            Wg[2 * reps[rep].widx] = s_work[0];
+            Wg[2 * reps[rep].widx + 1] = s_work[1];
             if (NPT && boxes_out)
                 for (int c = 0; c < 3; ++c) boxes_out[3 * reps[rep].widx + c] = mu_tot[c] * reps[rep].box0[c];
         }
@@ -989,7 +989,7 @@ size_t cluster_smem_bytes(int n_max, int nb_nst_max, int lut_max, bool npt)
     b += sizeof(float) * (2 * 16 * NSV + NSV);
     b += 16;  // alignment of s_f
     b += sizeof(float4) * SLOTS + sizeof(float2) * SLOTS + sizeof(float) * (32 + NWARP * NRED * 2) +
-         sizeof(unsigned) * 4;
+         sizeof(unsigned) * 4 + sizeof(double) * 4;
     if (npt) {  // s_vir, s_vred, s_vcta, s_mu and their alignments
         b = ((b + 15) & ~(size_t)15) + sizeof(float4) * SLOTS + sizeof(float) * (NWARP * 6 + 16 * 6);
         b = ((b + 7) & ~(size_t)7) + sizeof(double) * 4;
