@@ -197,12 +197,12 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     unsigned char* s_end = (unsigned char*)(s_work + 4);
     float4* s_vir = nullptr;  // barostat: [TPA - 1][SLOTS] pair-lane virials
     float* s_vred = nullptr;  // [NWARP][6] warp sums of the virial
-    double* s_mu = nullptr;   // [3] the step's scale factors
+    ne_baro_smem* s_b = nullptr;  // the replica's barostat
     if constexpr (NPT) {
         s_vir = (float4*)(((size_t)s_end + 15) & ~(size_t)15);
         s_vred = (float*)(s_vir + (TPA - 1) * SLOTS);
-        s_mu = (double*)(((size_t)(s_vred + NWARP * 6) + 15) & ~(size_t)15);
-        s_end = (unsigned char*)(s_mu + 4);
+        s_b = (ne_baro_smem*)(((size_t)(s_vred + NWARP * 6) + 15) & ~(size_t)15);
+        s_end = (unsigned char*)(s_b + 1);
     }
     float4* s_tabP = (float4*)(((size_t)s_end + 15) & ~(size_t)15);  // [nk - 1 - k_lo]
     const int n_int = tab.nk - 1 - k_lo;
@@ -409,10 +409,19 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     }
     bool dead = false;  // the replica left the stencil range: its CTAs keep to the barriers only
     // barostat: the box and the sites scale by mu_tot per axis from the
-    // call's start (the same values in every CTA of the replica); stencil
-    // vectors are multiplied by it
-    double mu_tot[3] = {1.0, 1.0, 1.0};
+    // call's start (the same in every CTA of the replica); stencil vectors are
+    // multiplied by it
     float muf[3] = {1.f, 1.f, 1.f}, mu_min = 1.f;
+    if constexpr (NPT) {
+        if (threadIdx.x >= BTHREADS - 32) ne_baro_draw(*s_b, R_, s_begin);
+        if (threadIdx.x == BTHREADS - 64) {
+            for (int c = 0; c < 3; ++c) s_b->mu_tot[c] = 1.0;
+            s_b->box_ok = 1;
+            for (int c = 0; c < 3; ++c) s_b->box_ok = s_b->box_ok && R_.box0[c] > 2.0 * tab.r_c + 1.2;
+            ne_baro_box(*s_b, R_, S.dt);
+        }
+        __syncthreads();
+    }
 
 #pragma unroll 1
     for (long long it = 0; it <= n_steps && alive; ++it) {
@@ -455,8 +464,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             // the scaled stencil must still cover r_c + 2 max|u|, and the box
             // must keep two periodic images more than 2 r_c apart
             const float need = ((float)tab.r_c + 2.f * umax) / mu_min - (float)tab.r_c;
-            out_ = out_ || !(need <= 2.f * R_.D);
-            for (int c = 0; c < 3; ++c) out_ = out_ || !(mu_tot[c] * R_.box0[c] > 2.0 * tab.r_c + 1.2);
+            out_ = out_ || !(need <= 2.f * R_.D) || !s_b->box_ok;
         }
         if (!dead && out_) {
             // an atom beyond the stencil range: the replica's result is void;
@@ -684,14 +692,13 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                 if (valid && lane > 0) s_vir[(lane - 1) * SLOTS + slot] = make_float4(vxx, vyy, vzz, 0.f);
         }
         __syncthreads();
-        double mus[3] = {1.0, 1.0, 1.0};  // this step's scale factors (barostat)
         if constexpr (NPT) {
             if (!fin) {
                 // the diagonal virial of this CTA's atoms at x_s (double-float
                 // per axis: a fixed warp tree, then warp 0 over the warps) to
                 // global memory; after the barrier warp 0 of every CTA sums the
-                // replica's CTAs in a fixed order and thread 0 takes the
-                // barostat step of the cluster runner
+                // replica's CTAs in a fixed order and takes the barostat
+                // step of the cluster runner
                 const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
                 dfl vd[3] = {};
                 if (own && !dead) {
@@ -728,40 +735,23 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                 alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // virials visible
                 if (!alive) break;
                 if (w == 0) {
+                    const double lam = lam_tab[it + 1];
                     dfl t[3] = {};
                     const float* vp = bb.vir + (size_t)R_.cta0 * 6;
                     for (int r = l; r < C; r += 32)
                         for (int a3 = 0; a3 < 3; ++a3)
                             t[a3] = df_add(t[a3], {__ldcg(&vp[r * 6 + 2 * a3]), __ldcg(&vp[r * 6 + 2 * a3 + 1])});
                     warp_df3(t);
-                    if (l == 0) {
-                        double Wa[3];
-                        for (int a3 = 0; a3 < 3; ++a3) Wa[a3] = (double)t[a3].hi + (double)t[a3].lo;
-                        const double V = mu_tot[0] * R_.box0[0] * mu_tot[1] * R_.box0[1] * mu_tot[2] * R_.box0[2];
-                        const double lam = lam_tab[it + 1], dtd = S.dt;
-                        double z[3];
-                        ne_normals64(ne_philox_block(R_.seed, R_.replica, (unsigned)STREAM_BARO, 0u,
-                                                     (unsigned long long)s),
-                                     z);
-                        const double noise = sqrt(2.0 * R_.kT * R_.mp * dtd / V);
-                        if (R_.npt == 2) {
-                            for (int a3 = 0; a3 < 3; ++a3) {
-                                const double drive = (R_.dof / 3.0 * R_.kT + lam * Wa[a3]) / V - R_.P0;
-                                s_mu[a3] = exp(R_.mp * drive * dtd + noise * z[a3]);
-                            }
-                        } else {  // isotropic; a replica without the barostat has mp = 0: mu = 1
-                            const double drive = (R_.dof * R_.kT + lam * (Wa[0] + Wa[1] + Wa[2])) / (3.0 * V) - R_.P0;
-                            s_mu[0] = s_mu[1] = s_mu[2] = exp((R_.mp * drive * dtd + noise * z[0]) / 3.0);
-                        }
-                    }
+                    const dff W[3] = {{t[0].hi, t[0].lo}, {t[1].hi, t[1].lo}, {t[2].hi, t[2].lo}};
+                    ne_baro_step(*s_b, R_, W, lam, S.dt, tab.r_c, (int)(it & 31));
                 }
                 __syncthreads();
-                for (int a3 = 0; a3 < 3; ++a3) {
-                    mus[a3] = s_mu[a3];
-                    mu_tot[a3] *= mus[a3];
-                    muf[a3] = (float)mu_tot[a3];
-                }
+                for (int a3 = 0; a3 < 3; ++a3) muf[a3] = s_b->muf[a3];
                 mu_min = fminf(muf[0], fminf(muf[1], muf[2]));
+                // for the next step, by the last warps (which own no atom but at
+                // one thread per atom)
+                if (threadIdx.x == BTHREADS - 64) ne_baro_box(*s_b, R_, S.dt);
+                if ((it & 31) == 31 && threadIdx.x >= BTHREADS - 32) ne_baro_draw(*s_b, R_, s + 1);
             }
         }
 
@@ -828,10 +818,13 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                         const float dlt = 0.5f * dt * (v1 + v[c]);
                         if (!(fabsf(dlt) < 0.25f)) bad |= ST_ERANGE;
                         xr[c] += (long long)__float2int_rn(dlt * 4294967296.f);
+                        u[c] = fix_to_float(xr[c]);
                         // barostat: positions scale about the origin, so the
                         // displacement from the scaled site scales by mu
-                        if constexpr (NPT) xr[c] = __double2ll_rn(mus[c] * (double)xr[c]);
-                        u[c] = fix_to_float(xr[c]);
+                        if constexpr (NPT) {
+                            xr[c] = ne_baro_scale(*s_b, xr[c], u[c], c);
+                            u[c] = fix_to_float(xr[c]);
+                        }
                     }
                     ne_normals32(ne_philox_block(R_.seed, R_.replica, (unsigned)S.stream, (unsigned)ta,
                                                  (unsigned long long)(s + 1)),
@@ -881,7 +874,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         if (own)
             for (int c = 0; c < 3; ++c) {
                 // the site of the atom in the (scaled) box
-                const long long site = NPT ? __double2ll_rn(mu_tot[c] * (double)site_fix(c)) : site_fix(c);
+                const long long site = NPT ? __double2ll_rn(s_b->mu_tot[c] * (double)site_fix(c)) : site_fix(c);
                 xg[gi + c] = (double)(xr[c] + site) / XSCALE;
                 vg[gi + c] = (double)v[c];
             }
@@ -889,7 +882,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             Wg[2 * R_.widx] = s_work[0];
             Wg[2 * R_.widx + 1] = s_work[1];
             if (NPT && boxes_out)
-                for (int c = 0; c < 3; ++c) boxes_out[3 * R_.widx + c] = mu_tot[c] * R_.box0[c];
+                for (int c = 0; c < 3; ++c) boxes_out[3 * R_.widx + c] = s_b->mu_tot[c] * R_.box0[c];
         }
     }
 }
@@ -940,7 +933,7 @@ size_t brick_smem_bytes(int tpa, int nb_nst_max, int lut_max, bool npt)
         b = (b + 15) & ~(size_t)15;
         b += sizeof(float4) * (size_t)(tpa - 1) * slots + sizeof(float) * NWARP * 6;
         b = (b + 15) & ~(size_t)15;
-        b += sizeof(double) * 4;
+        b += sizeof(ne_baro_smem);
     }
     return ((b + 15) & ~(size_t)15) + 16;  // + alignment of the tables
 }

@@ -65,7 +65,11 @@ constexpr int SLOTS = THREADS / TPA;  // atoms per CTA (one CTA per SM)
 // columns (one CTA per SM); warp w uses TMEM lanes 32 (w mod 4) .. +31 (its
 // sub-partition's) and the CW columns from CW (w div 4): visit q of a thread
 // is column q of its lane for f'(r)/r and half of column QMAX + q / 2 for j
-// (two 16-bit slots a column), loaded FRB visits at a time.  Visits past
+// (two 16-bit slots a column), loaded FRB visits at a time.  With the barostat
+// the last NE_TM_STATE columns hold the state of the atom the thread owns
+// between its integrations: that kernel spilled 256 bytes a thread without
+// (four bcc 12^3, a step: 39.0 -> 37.4 us); the fixed-box kernel, which spills
+// 20, loses more by the eight visits the columns cost (26.8 -> 27.2 us).  Visits past
 // QMAX (a hot or disordered replica) take j from the wrapped-cell tables
 // and are recomputed in pass 2.
 constexpr int TM_COLS = NE_TM_COLS;
@@ -75,9 +79,7 @@ constexpr int FRB = NE_TM_BATCH;
 constexpr int NKT = 256;
 constexpr int NWARP = THREADS / 32;
 constexpr int WQ = NWARP / 4;  // warps per TMEM lane quarter
-constexpr int QMAX = TM_COLS / WQ * 2 / 3 / FRB * FRB;
-constexpr int CW = QMAX + QMAX / 2;  // TMEM columns per warp
-static_assert(NWARP % 4 == 0 && QMAX >= FRB && QMAX % FRB == 0 && WQ * CW <= TM_COLS, "TMEM columns per warp");
+constexpr int tm_qmax(bool state) { return (TM_COLS / WQ - (state ? NE_TM_STATE : 0)) * 2 / 3 / FRB * FRB; }
 
 // partial sums broadcast at the end of step s for step s+1: the energies
 // (double-float), then sum u and sum xi for the mean removal (FP32)
@@ -222,6 +224,9 @@ __global__ void __launch_bounds__(THREADS, 1)
               long long s_begin, long long n_steps, Tables tab, unsigned long long* work, int k_lo,
               const double* __restrict__ lam_tab, double* __restrict__ wcum, double* __restrict__ boxes_out)
 {
+    constexpr int QMAX = tm_qmax(NPT);
+    constexpr int CW = QMAX + QMAX / 2 + (NPT ? NE_TM_STATE : 0);  // TMEM columns per warp
+    static_assert(NWARP % 4 == 0 && QMAX >= FRB && QMAX % FRB == 0 && WQ * CW <= TM_COLS, "TMEM columns per warp");
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
@@ -256,14 +261,14 @@ __global__ void __launch_bounds__(THREADS, 1)
     double* s_work = (double*)(s_tm + 4);                         // [4] the work thread's W and U_E
     // barostat: the diagonal virial of the second pair lane of each slot, the
     // warps' double-float partials, every CTA's partial (written by the CTA
-    // into all CTAs of the cluster) and the step's scale factors
+    // into all CTAs of the cluster) and the replica's barostat
     float4* s_vir = (float4*)(((size_t)(s_work + 4) + 15) & ~(size_t)15);  // [SLOTS] (NPT)
     float* s_vred = (float*)(s_vir + (NPT ? SLOTS : 0));          // [NWARP][6] (NPT)
     float* s_vcta = s_vred + (NPT ? NWARP * 6 : 0);               // [16][6] (NPT)
-    double* s_mu = (double*)(((size_t)(s_vcta + (NPT ? 16 * 6 : 0)) + 7) & ~(size_t)7);  // [4] (NPT)
+    ne_baro_smem* s_b = (ne_baro_smem*)(((size_t)(s_vcta + (NPT ? 16 * 6 : 0)) + 7) & ~(size_t)7);  // (NPT)
     // spline intervals [k_lo, nk - 1) of phi, then of f: separate arrays, so
     // consecutive intervals fall in consecutive 16-byte bank groups
-    float4* s_tabP = (float4*)(((size_t)(s_mu + (NPT ? 4 : 0)) + 15) & ~(size_t)15);  // [nk-1-k_lo]
+    float4* s_tabP = (float4*)(((size_t)(s_b + (NPT ? 1 : 0)) + 15) & ~(size_t)15);  // [nk-1-k_lo]
     const int n_int = tab.nk - 1 - k_lo;  // intervals of the r grid held in shared memory
     float4* s_tabF = s_tabP + n_int;                                           // [nk-1-k_lo]
     {
@@ -343,6 +348,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     const unsigned tm_w = tm_base + ((unsigned)(32 * ((threadIdx.x >> 5) & 3)) << 16) +
                           (unsigned)(CW * (threadIdx.x >> 7));  // this warp's lanes and columns
     const unsigned tm_j = tm_w + (unsigned)QMAX;                    // its neighbour-slot columns
+    const unsigned tm_s = tm_j + (unsigned)(QMAX / 2);              // the owned atom's state
+    const bool own_warp = (int)(threadIdx.x >> 5) < own_warps;      // warp-uniform
     // the neighbour slots of this thread's first QMAX visits (entries past
     // the stencil, which no visit reaches, get slot 0); every atom of the
     // replica has a 16-byte entry in shared memory, so slots are < 2^16
@@ -382,11 +389,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     const float inv_dK = (float)(NKT - 1) / (2.f * Dr);
 
-    // ---- state of the owned atom: displacement from its site in fixed point
-    // (x * 2^32 - site * 2^32, registers), velocity and this step's normals
-    // in FP32
-    long long xr[3] = {0, 0, 0};
-    float v[3] = {0, 0, 0}, u[3] = {0, 0, 0}, xi[3] = {0, 0, 0};
+    // ---- state of the owned atom (with the barostat in tensor memory between
+    // integrations): displacement from its site in fixed point (x * 2^32 - site * 2^32),
+    // velocity and this step's normals in FP32
+    ne_atom_state A_ = {};
+    float u[3] = {0.f, 0.f, 0.f};
     int bad = 0;
     // the owned atom's spring, half-step factor and noise amplitude, and its
     // weights in the centre-of-mass sums: with species tables the spring sum
@@ -406,24 +413,28 @@ __global__ void __launch_bounds__(THREADS, 1)
         float um = 0.f;
         if (own) {
             for (int q = 0; q < 3; ++q) {
-                xr[q] = __double2ll_rn(xg[gi + q] * XSCALE) - site_fix(q);
-                v[q] = (float)vg[gi + q];
-                u[q] = fix_to_float(xr[q]);
+                A_.xr[q] = __double2ll_rn(xg[gi + q] * XSCALE) - site_fix(q);
+                A_.v[q] = (float)vg[gi + q];
+                u[q] = fix_to_float(A_.xr[q]);
             }
             const float4 uv = make_float4(u[0], u[1], u[2], 0.f);
             s_u[tsu] = uv;
             for (int r = 1; r < C; ++r) cluster.map_shared_rank(s_u, peer(r))[tsu] = uv;
             ne_normals32(ne_philox_block(reps[rep].seed, reps[rep].replica, (unsigned)S.stream, (unsigned)ta,
                                          (unsigned long long)s_begin),
-                         xi);
+                         A_.xi);
             const float u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
             pd[P_UE] = {0.5f * kf * u2, 0.f};
             const float wxi = spc ? R_.mfs[spq()] * R_.c2fs[spq()] : 1.f;
             for (int c = 0; c < 3; ++c) {
                 pf[P_UX - ND_ + c] = spc ? kf * u[c] : u[c];
-                pf[P_XX - ND_ + c] = spc ? wxi * xi[c] : xi[c];
+                pf[P_XX - ND_ + c] = spc ? wxi * A_.xi[c] : A_.xi[c];
             }
             um = sqrtf(u2);
+        }
+        if constexpr (NPT) {
+            __syncwarp();
+            if (own_warp) ne_tm_st_state(tm_s, A_);  // pass 1 waits for its stores
         }
         cta_sum_bcast<ND_, NF_>(cluster, pd, pf, um, s_red, s_slotP + (s_begin & 1) * 16 * NSV,
                                 s_slotM + (s_begin & 1) * 16, rank, C, own_warps);
@@ -449,10 +460,18 @@ __global__ void __launch_bounds__(THREADS, 1)
         s_work[1] = Wg[2 * reps[rep].widx + 1];
     }
     // barostat: the box and the lattice sites scale by mu_tot per axis from
-    // the call's start (every thread holds the same values: they come from
-    // the same sums); stencil vectors are multiplied by it
-    double mu_tot[3] = {1.0, 1.0, 1.0};
+    // the call's start (the same in every CTA: it comes from the same sums);
+    // stencil vectors are multiplied by it
     float muf[3] = {1.f, 1.f, 1.f}, mu_min = 1.f;
+    if constexpr (NPT) {
+        if (threadIdx.x >= THREADS - 32) ne_baro_draw(*s_b, reps[rep], s_begin);
+        if (threadIdx.x == THREADS - 64) {
+            for (int c = 0; c < 3; ++c) s_b->mu_tot[c] = 1.0;
+            s_b->box_ok = 1;
+            for (int c = 0; c < 3; ++c) s_b->box_ok = s_b->box_ok && reps[rep].box0[c] > 2.0 * tab.r_c + 1.2;
+            ne_baro_box(*s_b, reps[rep], S.dt);
+        }
+    }
 
 #pragma unroll 1
     for (long long it = 0; it <= n_steps; ++it) {
@@ -498,9 +517,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             // the scaled stencil must still cover r_c + 2 max|u|, and the box
             // must keep two periodic images more than 2 r_c apart
             const float need = ((float)tab.r_c + 2.f * umax) / mu_min - (float)tab.r_c;
-            out = out || !(need <= 2.f * reps[rep].D);
-            for (int c = 0; c < 3; ++c)
-                out = out || !(mu_tot[c] * reps[rep].box0[c] > 2.0 * tab.r_c + 1.2);
+            out = out || !(need <= 2.f * reps[rep].D) || !s_b->box_ok;
         }
         if (out) {
             if (threadIdx.x == 0) {
@@ -798,6 +815,13 @@ __global__ void __launch_bounds__(THREADS, 1)
             dfl pd[ND_] = {};
             float pf[NF_] = {};
             float un = 0.f;
+            if constexpr (NPT) {
+                __syncwarp();
+                if (own_warp) ne_tm_ld_state(tm_s, A_);
+                for (int c = 0; c < 3; ++c) u[c] = fix_to_float(A_.xr[c]);
+            }
+            long long(&xr)[3] = A_.xr;
+            float(&v)[3] = A_.v, (&xi)[3] = A_.xi;
             if (own) {
                 const float4 f1_ = s_f[threadIdx.x];
                 const float4 f = make_float4(fx + f1_.x, fy + f1_.y, fz + f1_.z, ep + f1_.w);
@@ -837,50 +861,35 @@ __global__ void __launch_bounds__(THREADS, 1)
                                  xi);
                 }
             }
+            double lam_next = 0.0;
+            if (NPT && threadIdx.x < 32) lam_next = lam_tab[it + 1];
             asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
             if constexpr (NPT) {
                 if (!fin) {
                     // the barostat step after the second drift (reading A23): the
                     // replica's diagonal virial at x_s from the C CTA partials
-                    // (fixed order), then one overdamped Langevin step of ln V
+                    // (fixed tree), then one overdamped Langevin step of ln V
                     // (isotropic) or of each ln L_a, with the first (or a-th)
                     // normal of Philox stream 5 at (atom 0, step s)
-                    if (threadIdx.x == 0) {
-                        const XRep& Rb = reps[rep];
-                        double Wa[3];
-                        for (int a3 = 0; a3 < 3; ++a3) {
-                            dfl acc = {0.f, 0.f};
-                            for (int r = 0; r < C; ++r) acc = df_add(acc, {s_vcta[r * 6 + 2 * a3], s_vcta[r * 6 + 2 * a3 + 1]});
-                            Wa[a3] = (double)acc.hi + (double)acc.lo;
-                        }
-                        const double V = mu_tot[0] * Rb.box0[0] * mu_tot[1] * Rb.box0[1] * mu_tot[2] * Rb.box0[2];
-                        const double lam = lam_tab[it + 1], dtd = S.dt;
-                        double z[3];
-                        ne_normals64(ne_philox_block(Rb.seed, Rb.replica, (unsigned)STREAM_BARO, 0u,
-                                                     (unsigned long long)s),
-                                     z);
-                        const double noise = sqrt(2.0 * Rb.kT * Rb.mp * dtd / V);
-                        if (Rb.npt == 2) {
-                            for (int a3 = 0; a3 < 3; ++a3) {
-                                const double drive = (Rb.dof / 3.0 * Rb.kT + lam * Wa[a3]) / V - Rb.P0;
-                                s_mu[a3] = exp(Rb.mp * drive * dtd + noise * z[a3]);
-                            }
-                        } else {
-                            const double drive = (Rb.dof * Rb.kT + lam * (Wa[0] + Wa[1] + Wa[2])) / (3.0 * V) - Rb.P0;
-                            s_mu[0] = s_mu[1] = s_mu[2] = exp((Rb.mp * drive * dtd + noise * z[0]) / 3.0);
-                        }
+                    if (threadIdx.x < 32) {
+                        const int r = threadIdx.x;
+                        dff W[3];
+                        for (int a3 = 0; a3 < 3; ++a3)
+                            W[a3] = dff_warp_sum(r < C ? dff{s_vcta[r * 6 + 2 * a3], s_vcta[r * 6 + 2 * a3 + 1]} : dff{0.f, 0.f});
+                        ne_baro_step(*s_b, reps[rep], W, lam_next, S.dt, tab.r_c, (int)(it & 31));
                     }
                     __syncthreads();
                     for (int a3 = 0; a3 < 3; ++a3) {
-                        const double mu = s_mu[a3];
-                        mu_tot[a3] *= mu;
-                        muf[a3] = (float)mu_tot[a3];
+                        muf[a3] = s_b->muf[a3];
                         if (own) {  // positions scale about the origin: the displacement from the scaled site by mu
-                            xr[a3] = __double2ll_rn(mu * (double)xr[a3]);
+                            xr[a3] = ne_baro_scale(*s_b, xr[a3], u[a3], a3);
                             u[a3] = fix_to_float(xr[a3]);
                         }
                     }
                     mu_min = fminf(muf[0], fminf(muf[1], muf[2]));
+                    // for the next step, by warps that own no atom
+                    if (threadIdx.x == THREADS - 64) ne_baro_box(*s_b, reps[rep], S.dt);
+                    if ((it & 31) == 31 && threadIdx.x >= THREADS - 32) ne_baro_draw(*s_b, reps[rep], s + 1);
                 }
             }
             if (own) {
@@ -901,10 +910,18 @@ __global__ void __launch_bounds__(THREADS, 1)
                 for (int c = 0; c < 3; ++c)
                     if (!isfinite(v[c])) bad |= ST_ENAN;
             }
+            if constexpr (NPT) {
+                __syncwarp();
+                if (own_warp) ne_tm_st_state(tm_s, A_);
+            }
             if (!fin)
                 cta_sum_bcast<ND_, NF_>(cluster, pd, pf, un, s_red, s_slotP + ((s + 1) & 1) * 16 * NSV,
                                         s_slotM + ((s + 1) & 1) * 16, rank, C, own_warps);
         }
+    }
+    if constexpr (NPT) {
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        if (own_warp) ne_tm_ld_state(tm_s, A_);
     }
     ne_tm_free(tm_base);  // every warp is past its last TMEM access
     if (bad) {
@@ -933,15 +950,15 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (own)
             for (int c = 0; c < 3; ++c) {
                 // the site of the atom in the (scaled) box
-                const long long site = NPT ? __double2ll_rn(mu_tot[c] * (double)site_fix(c)) : site_fix(c);
-                xg[gi + c] = (double)(xr[c] + site) / XSCALE;
-                vg[gi + c] = (double)v[c];
+                const long long site = NPT ? __double2ll_rn(s_b->mu_tot[c] * (double)site_fix(c)) : site_fix(c);
+                xg[gi + c] = (double)(A_.xr[c] + site) / XSCALE;
+                vg[gi + c] = (double)A_.v[c];
             }
         if (wthread) {
             Wg[2 * reps[rep].widx] = s_work[0];
             Wg[2 * reps[rep].widx + 1] = s_work[1];
             if (NPT && boxes_out)
-                for (int c = 0; c < 3; ++c) boxes_out[3 * reps[rep].widx + c] = mu_tot[c] * reps[rep].box0[c];
+                for (int c = 0; c < 3; ++c) boxes_out[3 * reps[rep].widx + c] = s_b->mu_tot[c] * reps[rep].box0[c];
         }
     }
 }
@@ -990,9 +1007,9 @@ size_t cluster_smem_bytes(int n_max, int nb_nst_max, int lut_max, bool npt)
     b += 16;  // alignment of s_f
     b += sizeof(float4) * SLOTS + sizeof(float2) * SLOTS + sizeof(float) * (32 + NWARP * NRED * 2) +
          sizeof(unsigned) * 4 + sizeof(double) * 4;
-    if (npt) {  // s_vir, s_vred, s_vcta, s_mu and their alignments
+    if (npt) {  // s_vir, s_vred, s_vcta, s_b and their alignments
         b = ((b + 15) & ~(size_t)15) + sizeof(float4) * SLOTS + sizeof(float) * (NWARP * 6 + 16 * 6);
-        b = ((b + 7) & ~(size_t)7) + sizeof(double) * 4;
+        b = ((b + 7) & ~(size_t)7) + sizeof(ne_baro_smem);
     }
     return ((b + 15) & ~(size_t)15) + 16;  // + alignment of the tables
 }

@@ -131,6 +131,150 @@ __device__ __forceinline__ void ne_tm_ld_f8u4(unsigned taddr_f, unsigned taddr_w
     for (int q = 0; q < 8; ++q) f[q] = __uint_as_float(r[q]);
 }
 
+// The state of the atom a thread owns, NE_TM_STATE columns of its lane: the
+// displacement from its site in fixed point (three 64-bit words), velocity and
+// the normals of the coming step.  Kept there between integrations it holds no
+// registers through the pair passes, which run at the launch bound's cap.
+#define NE_TM_STATE 12
+struct ne_atom_state {
+    long long xr[3];
+    float v[3], xi[3];
+};
+
+__device__ __forceinline__ void ne_tm_st_state(unsigned taddr, const ne_atom_state& a)
+{
+    const unsigned w[12] = {(unsigned)a.xr[0], (unsigned)(a.xr[0] >> 32), (unsigned)a.xr[1], (unsigned)(a.xr[1] >> 32),
+                            (unsigned)a.xr[2], (unsigned)(a.xr[2] >> 32), __float_as_uint(a.v[0]), __float_as_uint(a.v[1]),
+                            __float_as_uint(a.v[2]), __float_as_uint(a.xi[0]), __float_as_uint(a.xi[1]),
+                            __float_as_uint(a.xi[2])};
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 :
+                 : "r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 :
+                 : "r"(taddr + 8u), "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11])
+                 : "memory");
+}
+
+// (the stores before it have been waited for: tcgen05.wait::st)
+__device__ __forceinline__ void ne_tm_ld_state(unsigned taddr, ne_atom_state& a)
+{
+    unsigned r[8], w[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                 : "r"(taddr + 8u)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
+                 :
+                 : "memory");
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a.xr[c] = (long long)(((unsigned long long)r[2 * c + 1] << 32) | r[2 * c]);
+    a.v[0] = __uint_as_float(r[6]);
+    a.v[1] = __uint_as_float(r[7]);
+    a.v[2] = __uint_as_float(w[0]);
+    a.xi[0] = __uint_as_float(w[1]);
+    a.xi[1] = __uint_as_float(w[2]);
+    a.xi[2] = __uint_as_float(w[3]);
+}
+
+// The barostat of the crystal runners (reading A23), one replica a CTA.  GB300
+// issues a warp's FP64 instructions ~64 cycles apart, so what one thread did
+// between the virial and the integration -- the FP64 normal, square root,
+// divisions and exponential, ~300 of them -- held the whole CTA for ~9 us a step.
+// Here the normals of 32 steps are drawn at once, a step per lane, and 1 / V and
+// the noise amplitude follow from the box as soon as it is known, both by warps
+// that own no atom and while the others integrate; what is left behind the
+// virial is ~15 FP64 instructions.
+struct ne_baro_smem {
+    double z[32][3];      // normals of steps s_begin + 32 k .. + 31 (Philox stream 5, atom 0)
+    double mu_tot[3];     // box and lattice sites over those of the call's start, per axis
+    double em1[3];        // the step's scale factors minus one
+    double inv_v, noise;  // 1 / V and sqrt(2 kT m dt / V)
+    float muf[3], em1f[3];  // mu_tot and em1 in FP32
+    int small;            // every |em1| below 2e-4 (ne_baro_scale)
+    int box_ok;           // two periodic images of a site stay more than 2 r_c apart
+};
+
+// exp(x) - 1: the Taylor sum for the small arguments of a barostat step
+// (|x| < 1/64: the eighth term is below 2^-60 of the first), else expm1
+__device__ __forceinline__ double ne_baro_expm1(double x)
+{
+    if (fabs(x) >= 0.015625) return expm1(x);
+    double t = fma(x, 1.0 / 5040.0, 1.0 / 720.0);
+    t = fma(t, x, 1.0 / 120.0);
+    t = fma(t, x, 1.0 / 24.0);
+    t = fma(t, x, 1.0 / 6.0);
+    t = fma(t, x, 0.5);
+    return fma(t * x, x, x);
+}
+
+// normals of the 32 steps from s on, a step per lane
+__device__ __forceinline__ void ne_baro_draw(ne_baro_smem& b, const XRep& R, long long s)
+{
+    double z[3];
+    ne_normals64(ne_philox_block(R.seed, R.replica, (unsigned)STREAM_BARO, 0u,
+                                 (unsigned long long)(s + (threadIdx.x & 31))),
+                 z);
+    for (int c = 0; c < 3; ++c) b.z[threadIdx.x & 31][c] = z[c];
+}
+
+// 1 / V and the noise amplitude of the box mu_tot, by one thread
+__device__ __forceinline__ void ne_baro_box(ne_baro_smem& b, const XRep& R, double dt)
+{
+    const double V = b.mu_tot[0] * R.box0[0] * b.mu_tot[1] * R.box0[1] * b.mu_tot[2] * R.box0[2];
+    b.inv_v = 1.0 / V;
+    b.noise = sqrt(2.0 * R.kT * R.mp * dt / V);
+}
+
+// The step's scale factors from the diagonal virial W (double-float per axis,
+// the same in every lane), by lanes 0 .. 2 of one warp; i: the step's place in z
+__device__ __forceinline__ void ne_baro_step(ne_baro_smem& b, const XRep& R, const dff (&W)[3], double lam, double dt,
+                                             double r_c, int i)
+{
+    const int a = threadIdx.x & 31;
+    if (a < 3) {
+        double x;
+        if (R.npt == 2) {
+            const double Wa = (double)(a == 0 ? W[0].hi : (a == 1 ? W[1].hi : W[2].hi)) +
+                              (double)(a == 0 ? W[0].lo : (a == 1 ? W[1].lo : W[2].lo));
+            const double drive = (R.dof / 3.0 * R.kT + lam * Wa) * b.inv_v - R.P0;
+            x = R.mp * drive * dt + b.noise * b.z[i][a];
+        } else {  // isotropic; a replica without the barostat has mp = 0
+            const dff w = dff_add(dff_add(W[0], W[1]), W[2]);
+            const double drive = (R.dof * R.kT + lam * ((double)w.hi + (double)w.lo)) * (1.0 / 3.0) * b.inv_v - R.P0;
+            x = (R.mp * drive * dt + b.noise * b.z[i][0]) * (1.0 / 3.0);
+        }
+        const double e = ne_baro_expm1(x), mu = fma(e, b.mu_tot[a], b.mu_tot[a]);
+        b.em1[a] = e;
+        b.mu_tot[a] = mu;
+        b.muf[a] = (float)mu;
+        const bool ok = mu * R.box0[a] > 2.0 * r_c + 1.2;
+        b.em1f[a] = (float)e;
+        const unsigned all = __ballot_sync(7u, ok), sm = __ballot_sync(7u, fabs(e) < 2e-4);
+        if (a == 0) {
+            b.box_ok = all == 7u;
+            b.small = sm == 7u;
+        }
+    }
+}
+
+// A displacement in fixed point (2^-32 A) scaled by 1 + em1 of axis c: for
+// small factors by its change, from the FP32 displacement u (the change's error,
+// 2^-23 of |e u| <= 4e-4 A, is below a quarter of the grid; a usual step's
+// e ~ 1e-5 leaves a hundredth), else in FP64
+__device__ __forceinline__ long long ne_baro_scale(const ne_baro_smem& b, long long xr, float u, int c)
+{
+    if (b.small) return xr + (long long)__float2int_rn(b.em1f[c] * u * 4294967296.f);
+    return __double2ll_rn(fma(b.em1[c], (double)xr, (double)xr));
+}
+
 // Warp 0 of the CTA takes all NE_TM_COLS columns (the base address goes to
 // *s_slot in shared memory); the caller then makes it visible with
 // tcgen05.fence::before_thread_sync, a CTA barrier and
