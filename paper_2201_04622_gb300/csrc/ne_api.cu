@@ -58,7 +58,7 @@ struct CrPlan {
 struct ne_ctx {
     ne_eam_params eam{};
     int max_atoms = 0, max_rep = 0, tiles_cap = 0, cells_cap = 0;
-    int sms = 0;        // SMs of the context's device
+    int sms = 0, smem_optin = 0;  // SMs of the context's device, shared memory a block may have
     int tpa = 0;        // threads per atom of the pair passes (0: by the batch's size)
     int cluster_c = 0;  // crystal runner: CTAs per cluster (0: chosen per batch)
     int last_nrep = 0;  // replicas of the last multi-kernel run (ne_ctx_boxes)
@@ -75,7 +75,8 @@ struct ne_ctx {
     int *nbr = nullptr, *ncnt = nullptr, *sl = nullptr, *scnt = nullptr;
     int *cellof = nullptr, *cslot = nullptr, *craw = nullptr, *cstart = nullptr, *ccount = nullptr;
     float4* csort = nullptr;
-    unsigned* nl_done = nullptr;
+    unsigned *nl_done = nullptr, *grp_done = nullptr;
+    double* partG = nullptr;
     double *partA = nullptr, *partB = nullptr, *tot = nullptr, *W = nullptr, *scratch = nullptr;
     unsigned* tile_done = nullptr;
     int *flags = nullptr, *building = nullptr, *status = nullptr, *tile_rep = nullptr;
@@ -105,8 +106,7 @@ struct ne_ctx {
     cudaEvent_t gev[17] = {};
     float4* st_vec = nullptr;
     float* st_dist = nullptr;
-    float* bins = nullptr;
-    int bins_blocks = 0;
+    unsigned long long* bins = nullptr;  // mixed backward: 64-bit bins (allocated on first use)
     std::vector<RepDev> rep_h;
     std::vector<int> tile_rep_h;
     int last_bits = 0;
@@ -258,7 +258,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     if (n_tot > ctx->max_atoms) return fail(ctx, NE_ENOMEM, "atom count exceeds the context");
     ctx->rep_h.assign(n_rep, RepDev{});
     ctx->tile_rep_h.clear();
-    int cells = 0, npt_any = 0;
+    int cells = 0, npt_any = 0, groups = 0;
     const double rc = ctx->eam.r_c;
     for (int r = 0; r < n_rep; ++r) {
         const ne_md_params& m = md[(size_t)r * md_stride];
@@ -302,6 +302,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
         R.n = n;
         R.tile0 = (int)ctx->tile_rep_h.size();
         R.ntile = (n + NE_TILE - 1) / NE_TILE;
+        R.grp0 = groups;
+        groups += (R.ntile + GROUP_TILES - 1) / GROUP_TILES;
         for (int t = 0; t < R.ntile; ++t) ctx->tile_rep_h.push_back(r);
         R.cell_off = cells;
         cells += R.nc[0] * R.nc[1] * R.nc[2];
@@ -341,6 +343,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.n_tiles = n_tiles;
     for (const RepDev& R : ctx->rep_h) B.n_max = std::max(B.n_max, R.n);
     B.sms = ctx->sms;
+    B.smem_optin = ctx->smem_optin;
     B.g = ctx->tpa > 0 ? ctx->tpa : ne::lanes_per_atom(n_tot);
     B.rep = ctx->rep;
     B.tile_rep = ctx->tile_rep;
@@ -369,6 +372,9 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.ccount = ctx->ccount;
     B.partA = ctx->partA;
     B.partB = ctx->partB;
+    B.partG = ctx->partG;
+    B.n_grp = groups;
+    B.grp_done = ctx->grp_done;
     B.tot = ctx->tot;
     B.tile_done = ctx->tile_done;
     B.nl_done = ctx->nl_done;
@@ -420,14 +426,13 @@ void force_eval(const DevBatch& B, bool mixed, cudaStream_t st)
 struct GradAcc {
     double* gtheta;
     const double* w;
-    float* bins;
-    int nbb;
+    unsigned long long* bins;
     long long s_off;
 };
 
 void grad_at(const DevBatch& B, bool mixed, const GradAcc* ga, const long long* ctr, int j, cudaStream_t st)
 {
-    if (ga) ne::launch_backward(B, mixed, 0.0, ga->gtheta, ga->bins, ga->nbb, true, st, ga->w, ctr, j,
+    if (ga) ne::launch_backward(B, mixed, 0.0, ga->gtheta, ga->bins, true, st, ga->w, ctr, j,
                                 ga->s_off, false);
 }
 
@@ -646,6 +651,7 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     int dev = 0;
     A(cudaGetDevice(&dev));
     A(cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, dev));
+    A(cudaDeviceGetAttribute(&ctx->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     A(dalloc(&ctx->theta, 6 * nk));
     A(dalloc(&ctx->pf32, 2 * nk));
     A(dalloc(&ctx->pf64, 2 * nk));
@@ -672,6 +678,9 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->cstart, (size_t)ctx->cells_cap + R));
     A(dalloc(&ctx->ccount, (size_t)ctx->cells_cap));
     A(dalloc(&ctx->nl_done, R));
+    const size_t grp_cap = (size_t)ctx->tiles_cap / GROUP_TILES + R + 1;
+    A(dalloc(&ctx->grp_done, grp_cap));
+    A(dalloc(&ctx->partG, grp_cap * (NPA + NPB)));
     A(dalloc(&ctx->partA, (size_t)ctx->tiles_cap * NE_PAIR_SUB * NPA));
     A(dalloc(&ctx->partB, (size_t)ctx->tiles_cap * NPB));
     A(dalloc(&ctx->tot, R * NTOT));
@@ -697,6 +706,7 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     // the list build leaves these at zero
     if (ok) ok = cudaMemset(ctx->ccount, 0, sizeof(int) * (size_t)ctx->cells_cap) == cudaSuccess;
     if (ok) ok = cudaMemset(ctx->nl_done, 0, sizeof(unsigned) * R) == cudaSuccess;
+    if (ok) ok = cudaMemset(ctx->grp_done, 0, sizeof(unsigned) * grp_cap) == cudaSuccess;
     if (ok) ok = cudaMemset(ctx->building, 0, sizeof(int) * R) == cudaSuccess;
     if (!ok) {
         ne_ctx_destroy(ctx);
@@ -725,7 +735,7 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
     void* ptrs[] = {ctx->theta, ctx->pf32, ctx->pf64, ctx->F32, ctx->F64, ctx->pos32, ctx->posF,
                     ctx->pbuild, ctx->f32, ctx->f64, ctx->pos64, ctx->gs, ctx->rho, ctx->xi64, ctx->xi32,
                     ctx->nbr, ctx->ncnt, ctx->sl, ctx->scnt, ctx->cellof, ctx->cslot, ctx->craw, ctx->csort,
-                    ctx->cstart, ctx->ccount, ctx->nl_done, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
+                    ctx->cstart, ctx->ccount, ctx->nl_done, ctx->grp_done, ctx->partG, ctx->partA, ctx->partB, ctx->tot, ctx->W, ctx->scratch,
                     ctx->tile_done, ctx->flags, ctx->building, ctx->status, ctx->tile_rep, ctx->rep, ctx->step_ctr, ctx->rebuilds, ctx->xrep, ctx->work, ctx->st_vec, ctx->st_dist, ctx->lam_tab, ctx->run_lam,
                     ctx->bins};
     for (void* p : ptrs)
@@ -1022,6 +1032,22 @@ ne_status ne_spring_forces(const double* x_dev, const double* x0_dev, int n, dou
     return cudaGetLastError() == cudaSuccess ? NE_OK : NE_ECUDA;
 }
 
+// The mixed backward's bins, zeroed once: each launch leaves them at zero.
+static ne_status backward_bins(ne_ctx* ctx, cudaStream_t st)
+{
+    if (ctx->bins) return NE_OK;
+    const size_t bytes = ne::backward_bins_bytes(ctx->eam.n_knots);
+    unsigned long long* p = nullptr;
+    NE_CU(cudaMalloc((void**)&p, bytes));
+    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, st);
+    if (e != cudaSuccess) {
+        cudaFree(p);
+        return fail(ctx, NE_ECUDA, std::string("clearing the bins: ") + cudaGetErrorString(e));
+    }
+    ctx->bins = p;
+    return NE_OK;
+}
+
 static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_dev, int n, const double box[3],
                                double gE, double* gx_dev, double* gtheta_dev, bool accumulate, void* stream)
 {
@@ -1046,15 +1072,11 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
     if (gx_dev) ne::launch_export(B, mixed, gx_dev, nullptr, st);
     if (mixed && !ne::backward_fits(ctx->eam.n_knots))
         return fail(ctx, NE_EINVAL, "mixed backward: n_knots too large for one block's shared-memory bins");
-    int nbb = ne::backward_bin_blocks(B);
-    if (mixed && nbb > ctx->bins_blocks) {
-        if (ctx->bins) cudaFree(ctx->bins);
-        ctx->bins = nullptr;
-        ctx->bins_blocks = 0;
-        NE_CU(cudaMalloc((void**)&ctx->bins, ne::backward_bins_bytes(ctx->eam.n_knots, nbb)));
-        ctx->bins_blocks = nbb;
+    if (mixed) {
+        s = backward_bins(ctx, st);
+        if (s) return s;
     }
-    ne::launch_backward(B, mixed, gE, gtheta_dev, ctx->bins, nbb, accumulate, st);
+    ne::launch_backward(B, mixed, gE, gtheta_dev, ctx->bins, accumulate, st);
     if (gx_dev) ne::launch_scale(gx_dev, 3 * n, -gE, st);  // dU/dx = -F times gE
     return finish(ctx, st);
 }
@@ -1173,17 +1195,13 @@ static ne_status segment_impl(ne_ctx* ctx, const ne_md_params* md, int n_rep, co
     Sched S = make_sched(md[0]);
     if (n_steps == 0) return finish(ctx, st);
     const bool mixed = md[0].prec == NE_MIXED;
-    GradAcc ga{gtheta, gw, nullptr, 0, s_begin};
+    GradAcc ga{gtheta, gw, nullptr, s_begin};
     if (gtheta) {
         if (mixed && !ne::backward_fits(ctx->eam.n_knots))
             return fail(ctx, NE_EINVAL, "mixed backward: n_knots too large for one block's shared-memory bins");
-        ga.nbb = ne::backward_bin_blocks(B);
-        if (mixed && ga.nbb > ctx->bins_blocks) {
-            if (ctx->bins) cudaFree(ctx->bins);
-            ctx->bins = nullptr;
-            ctx->bins_blocks = 0;
-            NE_CU(cudaMalloc((void**)&ctx->bins, ne::backward_bins_bytes(ctx->eam.n_knots, ga.nbb)));
-            ctx->bins_blocks = ga.nbb;
+        if (mixed) {
+            s = backward_bins(ctx, st);
+            if (s) return s;
         }
         ga.bins = ctx->bins;
         // the backward kernel's shared-memory attribute, once, outside any capture

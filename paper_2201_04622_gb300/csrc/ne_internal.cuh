@@ -33,6 +33,7 @@ struct __align__(32) ned4 {
 };
 
 #define NE_TILE 64
+#define GROUP_TILES 64  // tiles of a replica whose partials pass 2 sums first
 #define NE_PAIR_SUB 8   // most pair blocks per tile (32 lanes per atom)
 // list entry: neighbour in the low 27 bits, above them the code 9 (a + 1) + 3 (b + 1) + c + 1 of the
 // shift (a, b, c), each in {-1, 0, 1}, in box lengths, that is added to r_j - r_i
@@ -69,6 +70,7 @@ struct RepDev {
     double rlist2;   // (r_c + skin)^2
     float half_skin2;
     int off, n, tile0, ntile;
+    int grp0;        // first of its groups of GROUP_TILES tiles
     int nc[3];       // cells per axis; 0 = all pairs
     int cell_off;
     int dof;
@@ -119,7 +121,8 @@ struct DevBatch {
     int n_rep, n_tot, n_tiles;
     int n_max;         // atoms of the largest replica
     int g;             // lanes per atom in the pair passes
-    int sms;           // SMs of the device
+    int sms;           // SMs of the device, and the most shared memory one of its blocks may have
+    int smem_optin;
     const RepDev* rep;
     const int* tile_rep;
     double* x;
@@ -145,8 +148,11 @@ struct DevBatch {
     int* craw;         // atoms by cell, unsorted inside a cell (list build)
     int* cstart;
     int* ccount;       // atoms per cell; zero between list builds
-    double* partA;     // [NPA][pair blocks]
-    double* partB;     // [NPB][n_tiles]
+    double* partA;     // [NPA][pair blocks], float2 (hi, lo) on the mixed path
+    double* partB;     // [NPB][n_tiles], likewise
+    double* partG;     // [NPA + NPB][n_grp] sums over groups of tiles
+    int n_grp;
+    unsigned* grp_done;
     double* tot;
     unsigned* tile_done;
     unsigned* nl_done;
@@ -304,10 +310,12 @@ __device__ __forceinline__ dff dff_warp_sum(dff v)
 }
 
 // Sum of nt consecutive partials, by one warp: lane l adds entries l, l + 32,
-// ... in four interleaved chains (a serial FP64 chain's latency was the cost
-// on a 65,536-atom replica), then a fixed xor-shuffle tree; every lane returns
-// the total, and the order depends only on nt, never on scheduling.  Called by
-// all 32 lanes.
+// ... in four interleaved chains, then a fixed xor-shuffle tree; every lane
+// returns the total, and the order depends only on nt, never on scheduling.
+// Called by all 32 lanes.  Partials are doubles on the FP64 path and
+// double-float pairs, sixteen loads in flight, on the mixed one (serial FP64
+// adds of a 65,536-atom replica's 2048 partials, 15 quantities in the one
+// finishing block, cost 13 us).
 __device__ __forceinline__ double ne_warp_part_sum(const double* part, int nt)
 {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -319,6 +327,46 @@ __device__ __forceinline__ double ne_warp_part_sum(const double* part, int nt)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
+}
+
+__device__ __forceinline__ float2 ne_warp_part_sum_e(const float2* part, int nt)
+{
+    dff acc[4] = {};
+    for (int t = threadIdx.x & 31; t < nt; t += 512) {
+        float2 v[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) v[c] = t + 32 * c < nt ? __ldcg(&part[t + 32 * c]) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+            if (t + 32 * c < nt) acc[c & 3] = dff_add(acc[c & 3], {v[c].x, v[c].y});
+    }
+    const dff s = dff_warp_sum(dff_add(dff_add(acc[0], acc[1]), dff_add(acc[2], acc[3])));
+    return make_float2(s.hi, s.lo);
+}
+
+__device__ __forceinline__ double ne_warp_part_sum_e(const double* part, int nt) { return ne_warp_part_sum(part, nt); }
+
+__device__ __forceinline__ double ne_warp_part_sum(const float2* part, int nt)
+{
+    const float2 s = ne_warp_part_sum_e(part, nt);
+    return (double)s.x + (double)s.y;
+}
+
+// nt partials from entry `at` of a partials array of either kind
+__device__ __forceinline__ double ne_warp_part_sum(const DevBatch& B, const double* part, size_t at, int nt)
+{
+    return B.pos64 ? ne_warp_part_sum(part + at, nt) : ne_warp_part_sum((const float2*)part + at, nt);
+}
+
+// One more on a ticket, after this thread's earlier writes (and, behind a
+// barrier, its block's); returns the count before.  A release only:
+// __threadfence also drops the SM's L1, which the blocks next to a finishing
+// one pay for.
+__device__ __forceinline__ unsigned ne_ticket(unsigned* p)
+{
+    unsigned old;
+    asm volatile("atom.release.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+    return old;
 }
 
 __device__ __forceinline__ void ne_set_status(int* status, int bits)
@@ -352,14 +400,12 @@ void launch_msd_sample(const DevBatch& B, double* acc, cudaStream_t st);
 // gE, or with gw != nullptr the per-step weight gw[*ctr + j - s_off] read on
 // the device (runs replayed from graphs); set_attr: set the kernel's shared-
 // memory attribute (not inside a stream capture)
-size_t backward_block_bytes(int nk);  // one mixed backward block's bins (device and shared memory)
-size_t backward_bins_bytes(int nk, int n_blocks);  // the whole bins buffer: F's (zeroed once), then the blocks'
-bool backward_fits(int nk);           // those bins fit one block's shared memory
+size_t backward_bins_bytes(int nk);   // the mixed backward's global bins, zero between launches
+bool backward_fits(int nk);           // a block's low words fit its shared memory
 void launch_backward(const DevBatch& B, bool mixed, double gE, double* gtheta,
-                     float* bins, int n_bin_blocks, bool accumulate, cudaStream_t st,
+                     unsigned long long* bins, bool accumulate, cudaStream_t st,
                      const double* gw = nullptr, const long long* ctr = nullptr, int j = 0,
                      long long s_off = 0, bool set_attr = true);
-int backward_bin_blocks(const DevBatch& B);
 cudaError_t prepare_backward(const DevBatch& B);  // the mixed backward kernel's shared-memory attribute
 void launch_virial(const DevBatch& B, double* out, cudaStream_t st);
 }  // namespace ne

@@ -282,14 +282,18 @@ __global__ void __launch_bounds__(STEP_THREADS)
     if constexpr (MIXED) {
         if (threadIdx.x < 15 && threadIdx.x / 3 < nq) {
             const int k = threadIdx.x / 3, d = threadIdx.x % 3;
+            float2* const pf = (float2*)B.partB + tile;
             dff t = dff_add({s_dff[k][2 * d].x, s_dff[k][2 * d].y}, {s_dff[k][2 * d + 1].x, s_dff[k][2 * d + 1].y});
             if (k == 0 || k == 2) {
-                pbt[((k == 0 ? PB_UX : PB_XIX) + d) * np] = (double)t.hi + (double)t.lo;
+                pf[((k == 0 ? PB_UX : PB_XIX) + d) * np] = make_float2(t.hi, t.lo);
             } else if (d == 0 && (k != 3 || P.nsp)) {
                 for (int w2 = 2; w2 < 6; ++w2) t = dff_add(t, {s_dff[k][w2].x, s_dff[k][w2].y});
-                const double tot = (double)t.hi + (double)t.lo;
-                pbt[(k == 1 ? PB_U2 : (k == 3 ? PB_UE : PB_KE)) * np] = tot;
-                if (k == 1 && !P.nsp) pbt[PB_UE * np] = 0.5 * P.k * tot;
+                pf[(k == 1 ? PB_U2 : (k == 3 ? PB_UE : PB_KE)) * np] = make_float2(t.hi, t.lo);
+                if (k == 1 && !P.nsp) {
+                    const double ue = 0.5 * P.k * ((double)t.hi + (double)t.lo);
+                    const float h = (float)ue;
+                    pf[PB_UE * np] = make_float2(h, (float)(ue - (double)h));
+                }
             }
         }
     } else if (threadIdx.x < 128) {
@@ -356,7 +360,7 @@ __global__ void k_trace_T(DevBatch B, const long long* __restrict__ step_base, i
     const long long s = *step_base + j;
     if (!B.trace || s % B.trace_stride != 0 || s / B.trace_stride >= B.trace_rows) return;
     const RepDev& P = B.rep[0];
-    const double ke = ne_warp_part_sum(B.partB + (size_t)PB_KE * B.n_tiles + P.tile0, P.ntile);
+    const double ke = ne_warp_part_sum(B, B.partB, (size_t)PB_KE * B.n_tiles + P.tile0, P.ntile);
     const double kB = 8.617333262e-5;
     if (threadIdx.x == 0) B.trace[8 * (s / B.trace_stride) + 5] = 2.0 * ke / (P.dof * kB);
 }
@@ -520,10 +524,10 @@ __global__ void k_msd_sample(DevBatch B, double* acc)
     const int rep = blockIdx.x;
     const RepDev& P = B.rep[rep];
     double s[4];
-    s[0] = ne_warp_part_sum(B.partB + (size_t)PB_UX * B.n_tiles + P.tile0, P.ntile);
-    s[1] = ne_warp_part_sum(B.partB + (size_t)PB_UY * B.n_tiles + P.tile0, P.ntile);
-    s[2] = ne_warp_part_sum(B.partB + (size_t)PB_UZ * B.n_tiles + P.tile0, P.ntile);
-    s[3] = ne_warp_part_sum(B.partB + (size_t)PB_U2 * B.n_tiles + P.tile0, P.ntile);
+    s[0] = ne_warp_part_sum(B, B.partB, (size_t)PB_UX * B.n_tiles + P.tile0, P.ntile);
+    s[1] = ne_warp_part_sum(B, B.partB, (size_t)PB_UY * B.n_tiles + P.tile0, P.ntile);
+    s[2] = ne_warp_part_sum(B, B.partB, (size_t)PB_UZ * B.n_tiles + P.tile0, P.ntile);
+    s[3] = ne_warp_part_sum(B, B.partB, (size_t)PB_U2 * B.n_tiles + P.tile0, P.ntile);
     if (threadIdx.x != 0) return;
     const double invN = 1.0 / P.n;
     acc[rep] += s[3] * invN - (s[0] * s[0] + s[1] * s[1] + s[2] * s[2]) * invN * invN;
