@@ -257,8 +257,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     const int n_tot = off[n_rep];
     if (n_tot > ctx->max_atoms) return fail(ctx, NE_ENOMEM, "atom count exceeds the context");
     ctx->rep_h.assign(n_rep, RepDev{});
-    ctx->tile_rep_h.clear();
-    int cells = 0, npt_any = 0, groups = 0;
+    int cells = 0, npt_any = 0, groups = 0, n_tiles = 0;
     const double rc = ctx->eam.r_c;
     for (int r = 0; r < n_rep; ++r) {
         const ne_md_params& m = md[(size_t)r * md_stride];
@@ -300,11 +299,11 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
         R.half_skin2 = (float)(0.25 * skin * skin);
         R.off = off[r];
         R.n = n;
-        R.tile0 = (int)ctx->tile_rep_h.size();
+        R.tile0 = n_tiles;
         R.ntile = (n + NE_TILE - 1) / NE_TILE;
         R.grp0 = groups;
         groups += (R.ntile + GROUP_TILES - 1) / GROUP_TILES;
-        for (int t = 0; t < R.ntile; ++t) ctx->tile_rep_h.push_back(r);
+        n_tiles += R.ntile;
         R.cell_off = cells;
         cells += R.nc[0] * R.nc[1] * R.nc[2];
         R.dof = m.fix_cm ? 3 * n - 3 : 3 * n;
@@ -327,16 +326,22 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     ctx->boxes_from_runner = false;
     int species_all = 1;
     for (int r = 0; r < n_rep; ++r) species_all &= ctx->rep_h[r].nsp >= 2;
-    const int n_tiles = (int)ctx->tile_rep_h.size();
     if (n_tiles > ctx->tiles_cap) return fail(ctx, NE_ENOMEM, "tile capacity exceeded");
     if (cells > ctx->cells_cap) return fail(ctx, NE_ENOMEM, "cell capacity exceeded");
-    NE_CU(cudaMemcpyAsync(ctx->rep, ctx->rep_h.data(), sizeof(RepDev) * n_rep, cudaMemcpyHostToDevice, st));
-    NE_CU(cudaMemcpyAsync(ctx->tile_rep, ctx->tile_rep_h.data(), sizeof(int) * n_tiles,
-                          cudaMemcpyHostToDevice, st));
-    NE_CU(cudaMemsetAsync(ctx->tile_done, 0, sizeof(unsigned) * n_rep, st));
-    NE_CU(cudaMemsetAsync(ctx->flags, 0, sizeof(int) * n_rep, st));
-    NE_CU(cudaMemsetAsync(ctx->status, 0, sizeof(int), st));
-    NE_CU(cudaMemsetAsync(ctx->tot, 0, sizeof(double) * NTOT * n_rep, st));
+    if (n_rep <= ne::SETUP_MAX) {
+        ne::launch_setup(ctx->rep_h.data(), n_rep, ctx->rep, ctx->tile_rep, ctx->tile_done, ctx->flags, ctx->status,
+                         ctx->tot, st);
+    } else {
+        ctx->tile_rep_h.clear();
+        for (int r = 0; r < n_rep; ++r) ctx->tile_rep_h.insert(ctx->tile_rep_h.end(), ctx->rep_h[r].ntile, r);
+        NE_CU(cudaMemcpyAsync(ctx->rep, ctx->rep_h.data(), sizeof(RepDev) * n_rep, cudaMemcpyHostToDevice, st));
+        NE_CU(cudaMemcpyAsync(ctx->tile_rep, ctx->tile_rep_h.data(), sizeof(int) * n_tiles,
+                              cudaMemcpyHostToDevice, st));
+        NE_CU(cudaMemsetAsync(ctx->tile_done, 0, sizeof(unsigned) * n_rep, st));
+        NE_CU(cudaMemsetAsync(ctx->flags, 0, sizeof(int) * n_rep, st));
+        NE_CU(cudaMemsetAsync(ctx->status, 0, sizeof(int), st));
+        NE_CU(cudaMemsetAsync(ctx->tot, 0, sizeof(double) * NTOT * n_rep, st));
+    }
     B = DevBatch{};
     B.n_rep = n_rep;
     B.n_tot = n_tot;
@@ -397,10 +402,10 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
 ne_status finish(ne_ctx* ctx, cudaStream_t st)
 {
     NE_CU(cudaGetLastError());
-    // the status word lands in pinned host memory: the copy is a plain DMA
-    NE_CU(cudaMemcpyAsync(ctx->status_host, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    // the status word goes straight to pinned host memory
+    ne::launch_status_out(ctx->status, ctx->status_host, st);
     NE_CU(cudaStreamSynchronize(st));
-    const int bits = *ctx->status_host;
+    const int bits = *(volatile int*)ctx->status_host;
     ctx->last_bits = bits;
     if (bits & ST_ENAN) return fail(ctx, NE_ENAN, "non-finite position, velocity or energy");
     if (bits & ST_ERANGE) return fail(ctx, NE_ERANGE, "pair distance below 0.2 A, density >= rho_max, or an atom beyond the crystal runner's stencil range");
@@ -472,8 +477,7 @@ ne_status run_steps(ne_ctx* ctx, DevBatch& B, const Sched& S, bool mixed, long l
                     long long msd_from = 0, int msd_stride = 0, const GradAcc* ga = nullptr)
 {
     long long* ctr = ctx->step_ctr;
-    NE_CU(cudaMemcpyAsync(ctr, &s_begin, sizeof(long long), cudaMemcpyHostToDevice, st));
-    NE_CU(cudaStreamSynchronize(st));
+    ne::launch_set_step(ctr, s_begin, st);
     ne_status ls = run_lambda(ctx, B, S, s_begin, n_steps, st);
     if (ls) return ls;
     // list from the lattice sites (from the positions when a barostat may
@@ -552,8 +556,7 @@ ne_status profile_steps(ne_ctx* ctx, DevBatch& B, const Sched& S, bool mixed, lo
                         long long n_steps, double* ms, long long* counts, cudaStream_t st)
 {
     long long* ctr = ctx->step_ctr;
-    NE_CU(cudaMemcpyAsync(ctr, &s_begin, sizeof(long long), cudaMemcpyHostToDevice, st));
-    NE_CU(cudaStreamSynchronize(st));
+    ne::launch_set_step(ctr, s_begin, st);
     ne_status ls = run_lambda(ctx, B, S, s_begin, n_steps, st);
     if (ls) return ls;
     ne::launch_nl_build(B, 1, 1, st);
