@@ -277,7 +277,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
             R.invL[d] = 1.0 / R.L[d];
             R.Lf[d] = (float)R.L[d];
             R.iLf[d] = (float)R.invL[d];
-            R.nc[d] = geometry ? (int)std::min(std::floor(shrink * R.L[d] / rl), 1024.0) : 0;
+            // (the margin covers the FP32 binning)
+            R.nc[d] = geometry ? (int)std::min(std::floor(shrink * R.L[d] / (rl + 1e-3)), 1024.0) : 0;
         }
         // cells of edge >= r_c + skin; fewer (larger) cells when the box is
         // sparse, so the cell count stays below 2n + 27
@@ -999,7 +1000,7 @@ ne_status ne_eam_energy_forces(ne_ctx* ctx, ne_precision prec, const double* x_d
     ne::launch_nl_build(B, 1, 0, st);
     ne::launch_pass1(B, mixed, st);
     ne::launch_pass2(B, mixed, st);
-    ne::launch_export(B, mixed, f_dev, e_dev, st);
+    ne::launch_export(B, mixed, f_dev, e_dev, 1.0, st);
     return finish(ctx, st);
 }
 
@@ -1072,7 +1073,7 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
     ne::launch_nl_build(B, 1, 0, st);
     ne::launch_pass1(B, mixed, st);
     ne::launch_pass2(B, mixed, st);
-    if (gx_dev) ne::launch_export(B, mixed, gx_dev, nullptr, st);
+    if (gx_dev) ne::launch_export(B, mixed, gx_dev, nullptr, -gE, st);  // dU/dx = -F times gE
     if (mixed && !ne::backward_fits(ctx->eam.n_knots))
         return fail(ctx, NE_EINVAL, "mixed backward: n_knots too large for one block's shared-memory bins");
     if (mixed) {
@@ -1080,7 +1081,6 @@ static ne_status backward_impl(ne_ctx* ctx, ne_precision prec, const double* x_d
         if (s) return s;
     }
     ne::launch_backward(B, mixed, gE, gtheta_dev, ctx->bins, accumulate, st);
-    if (gx_dev) ne::launch_scale(gx_dev, 3 * n, -gE, st);  // dU/dx = -F times gE
     return finish(ctx, st);
 }
 
@@ -2153,13 +2153,3 @@ ne_status ne_rs_free_energy(int n, double T0, double F0_T0, double lambda_f, lon
 }
 
 }  // extern "C"
-
-// dU/dx = -F scaled by the upstream gradient (used by ne_eam_backward).
-__global__ void k_scale(double* p, int n, double s)
-{
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) p[q] *= s;
-}
-
-namespace ne {
-void launch_scale(double* p, int n, double s, cudaStream_t st) { k_scale<<<64, 256, 0, st>>>(p, n, s); }
-}  // namespace ne

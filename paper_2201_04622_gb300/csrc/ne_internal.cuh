@@ -397,11 +397,10 @@ void launch_set_step(long long* step_base, long long s, cudaStream_t st);
 void launch_advance(long long* step_base, long long by, cudaStream_t st);
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,
                   double* z, cudaStream_t st);
-void launch_scale(double* p, int n, double s, cudaStream_t st);
 void launch_init_velocities(const DevBatch& B, int fix_cm, cudaStream_t st);
 void launch_spring(const double* x, const double* x0, int n, double k, double* f, double* e,
                    double* scratch, cudaStream_t st);
-void launch_export(const DevBatch& B, bool mixed, double* f_out, double* e_out, cudaStream_t st);
+void launch_export(const DevBatch& B, bool mixed, double* f_out, double* e_out, double scale, cudaStream_t st);
 void launch_msd_sample(const DevBatch& B, double* acc, cudaStream_t st);
 // gE, or with gw != nullptr the per-step weight gw[*ctr + j - s_off] read on
 // the device (runs replayed from graphs); set_attr: set the kernel's shared-

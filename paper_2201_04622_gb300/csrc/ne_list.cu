@@ -5,7 +5,7 @@
 // nothing to do:
 //   k_nl_cells  reference positions (the lattice sites at the start of a run,
 //               the current positions after an atom strayed more than
-//               skin / 2), wrapped and binned into cells of edge >= r_c + skin.
+//               skin / 2), wrapped and binned into cells of edge > r_c + skin.
 //               One thread per atom over all SMs; the block that finishes a
 //               replica's last tile forms its cell starts and writes the atoms
 //               sorted by cell, each cell's by index, so the order does not
@@ -14,11 +14,11 @@
 //               when the box holds < 3 cells per axis) within r_c + skin,
 //               minimum image, FP32 distances with a 1e-3 A margin so that
 //               rounding never drops a pair.
+#include <type_traits>
+
 #include "ne_internal.cuh"
 
 namespace {
-
-__device__ __forceinline__ double wrap(double x, double L, double invL) { return x - L * floor(x * invL); }
 
 constexpr int CELL_THREADS = 1024;
 constexpr int CELL_TILES = CELL_THREADS / NE_TILE;
@@ -51,7 +51,7 @@ __device__ __forceinline__ void rank_cells(const DevBatch& B, int rep, int first
 // Cell starts and the atoms by cell (and, for a replica that one block sorts,
 // the sorted copy) of one replica whose atoms are all counted, by the whole
 // block.
-__device__ void sort_cells(const DevBatch& B, int rep, int* s_warp)
+__device__ void sort_cells(const DevBatch& B, int rep, bool scatter, int* s_warp)
 {
     const RepDev& P = B.rep[rep];
     const int tid = threadIdx.x, n = P.n, off = P.off;
@@ -90,6 +90,7 @@ __device__ void sort_cells(const DevBatch& B, int rep, int* s_warp)
         count[c] = 0;  // zero for the next build
     }
     if (tid == 0) start[ncell] = n;
+    if (!scatter) return;
     __syncthreads();
     for (int a0 = tid; a0 < n; a0 += 8 * CELL_THREADS) {
         int c[8], k[8];  // eight atoms in flight: the chain is cell -> start -> store
@@ -113,9 +114,11 @@ __device__ void sort_cells(const DevBatch& B, int rep, int* s_warp)
 // then the finishing block scans and scatters its replica's atoms.  Before, one
 // 512-thread block counted, scanned and sorted each cell by insertion (176 us
 // for 65,536 atoms, 40 us for 2000) and one thread an atom walked its cells
-// (176 and 253 us).  Whole calls, before and now: energy and forces of 70,304
-// atoms in FP64 1232 -> 973 us, energy and gradients of 65,536 atoms 1504 ->
-// 1091 us, the 200-step spring fit of 2000 atoms at 1400 K 17.0 -> 13.6 ms.
+// (176 and 253 us).  Whole calls, before and with this build: energy and forces of
+// 70,304 atoms in FP64 1232 -> 973 us, energy and gradients of 65,536 atoms 1504
+// -> 1091 us, the 200-step spring fit of 2000 atoms at 1400 K 17.0 -> 13.6 ms.
+// The image index and the cell in FP32 (the cells are 1e-3 A wider than r_c +
+// skin) took another 8 us of FP64 out.
 __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force, int from_sites)
 {
     __shared__ int s_warp[32];
@@ -130,9 +133,20 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
     if (go && a < P.n) {
         const int i = P.off + a;
         const double* X = from_sites ? B.x0 : B.x;
+        // image index in FP32, the shift, only for an atom outside the box, in
+        // FP64 (as the step kernel)
         double w[3];
-        for (int d = 0; d < 3; ++d) w[d] = wrap(X[3 * i + d], P.L[d], P.invL[d]);
-        const float4 p = make_float4((float)w[0], (float)w[1], (float)w[2], __int_as_float(a));
+        float wf[3];
+        for (int d = 0; d < 3; ++d) {
+            w[d] = X[3 * i + d];
+            wf[d] = (float)w[d];
+            const float n = floorf(wf[d] * P.iLf[d]);
+            if (n != 0.f) {
+                w[d] -= P.L[d] * (double)n;
+                wf[d] = (float)w[d];
+            }
+        }
+        const float4 p = make_float4(wf[0], wf[1], wf[2], __int_as_float(a));
         B.pbuild[i] = p;
         if (!from_sites) {  // what the pair passes read
             B.pos32[i] = make_float4(p.x, p.y, p.z, __int_as_float(0));
@@ -143,7 +157,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
         } else {
             int c3[3];
             for (int d = 0; d < 3; ++d) {
-                const int q = (int)(w[d] * P.invL[d] * P.nc[d]);
+                const int q = (int)(wf[d] * P.iLf[d] * (float)P.nc[d]);
                 c3[d] = min(max(q, 0), P.nc[d] - 1);
             }
             const int c = (c3[0] * P.nc[1] + c3[1]) * P.nc[2] + c3[2];
@@ -169,9 +183,23 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
     }
     __syncthreads();
     for (int q = 0; q < CELL_TILES; ++q) {
-        if (s_done[q] >= 0) sort_cells(B, s_done[q], s_warp);
+        if (s_done[q] >= 0) sort_cells(B, s_done[q], !(force && B.rep[s_done[q]].n > SORT_IN_BLOCK), s_warp);
         __syncthreads();
     }
+}
+
+// the scatter of a forced build of large replicas (the finishing block's own
+// takes ~20 us at 65,536 atoms; inside a run, where builds are rare, the launch
+// would cost every step)
+__global__ void __launch_bounds__(256) k_nl_scatter(DevBatch B)
+{
+    const int tile = blockIdx.x * (256 / NE_TILE) + threadIdx.x / NE_TILE;
+    if (tile >= B.n_tiles) return;
+    const int rep = B.tile_rep[tile];
+    const RepDev& P = B.rep[rep];
+    const int a = (tile - P.tile0) * NE_TILE + threadIdx.x % NE_TILE;
+    if (P.nc[0] == 0 || P.n <= SORT_IN_BLOCK || a >= P.n) return;
+    B.craw[P.off + (B.cstart + P.cell_off + rep)[B.cellof[P.off + a]] + B.cslot[P.off + a]] = a;
 }
 
 __global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
@@ -186,7 +214,10 @@ __global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
 
 // G lanes per atom walk its 27 cells: the z neighbours of a cell are one run
 // of the sorted copy (two at the box edge), so the lanes read consecutive
-// 16-byte entries, and a ballot packs the lanes' hits in order.
+// 16-byte entries, and a ballot packs the lanes' hits in order.  Bound by
+// instructions (72 % issue): a run's image is known from its cells, so a
+// candidate is three differences and a test, without a nearest-image rounding
+// (20 replicas with a 2.6 A skin, ~2000 candidates an atom: 191 -> 123 us).
 constexpr int LIST_THREADS = 256;
 
 template <int G>
@@ -211,22 +242,25 @@ __device__ void list_block(const DevBatch& B, int blk)
     const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     int cnt = 0;
     // entries [lo, hi) of the sorted copy (empty for a lane group with no atom)
-    auto scan = [&](int lo, int hi) {
+    // that lie `code` box lengths off; ALL: each at its nearest image instead
+    auto scan = [&](auto all, int lo, int hi, int code, float px, float py, float pz) {
         const int trips = __reduce_max_sync(0xffffffffu, (unsigned)(hi > lo ? (hi - lo + G - 1) / G : 0));
         for (int t = 0; t < trips; ++t) {
             const int p = lo + t * G + lane;
             bool hit = false;
-            int b = 0, code = 0;
+            int b = 0;
             if (p < hi) {
                 const float4 pj = B.csort[off + p];
                 b = __float_as_int(pj.w);
-                float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-                const float n0 = rintf(dx * iL0), n1 = rintf(dy * iL1), n2 = rintf(dz * iL2);
-                dx -= L0 * n0;
-                dy -= L1 * n1;
-                dz -= L2 * n2;
-                code = NE_IMG_NONE - (int)(9.f * n0 + 3.f * n1 + n2);
-                hit = b != a && dx * dx + dy * dy + dz * dz < rl2;
+                float dx = pj.x - px, dy = pj.y - py, dz = pj.z - pz;
+                if constexpr (all.value) {
+                    const float n0 = rintf(dx * iL0), n1 = rintf(dy * iL1), n2 = rintf(dz * iL2);
+                    dx -= L0 * n0;
+                    dy -= L1 * n1;
+                    dz -= L2 * n2;
+                    code = NE_IMG_NONE - (int)(9.f * n0 + 3.f * n1 + n2);
+                }
+                hit = dx * dx + dy * dy + dz * dz < rl2 && b != a;
             }
             const unsigned m = (__ballot_sync(0xffffffffu, hit) >> gsh) & gmask;
             const int at = cnt + __popc(m & ((1u << lane) - 1u));
@@ -235,23 +269,30 @@ __device__ void list_block(const DevBatch& B, int blk)
         }
     };
     if (P.nc[0] == 0) {
-        scan(0, valid ? P.n : 0);
+        scan(std::true_type(), 0, valid ? P.n : 0, 0, pi.x, pi.y, pi.z);
     } else {
         const int nc0 = P.nc[0], nc1 = P.nc[1], nc2 = P.nc[2];
         const int* start = B.cstart + P.cell_off + rep;
         const int c = valid ? B.cellof[i] : 0;
         const int cx = c / (nc1 * nc2), cy = (c / nc2) % nc1, cz = c % nc2;
-        // z cells cz - 1 .. cz + 1 in order: [z0, z1) and, across the edge, [z2, z3)
-        int z0 = cz - 1, z1 = cz + 2, z2 = 0, z3 = 0;
-        if (cz == 0) z0 = nc2 - 1, z1 = nc2, z3 = 2;
-        if (cz == nc2 - 1) z1 = nc2, z3 = 1;
+        // z cells cz - 1 .. cz + 1 in order: [z0, z1) and, across the edge,
+        // [z2, z3); the image of each run is that of its cells
+        int z0 = cz - 1, z1 = cz + 2, z3 = 0, sz0 = 0, sz1 = 0;
+        if (cz == 0) z0 = nc2 - 1, z1 = nc2, z3 = 2, sz0 = -1;
+        if (cz == nc2 - 1) z1 = nc2, z3 = 1, sz1 = 1;
 #pragma unroll 1
         for (int r = 0; r < 9; ++r) {
-            const int o = (((cx + r / 3 - 1 + nc0) % nc0) * nc1 + (cy + r % 3 - 1 + nc1) % nc1) * nc2;
-            scan(valid ? start[o + z0] : 0, valid ? start[o + z1] : 0);
+            const int x = cx + r / 3 - 1, y = cy + r % 3 - 1;
+            const int sx = x < 0 ? -1 : (x >= nc0 ? 1 : 0), sy = y < 0 ? -1 : (y >= nc1 ? 1 : 0);
+            const int o = ((x - sx * nc0) * nc1 + y - sy * nc1) * nc2;
+            const int code = NE_IMG_NONE + 9 * sx + 3 * sy;
+            const float px = pi.x - (float)sx * L0, py = pi.y - (float)sy * L1;
+            scan(std::false_type(), valid ? start[o + z0] : 0, valid ? start[o + z1] : 0, code + sz0, px, py,
+                 pi.z - (float)sz0 * L2);
             if (__any_sync(0xffffffffu, z3 > 0)) {
                 const bool two = valid && z3 > 0;
-                scan(two ? start[o + z2] : 0, two ? start[o + z3] : 0);
+                scan(std::false_type(), two ? start[o] : 0, two ? start[o + z3] : 0, code + sz1, px, py,
+                     pi.z - (float)sz1 * L2);
             }
         }
     }
@@ -277,6 +318,8 @@ void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t 
 {
     k_nl_cells<<<(B.n_tiles + CELL_TILES - 1) / CELL_TILES, CELL_THREADS, 0, st>>>(B, force, from_sites);
     const auto grid = [&](int want) { return want < 6 * B.sms ? want : 6 * B.sms; };
+    if (force && B.n_max > SORT_IN_BLOCK)
+        k_nl_scatter<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
     if (B.n_max > SORT_IN_BLOCK)
         k_nl_sort<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
     // a warp an atom up to 8192 atoms (a quarter of a million threads, one

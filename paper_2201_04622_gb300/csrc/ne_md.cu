@@ -523,26 +523,16 @@ __global__ void __launch_bounds__(1024) k_spring(const double* __restrict__ x, c
     if (threadIdx.x == 0 && e) *e = red[0];
 }
 
-// EAM forces and energy of replica 0 to caller buffers.
+// EAM forces, times scale, and energy of replica 0 to caller buffers.
 template <bool MIXED>
-__global__ void k_export(DevBatch B, double* f, double* e)
+__global__ void k_export(DevBatch B, double* f, double* e, double scale)
 {
     const RepDev& P = B.rep[0];
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < P.n; a += gridDim.x * blockDim.x) {
-        const int i = P.off + a;
-        if (f) {
-            if constexpr (MIXED) {
-                float4 g = B.f32[i];
-                f[3 * a] = g.x;
-                f[3 * a + 1] = g.y;
-                f[3 * a + 2] = g.z;
-            } else {
-                f[3 * a] = B.f64[3 * i];
-                f[3 * a + 1] = B.f64[3 * i + 1];
-                f[3 * a + 2] = B.f64[3 * i + 2];
-            }
+    if (f)
+        for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < 3 * P.n; q += gridDim.x * blockDim.x) {
+            const size_t i = (size_t)P.off + q / 3;
+            f[q] = scale * (MIXED ? (double)((const float*)B.f32)[4 * i + q % 3] : B.f64[3 * i + q % 3]);
         }
-    }
     if (blockIdx.x == 0 && threadIdx.x == 0 && e) *e = B.tot[TOT_UEMB] + B.tot[TOT_UPAIR];
 }
 
@@ -665,12 +655,13 @@ void launch_spring(const double* x, const double* x0, int n, double k, double* f
     k_spring<<<1, 1024, 0, st>>>(x, x0, n, k, f, e);
 }
 
-void launch_export(const DevBatch& B, bool mixed, double* f_out, double* e_out, cudaStream_t st)
+void launch_export(const DevBatch& B, bool mixed, double* f_out, double* e_out, double scale, cudaStream_t st)
 {
+    const int want = f_out ? (3 * B.n_tot + 255) / 256 : 1, grid = want < 4 * B.sms ? want : 4 * B.sms;
     if (mixed)
-        k_export<true><<<64, 256, 0, st>>>(B, f_out, e_out);
+        k_export<true><<<grid, 256, 0, st>>>(B, f_out, e_out, scale);
     else
-        k_export<false><<<64, 256, 0, st>>>(B, f_out, e_out);
+        k_export<false><<<grid, 256, 0, st>>>(B, f_out, e_out, scale);
 }
 
 void launch_msd_sample(const DevBatch& B, double* acc, cudaStream_t st)

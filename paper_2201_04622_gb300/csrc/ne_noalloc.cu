@@ -164,7 +164,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
         R.invL[d] = 1.0 / box[d];
         R.Lf[d] = (float)R.L[d];
         R.iLf[d] = (float)R.invL[d];
-        R.nc[d] = (int)std::min(std::floor(box[d] / rc), 1024.0);
+        R.nc[d] = (int)std::min(std::floor(box[d] / (rc + 1e-3)), 1024.0);  // the margin covers the FP32 binning
     }
     while ((long long)R.nc[0] * R.nc[1] * R.nc[2] > 2ll * n + 27) {
         int d = R.nc[0] >= R.nc[1] && R.nc[0] >= R.nc[2] ? 0 : (R.nc[1] >= R.nc[2] ? 1 : 2);
@@ -260,7 +260,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     ne::launch_nl_build(B, 1, 0, st);
     ne::launch_pass1(B, mixed, st);
     ne::launch_pass2(B, mixed, st);
-    ne::launch_export(B, mixed, f_dev, e_dev, st);
+    ne::launch_export(B, mixed, f_dev, e_dev, 1.0, st);
     if (cudaGetLastError() != cudaSuccess) return NE_ECUDA;
     int bits = 0;
     if (cudaMemcpyAsync(&bits, B.status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
