@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
 {
     __shared__ int s_warp[32];
     __shared__ int s_done[CELL_TILES];  // replica whose last tile this block finished, or -1
+    ne_chain();
     const int tl = threadIdx.x / NE_TILE;
     const int tile = blockIdx.x * CELL_TILES + tl;
     const int rep = tile < B.n_tiles ? B.tile_rep[tile] : 0;
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
 // would cost every step)
 __global__ void __launch_bounds__(256) k_nl_scatter(DevBatch B)
 {
+    ne_chain();
     const int tile = blockIdx.x * (256 / NE_TILE) + threadIdx.x / NE_TILE;
     if (tile >= B.n_tiles) return;
     const int rep = B.tile_rep[tile];
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(256) k_nl_scatter(DevBatch B)
 
 __global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
 {
+    ne_chain();
     const int tile = blockIdx.x * (256 / NE_TILE) + threadIdx.x / NE_TILE;
     if (tile >= B.n_tiles) return;
     const int rep = B.tile_rep[tile];
@@ -307,6 +310,7 @@ __device__ void list_block(const DevBatch& B, int blk)
 template <int G>
 __global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
 {
+    ne_chain();
     for (int blk = blockIdx.x; blk < B.n_tiles * (NE_TILE * G / LIST_THREADS); blk += gridDim.x) list_block<G>(B, blk);
 }
 
@@ -316,18 +320,18 @@ namespace ne {
 
 void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t st)
 {
-    k_nl_cells<<<(B.n_tiles + CELL_TILES - 1) / CELL_TILES, CELL_THREADS, 0, st>>>(B, force, from_sites);
+    ne_launch(k_nl_cells, (B.n_tiles + CELL_TILES - 1) / CELL_TILES, CELL_THREADS, 0, st, B, force, from_sites);
     const auto grid = [&](int want) { return want < 6 * B.sms ? want : 6 * B.sms; };
     if (force && B.n_max > SORT_IN_BLOCK)
-        k_nl_scatter<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
+        ne_launch(k_nl_scatter, (B.n_tiles + 3) / 4, 256, 0, st, B);
     if (B.n_max > SORT_IN_BLOCK)
-        k_nl_sort<<<(B.n_tiles + 3) / 4, 256, 0, st>>>(B);
+        ne_launch(k_nl_sort, (B.n_tiles + 3) / 4, 256, 0, st, B);
     // a warp an atom up to 8192 atoms (a quarter of a million threads, one
     // wave), eight lanes above: fewer idle lanes at the ends of the short runs
     if (B.n_tot <= 8192)
-        k_nl_list<32><<<grid(B.n_tiles * (NE_TILE * 32 / LIST_THREADS)), LIST_THREADS, 0, st>>>(B);
+        ne_launch(k_nl_list<32>, grid(B.n_tiles * (NE_TILE * 32 / LIST_THREADS)), LIST_THREADS, 0, st, B);
     else
-        k_nl_list<8><<<grid(B.n_tiles * (NE_TILE * 8 / LIST_THREADS)), LIST_THREADS, 0, st>>>(B);
+        ne_launch(k_nl_list<8>, grid(B.n_tiles * (NE_TILE * 8 / LIST_THREADS)), LIST_THREADS, 0, st, B);
 }
 
 }  // namespace ne

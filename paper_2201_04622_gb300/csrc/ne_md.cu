@@ -143,6 +143,15 @@ __global__ void __launch_bounds__(STEP_THREADS)
     const long long s = *step_base + j;
     const double* T = B.tot + (size_t)rep * NTOT;
     const bool draw = do_open || !do_close;  // a step follows: its normals
+    // the normals of the coming step, which depend on nothing that a kernel of
+    // the chain writes, while pass 2 drains
+    R z = 0;
+    if (valid && draw) {
+        const uint4 ph = ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
+                                         (unsigned long long)(do_open ? s + 1 : s));
+        z = MIXED ? (R)ne_normal32(ph, c) : (R)ne_normal64(ph, c);
+    }
+    ne_chain();
     if (threadIdx.x < 32) {
         // lanes 0-8: mean F0, the spring's mean and the noise mean (per unit
         // mass with species tables: the mass-weighted constraint); 9-11 the
@@ -246,9 +255,6 @@ __global__ void __launch_bounds__(STEP_THREADS)
         s_d2[c][al] = d * d;
         s_code[c][al] = (int)nb;
         if (draw) {
-            const uint4 ph = ne_philox_block(P.seed, P.replica, (unsigned)S.stream, (unsigned)a,
-                                             (unsigned long long)(do_open ? s + 1 : s));
-            const R z = MIXED ? (R)ne_normal32(ph, c) : (R)ne_normal64(ph, c);
             if constexpr (MIXED) B.xi32[e] = z;
             else B.xi64[e] = z;
             p_xi = P.nsp ? mi * c2i * z : z;
@@ -394,7 +400,11 @@ __global__ void __launch_bounds__(128) k_setup(const __grid_constant__ SetupArgs
     }
 }
 
-__global__ void k_status_out(const int* status, int* host) { *host = *status; }
+__global__ void k_status_out(const int* status, int* host)
+{
+    ne_chain();
+    *host = *status;
+}
 
 __global__ void k_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n,
                         int mixed, double* z)
@@ -527,6 +537,7 @@ __global__ void __launch_bounds__(1024) k_spring(const double* __restrict__ x, c
 template <bool MIXED>
 __global__ void k_export(DevBatch B, double* f, double* e, double scale)
 {
+    ne_chain();
     const RepDev& P = B.rep[0];
     if (f)
         for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < 3 * P.n; q += gridDim.x * blockDim.x) {
@@ -608,9 +619,9 @@ void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long*
                  int do_close, int do_open, cudaStream_t st)
 {
     if (mixed)
-        k_step<true><<<B.n_tiles, STEP_THREADS, 0, st>>>(B, S, step_base, j, do_close, do_open);
+        ne_launch(k_step<true>, B.n_tiles, STEP_THREADS, 0, st, B, S, step_base, j, do_close, do_open);
     else
-        k_step<false><<<B.n_tiles, STEP_THREADS, 0, st>>>(B, S, step_base, j, do_close, do_open);
+        ne_launch(k_step<false>, B.n_tiles, STEP_THREADS, 0, st, B, S, step_base, j, do_close, do_open);
     if (B.trace && do_open) k_trace_T<<<1, 32, 0, st>>>(B, step_base, j);
 }
 
@@ -640,7 +651,7 @@ void launch_setup(const RepDev* reps, int n_rep, RepDev* rep, int* tile_rep, uns
     }
 }
 
-void launch_status_out(const int* status, int* host, cudaStream_t st) { k_status_out<<<1, 1, 0, st>>>(status, host); }
+void launch_status_out(const int* status, int* host, cudaStream_t st) { ne_launch(k_status_out, 1, 1, 0, st, status, host); }
 
 void launch_init_velocities(const DevBatch& B, int fix_cm, cudaStream_t st)
 {
@@ -659,9 +670,9 @@ void launch_export(const DevBatch& B, bool mixed, double* f_out, double* e_out, 
 {
     const int want = f_out ? (3 * B.n_tot + 255) / 256 : 1, grid = want < 4 * B.sms ? want : 4 * B.sms;
     if (mixed)
-        k_export<true><<<grid, 256, 0, st>>>(B, f_out, e_out, scale);
+        ne_launch(k_export<true>, grid, 256, 0, st, B, f_out, e_out, scale);
     else
-        k_export<false><<<grid, 256, 0, st>>>(B, f_out, e_out, scale);
+        ne_launch(k_export<false>, grid, 256, 0, st, B, f_out, e_out, scale);
 }
 
 void launch_msd_sample(const DevBatch& B, double* acc, cudaStream_t st)
