@@ -374,11 +374,14 @@ __device__ __forceinline__ unsigned ne_ticket(unsigned* p)
 // blocks take their places on the SMs while the one before drains; every one
 // of its threads calls ne_chain before it reads what an earlier kernel of the
 // chain writes, and before it returns (a kernel that ended without having
-// waited would let the next one pass its wait too early).  What bounds a step
-// of a small replica are the latencies of five kernels and the gaps between
-// them: 128 atoms in FP64, replayed from a graph, 33.1 -> 29.3 us a step;
-// 2000 atoms launched one by one 35 -> 24 us; 65,536 atoms with the parameter
-// gradient 155 -> 150 us.
+// waited would let the next one pass its wait too early).  Before it a thread
+// reads only what is fixed for the whole call: the tiles' replicas, the replica
+// table but for a barostatted box (the call's other kernels, k_setup first,
+// are launched plainly and end before the chain's first begins).  What bounds
+// a step of a small replica are the latencies of five kernels and the gaps
+// between them: 128 atoms in FP64, replayed from a graph, 33.1 -> 29.3 us a
+// step; 2000 atoms launched one by one 35 -> 24 us; 65,536 atoms with the
+// parameter gradient 155 -> 150 us.
 __device__ __forceinline__ void ne_chain()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -123,10 +123,10 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
 {
     __shared__ int s_warp[32];
     __shared__ int s_done[CELL_TILES];  // replica whose last tile this block finished, or -1
-    ne_chain();
     const int tl = threadIdx.x / NE_TILE;
     const int tile = blockIdx.x * CELL_TILES + tl;
     const int rep = tile < B.n_tiles ? B.tile_rep[tile] : 0;
+    ne_chain();
     const bool go = tile < B.n_tiles && (force || B.flags[rep] != 0);
     if (!__syncthreads_or(go)) return;
     const RepDev& P = B.rep[rep];
@@ -224,11 +224,10 @@ __global__ void __launch_bounds__(256) k_nl_sort(DevBatch B)
 constexpr int LIST_THREADS = 256;
 
 template <int G>
-__device__ void list_block(const DevBatch& B, int blk)
+__device__ void list_block(const DevBatch& B, int blk, int rep)
 {
     constexpr int AT = LIST_THREADS / G, SUB = NE_TILE / AT;
     const int tile = blk / SUB;
-    const int rep = B.tile_rep[tile];
     if (!B.building[rep]) return;
     const RepDev& P = B.rep[rep];
     const int lane = threadIdx.x % G;
@@ -310,8 +309,15 @@ __device__ void list_block(const DevBatch& B, int blk)
 template <int G>
 __global__ void __launch_bounds__(LIST_THREADS) k_nl_list(DevBatch B)
 {
+    constexpr int SUB = NE_TILE * G / LIST_THREADS;
+    int blk = blockIdx.x, rep = B.tile_rep[blk / SUB];
     ne_chain();
-    for (int blk = blockIdx.x; blk < B.n_tiles * (NE_TILE * G / LIST_THREADS); blk += gridDim.x) list_block<G>(B, blk);
+    for (;;) {
+        list_block<G>(B, blk, rep);
+        blk += gridDim.x;
+        if (blk >= B.n_tiles * SUB) break;
+        rep = B.tile_rep[blk / SUB];
+    }
 }
 
 }  // namespace
