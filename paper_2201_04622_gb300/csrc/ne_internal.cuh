@@ -377,15 +377,18 @@ __device__ __forceinline__ unsigned ne_ticket(unsigned* p)
 // waited would let the next one pass its wait too early).  Before it a thread
 // reads only what is fixed for the whole call: the tiles' replicas, the replica
 // table but for a barostatted box (the call's other kernels, k_setup first,
-// are launched plainly and end before the chain's first begins).  What bounds
-// a step of a small replica are the latencies of five kernels and the gaps
-// between them: 128 atoms in FP64, replayed from a graph, 33.1 -> 29.3 us a
-// step; 2000 atoms launched one by one 35 -> 24 us; 65,536 atoms with the
-// parameter gradient 155 -> 150 us.
+// are launched plainly and end before the chain's first begins).  The next
+// kernel is let in after the wait: let in before it, the step kernel's normals
+// ran beside pass 1 and took its FP64 slots (15.8 ms against 16.6 to 19.8,
+// with the SMs that the blocks fell on, for the 600 steps of 128 atoms).
+// What bounds a step of a small replica are the latencies of five kernels and
+// the gaps between them: 128 atoms in FP64, replayed from a graph, 33.1 -> 25.8
+// us a step; 2000 atoms launched one by one 35 -> 22 us; 65,536 atoms with the
+// parameter gradient 155 -> 149 us.
 __device__ __forceinline__ void ne_chain()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename... P, typename... A>
