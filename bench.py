@@ -489,7 +489,7 @@ def run_ours(args):
         else:
             ops = (16.0 if top == "density" else 30.0) * pairs_per_atom * n_atoms
             ach = ops / (per[top] * 1e-3)
-            roof = {"bound": "alu", "kernel": "k_density (pass 1)" if top == "density" else "k_force (pass 2)",
+            roof = {"bound": "alu", "kernel": "k_pass1 (density, pair forces)" if top == "density" else "k_pass2 (embedding forces)",
                     "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "T lane-ops/s", "frac": ach / peak,
                     "traffic": None, "per_launch_ms": per,
                     "algorithmic": "%d FP32 lane instructions per pair inside r_c x %.1f pairs per atom"
@@ -499,9 +499,11 @@ def run_ours(args):
             # forward kernels (same launches without the backward)
             roof["backward_ms_per_step"] = ms / K - sum(per.values())
     steps_per_graph = 32
-    general_launches = 6 * K + (K - 1) // steps_per_graph + 10  # list prep, bin, list, pass 1, pass 2, step
+    # cells, (the cell sort of a replica above 16,384 atoms,) list, pass 1, pass 2, step
+    per_step = 5 + (max(offs[q + 1] - offs[q] for q in range(len(offs) - 1)) > 16384)
+    general_launches = per_step * K + (K - 1) // steps_per_graph + 10
     if path == "crystal":
-        launches = (c1[3] - c0[3]) + sum(6 * e[3] + e[3] // steps_per_graph + 10
+        launches = (c1[3] - c0[3]) + sum(5 * e[3] + e[3] // steps_per_graph + 10
                                          for e in timed_log if e[0] == "general")
     else:
         launches = general_launches + (2 * (K + 1) if grad else 0)  # backward: bins + reduction per step
