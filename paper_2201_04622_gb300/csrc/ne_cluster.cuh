@@ -202,19 +202,6 @@ struct ne_baro_smem {
     int box_ok;           // two periodic images of a site stay more than 2 r_c apart
 };
 
-// exp(x) - 1: the Taylor sum for the small arguments of a barostat step
-// (|x| < 1/64: the eighth term is below 2^-60 of the first), else expm1
-__device__ __forceinline__ double ne_baro_expm1(double x)
-{
-    if (fabs(x) >= 0.015625) return expm1(x);
-    double t = fma(x, 1.0 / 5040.0, 1.0 / 720.0);
-    t = fma(t, x, 1.0 / 120.0);
-    t = fma(t, x, 1.0 / 24.0);
-    t = fma(t, x, 1.0 / 6.0);
-    t = fma(t, x, 0.5);
-    return fma(t * x, x, x);
-}
-
 // normals of the 32 steps from s on, a step per lane
 __device__ __forceinline__ void ne_baro_draw(ne_baro_smem& b, const XRep& R, long long s)
 {

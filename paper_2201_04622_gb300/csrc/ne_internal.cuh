@@ -284,6 +284,19 @@ __device__ __forceinline__ float ne_normal32(uint4 w, int c)
     return sqrtf(-2.0f * logf(u0)) * (c == 1 ? sn : cs);
 }
 
+// exp(x) - 1: the Taylor sum for the small arguments of a barostat step
+// (|x| < 1/64: the eighth term is below 2^-60 of the first), else expm1
+__device__ __forceinline__ double ne_baro_expm1(double x)
+{
+    if (fabs(x) >= 0.015625) return expm1(x);
+    double t = fma(x, 1.0 / 5040.0, 1.0 / 720.0);
+    t = fma(t, x, 1.0 / 120.0);
+    t = fma(t, x, 1.0 / 24.0);
+    t = fma(t, x, 1.0 / 6.0);
+    t = fma(t, x, 0.5);
+    return fma(t * x, x, x);
+}
+
 // ------------------------------------------------------------------ misc
 // double-float (hi + lo, |lo| <= ulp(hi) / 2) sum of two such numbers from
 // FP32 operations (TwoSum of the high parts, the low parts added to its error)
