@@ -1,5 +1,5 @@
 """The multi-kernel path where it changes its form: the lanes per atom of the
-pair passes (32 up to 8192 atoms, 16 up to 24,576, 8 above) with the replica
+pair passes (32 up to 4096 atoms, 16 up to 16,384, 8 above) with the replica
 totals in groups (above 4096 atoms), the replica table as a launch argument
 (up to 24 replicas, six a launch) or copied, and the mixed parameter gradient
 with the bins of all three functions in shared memory or F's in global memory
@@ -34,7 +34,7 @@ def rel(a, b):
     return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(np.asarray(b)))
 
 
-@pytest.mark.parametrize("cell", [(16, 16, 16), (16, 16, 17), (22, 23, 24), (23, 23, 24)])
+@pytest.mark.parametrize("cell", [(16, 16, 8), (15, 12, 12), (16, 16, 32), (16, 16, 33)])
 def test_pair_passes_at_the_edges_of_the_lane_rule(cell):
     x0, box = O.create_crystal(O.BCC, W.A_BCC, *cell)
     p = O.eam(**W.EAM_FE_LIKE)
