@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(STEP_THREADS)
     const int a = (tile - P.tile0) * NE_TILE + al;
     const bool valid = a < P.n;
     const size_t e = 3 * (size_t)(P.off + (valid ? a : 0)) + c;
-    const long long s = *step_base + j;
+    const long long s = __ldcg(step_base) + j;  // from L2: the last chunk's end advanced it
     const double* T = B.tot + (size_t)rep * NTOT;
     const bool draw = do_open || !do_close;  // a step follows: its normals
     // the normals of the coming step, which depend on nothing that a kernel of
