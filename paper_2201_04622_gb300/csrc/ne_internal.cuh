@@ -389,8 +389,11 @@ __device__ __forceinline__ unsigned ne_ticket(unsigned* p)
 // chain writes, and before it returns (a kernel that ended without having
 // waited would let the next one pass its wait too early).  Before it a thread
 // reads only what is fixed for the whole call: the tiles' replicas, the replica
-// table but for a barostatted box (the call's other kernels, k_setup first,
-// are launched plainly and end before the chain's first begins).  The next
+// table but for a barostatted box.  The chain's first kernel, k_nl_cells, reads
+// nothing before its wait: the kernel before it (k_setup, which writes both
+// tables) is launched plainly and lets it in when its blocks end, but its
+// writes are sure to be seen only behind the wait.  A later kernel begins after
+// the wait of the one before it, and so after every write of that set-up.  The next
 // kernel is let in after the wait: let in before it, the step kernel's normals
 // ran beside pass 1 and took its FP64 slots (15.8 ms against 16.6 to 19.8,
 // with the SMs that the blocks fell on, for the 600 steps of 128 atoms).

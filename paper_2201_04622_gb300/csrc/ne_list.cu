@@ -125,8 +125,10 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
     __shared__ int s_done[CELL_TILES];  // replica whose last tile this block finished, or -1
     const int tl = threadIdx.x / NE_TILE;
     const int tile = blockIdx.x * CELL_TILES + tl;
-    const int rep = tile < B.n_tiles ? B.tile_rep[tile] : 0;
     ne_chain();
+    // (after the wait: in a single-point call the kernel before this one is
+    // k_setup, which writes the table)
+    const int rep = tile < B.n_tiles ? B.tile_rep[tile] : 0;
     const bool go = tile < B.n_tiles && (force || B.flags[rep] != 0);
     if (!__syncthreads_or(go)) return;
     const RepDev& P = B.rep[rep];
