@@ -297,6 +297,24 @@ __device__ __forceinline__ double ne_baro_expm1(double x)
     return fma(t * x, x, x);
 }
 
+// ------------------------------------------------------------------ box
+// x into [0, L) (w its FP32 copy; iL = 1 / L).  The image index is found in
+// FP32, the shift, only for an atom outside the box, taken off in FP64 (one
+// FMA's rounding).  The index of an atom N boxes away is off by up to N 2^-24,
+// so what is left is wrapped again until it lies inside: once for an atom near
+// the box, twice up to 2^24 boxes.  An atom beyond ~10^29 boxes stays outside.
+__device__ __forceinline__ void ne_wrap(double& x, float& w, double L, float iL)
+{
+    w = (float)x;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const float n = floorf(w * iL);
+        if (n == 0.f) break;
+        x = fma(-L, (double)n, x);
+        w = (float)x;
+    }
+}
+
 // ------------------------------------------------------------------ misc
 // double-float (hi + lo, |lo| <= ulp(hi) / 2) sum of two such numbers from
 // FP32 operations (TwoSum of the high parts, the low parts added to its error)

@@ -136,18 +136,11 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
     if (go && a < P.n) {
         const int i = P.off + a;
         const double* X = from_sites ? B.x0 : B.x;
-        // image index in FP32, the shift, only for an atom outside the box, in
-        // FP64 (as the step kernel)
         double w[3];
         float wf[3];
         for (int d = 0; d < 3; ++d) {
             w[d] = X[3 * i + d];
-            wf[d] = (float)w[d];
-            const float n = floorf(wf[d] * P.iLf[d]);
-            if (n != 0.f) {
-                w[d] -= P.L[d] * (double)n;
-                wf[d] = (float)w[d];
-            }
+            ne_wrap(w[d], wf[d], P.L[d], P.iLf[d]);
         }
         const float4 p = make_float4(wf[0], wf[1], wf[2], __int_as_float(a));
         B.pbuild[i] = p;

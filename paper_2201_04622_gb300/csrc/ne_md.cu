@@ -242,17 +242,12 @@ __global__ void __launch_bounds__(STEP_THREADS)
         if (do_close || do_open) B.v[e] = (double)v;
         p_ux = P.nsp ? ki * u : u;
         p_u2 = u * u;
-        // x wrapped (image index in FP32, the shift, only for an atom outside
-        // the box, in FP64), its image against the list build's and the
-        // displacement from there
-        float w = (float)x;
-        const float n = floorf(w * s_iLf[c]);
-        if constexpr (!MIXED) s_x64[c][al] = x;
-        if (n != 0.f) {
-            const double xw = x - s_L[c] * (double)n;
-            w = (float)xw;
-            if constexpr (!MIXED) s_x64[c][al] = xw;
-        }
+        // x wrapped, its image against the list build's and the displacement from
+        // there
+        double xw = x;
+        float w;
+        ne_wrap(xw, w, s_L[c], s_iLf[c]);
+        if constexpr (!MIXED) s_x64[c][al] = xw;
         const float nb = rintf((w - pb) * s_iLf[c]), d = fmaf(-s_Lf[c], nb, w - pb);
         s_w[c][al] = w;
         s_d2[c][al] = d * d;
