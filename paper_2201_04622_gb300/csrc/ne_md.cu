@@ -249,9 +249,12 @@ __global__ void __launch_bounds__(STEP_THREADS)
         ne_wrap(xw, w, s_L[c], s_iLf[c]);
         if constexpr (!MIXED) s_x64[c][al] = xw;
         const float nb = rintf((w - pb) * s_iLf[c]), d = fmaf(-s_Lf[c], nb, w - pb);
+        // (a position that no wrap takes into the box: no image code, but a list
+        // built around it)
+        const bool in = fabsf(nb) <= 1.f;
         s_w[c][al] = w;
-        s_d2[c][al] = d * d;
-        s_code[c][al] = (int)nb;
+        s_d2[c][al] = in || isnan(nb) ? d * d : __int_as_float(0x7f800000);
+        s_code[c][al] = in ? (int)nb : 0;
         if (draw) {
             if constexpr (MIXED) B.xi32[e] = z;
             else B.xi64[e] = z;

@@ -95,3 +95,36 @@ def test_a_run_far_from_the_origin(prec):
         assert np.allclose(out[1][1], out[0][1], rtol=1e-7, atol=1e-6 if prec == ne.NE_FP64 else 2e-4)
     finally:
         ne.ne_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("lat,cells", [(O.BCC, 4), (O.BCC, 7)])  # all pairs; cells
+@pytest.mark.parametrize("prec", [ne.NE_FP64, ne.NE_MIXED])
+@pytest.mark.parametrize("at", [2.0**100, 1e30, 3e38, 1e60])
+def test_a_position_beyond_any_box_stays_inside_the_tables(lat, cells, prec, at):
+    """One atom at a finite coordinate that FP32 cannot wrap: single-point calls
+    and runs return (with an error or without: the coordinate has no meaning),
+    and the context then gives the oracle's energy of the plain crystal."""
+    x0, box = O.create_crystal(lat, W.A_BCC, cells, cells, cells)
+    p = O.eam(**W.EAM_FE_LIKE)
+    Eo, _, _ = O.eam_energy_forces(p, O.eam_theta(p), x0, box)
+    ctx = ne.ne_ctx_create(ne.eam_params(**W.EAM_FE_LIKE), len(x0), 1)
+    md = ne.md_params(T=300.0, mass=MASS, k_spring=5.0, skin=0.4, prec=prec, t_eq=4, t_s=8, seed=3, replica=0, fix_cm=0)
+    far = x0.copy()
+    far[5] = (at, -at, at)
+    try:
+        e = T([0.0])
+        for _ in range(2):
+            try:
+                ne.ne_eam_energy_forces(ctx, prec, T(far), box, e=e)
+            except ne.NeError:
+                pass
+            for sites in (x0, far):
+                try:
+                    ne.ne_switch_run_segment(ctx, [md], [0, len(x0)], T(far), T(np.zeros_like(x0)), T(sites), [box],
+                                             torch.zeros((1, 2), dtype=torch.float64, device="cuda"), 0, 12)
+                except ne.NeError:
+                    pass
+            ne.ne_eam_energy_forces(ctx, prec, T(x0), box, e=e)
+            assert float(e) == pytest.approx(Eo, rel=1e-10 if prec == ne.NE_FP64 else 1e-6)
+    finally:
+        ne.ne_ctx_destroy(ctx)
