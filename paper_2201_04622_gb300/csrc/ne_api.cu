@@ -1382,8 +1382,8 @@ static bool same_sched(const Sched& a, const Sched& b)
            a.fn == b.fn && a.stream == b.stream && a.fix_cm == b.fix_cm;
 }
 
-// SMs that a brick launch leaves free where its atoms do not need them
-constexpr int BRICK_FREE_SMS = 8;
+// SMs that a brick launch spread over more CTAs than its atoms need leaves free
+constexpr int BRICK_FREE_SMS = 24;
 
 // Build the launch plan of a batch (stencils, replica table, cluster size,
 // size classes and their shared memory) and upload its device part.  Runs
@@ -1603,20 +1603,26 @@ static ne_status build_plan(ne_ctx* ctx, const ne_md_params* md, const ne_crysta
             }
             const int cap = ne::brick_max_ctas(tpa, smem, P.npt);
             if (total > cap) continue;
-            // where a quarter of the SMs or more would stay idle: more CTAs than
-            // the atoms need, down to 32 atoms each, while one more makes the
-            // fullest replica's CTAs smaller (a step is as long as its fullest
-            // SM).  A few SMs stay free for another stream's kernels
-            // (a replica on the multi-kernel path alongside)
+            // At one thread per atom (above ~58,000 atoms) and with a quarter of the
+            // SMs or more idle: more CTAs than the atoms need, while one more makes
+            // the fullest replica's CTAs smaller (a step is as long as its fullest
+            // SM).  One replica of bcc 32^3 alone, and beside a second on the
+            // multi-kernel path of another stream, us a step: 86 CTAs (as many as
+            // needed) 56.2 and 125.5, 114 45.0 and 129, 128 42.2 and 132, 144 50.7
+            // and 148; bcc 31 x 31 x 32, 81, 114, 128 and 144 CTAs: 57.1, 55.9,
+            // 50.9, 51.1.  With more threads per atom nothing is spread: bcc 13^3 takes
+            // 13.5 us on its 46 CTAs and 17 on 138, bcc 16^3 15.1 on 86 and 17 on 114,
+            // bcc 20^3 20.2 on 84 and 21 on 113 (the barrier grows), and two such
+            // launches of different contexts would no longer fit the device together.
             auto cta_atoms = [&](int r, int C) { return (((xr[r].n + C - 1) / C) + xr[r].nb - 1) / xr[r].nb * xr[r].nb; };
-            const bool spread = 4 * total <= 3 * cap;
+            const bool spread = tpa == 1 && 4 * total <= 3 * cap;
             while (spread && total < cap - BRICK_FREE_SMS) {
                 int big = 0;
                 for (int r = 1; r < n_rep; ++r)
                     if (cta_atoms(r, cr_[r]) > cta_atoms(big, cr_[big])) big = r;
                 int C = cr_[big] + 1;
                 while (total - cr_[big] + C <= cap - BRICK_FREE_SMS && cta_atoms(big, C) == cta_atoms(big, cr_[big])) ++C;
-                if (total - cr_[big] + C > cap - BRICK_FREE_SMS || cta_atoms(big, C) < 32) break;
+                if (total - cr_[big] + C > cap - BRICK_FREE_SMS) break;
                 total += C - cr_[big];
                 cr_[big] = C;
             }
