@@ -293,8 +293,8 @@ ne_status ne_spring_forces(const double* x_dev, const double* x0_dev, int n, dou
  * upstream gradient gE = dL/dU, writes gx_dev [n][3] = gE dU/dx = -gE F and
  * gtheta_dev [3][n_knots][2] = gE dU/dtheta for every knot value and slope of
  * phi, f and F.  rho is recomputed, not stored.  NE_MIXED: FP32 pair
- * arithmetic, FP32 per-block bins summed over the blocks in FP64, and the F
- * bins in exact 64-bit fixed point; NE_FP64: FP64 throughout. */
+ * arithmetic and weights, added in 64-bit fixed point (f's in a unit that
+ * follows the batch's |F'|); NE_FP64: FP64 throughout. */
 ne_status ne_eam_backward(ne_ctx* ctx, ne_precision prec, const double* x_dev, int n,
                           const double box[3], double gE, double* gx_dev,
                           double* gtheta_dev, void* stream);
@@ -402,8 +402,8 @@ ne_status ne_switch_run_segment_cum(ne_ctx* ctx, const ne_md_params* md, int n_r
  * F; value and slope per knot), accumulated.  E.g. w = 1 every `stride`
  * steps at lambda = 0 gives sum dU/dtheta for <dU/dtheta> = dF_0/dtheta, and
  * w_k = lambda_k - lambda_(k-stride) over a switch the derivative of W at
- * fixed trajectory.  Mixed precision bins in FP32 per block and sums them in
- * FP64; FP64 adds with FP64 atomics.  Errors as ne_switch_run_segment. */
+ * fixed trajectory.  Mixed precision adds FP32 weights in 64-bit fixed point;
+ * FP64 adds with FP64 atomics.  Errors as ne_switch_run_segment. */
 ne_status ne_switch_run_segment_grad(ne_ctx* ctx, const ne_md_params* md, int n_rep,
                                      const int* offsets_host, double* x_dev, double* v_dev,
                                      const double* x0_dev, const double* boxes_host, double* W_dev,
