@@ -177,6 +177,10 @@ ne_status ne_ctx_set_cluster_size(ne_ctx* ctx, int ctas);
  * to the rounding of the replica sums. */
 ne_status ne_ctx_set_runner(ne_ctx* ctx, int runner);
 
+/* Polls (an L2 round trip each) after which a wait between the brick runner's
+ * CTAs gives up and the call returns NE_ETIMEOUT; 0: the default, a few seconds. */
+ne_status ne_ctx_set_wait_limit(ne_ctx* ctx, unsigned polls);
+
 /* Boxes [n_rep][3] (host) at the end of the last multi-kernel run or
  * segment of this context, or of its last crystal-runner call with the
  * barostat, in the order of its replicas: with the barostat
@@ -191,8 +195,9 @@ ne_status ne_ctx_boxes(ne_ctx* ctx, int n_rep, double* boxes_host);
  * pairs -- lattice-stencil entries examined and pairs found inside r_c by
  * ne_crystal_run_segment (pass 1), for algorithmic operation counts;
  * crystal_launches -- kernels launched by ne_crystal_run_segment (one cluster
- * kernel per replica size class a call, plus one lambda-table kernel on the
- * first call of each schedule).  Synchronises the device. */
+ * kernel per replica size class a call, or the brick runner's two, plus one
+ * lambda-table kernel on the first call of each schedule).  Synchronises the
+ * device. */
 ne_status ne_ctx_counters(ne_ctx* ctx, long long* list_builds, long long* stencil_visits,
                           long long* pairs, long long* crystal_launches);
 
@@ -431,7 +436,8 @@ typedef struct {
  * > 2 r_c + 1.2 A; replicas above 4096 atoms run on the brick runner
  * (ne_ctx_set_runner), which needs the batch's CTAs (one per 96-768 atoms)
  * to fit the device at once (NE_ENOMEM otherwise); a barrier wait that
- * lasts longer than a few seconds gives NE_ETIMEOUT.  The barostat
+ * lasts longer than a few seconds gives NE_ETIMEOUT and leaves x, v and W of
+ * every replica as they were.  The barostat
  * (md[r].npt, reversible-scaling path) runs on both runners: the box and
  * the lattice sites scale with it, ne_ctx_boxes reads the boxes the call
  * reached, and the next segment takes cr[r].a = box edge / cells (and, per

@@ -95,7 +95,7 @@ struct ne_ctx {
     bool lam_valid = false;
     CrPlan plan;                // launch plan of the last crystal-runner batch
     int runner = 0;             // 0 automatic, 1 cluster runner only, 2 brick runner for every batch
-    ne::BrickBufs bb{};         // brick runner's exchange buffers (allocated on first use)
+    ne::BrickBufs bb{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, NE_SPIN_LIMIT};  // brick runner (buffers allocated on first use)
     int* cta_rep = nullptr;     // brick runner: replica of each CTA
     int bb_ctas = 0;            // CTAs the partials buffer holds
     double* cr_boxes = nullptr; // crystal runner with the barostat: each replica's box at the call's end
@@ -751,7 +751,7 @@ ne_status ne_ctx_destroy(ne_ctx* ctx)
         if (ctx->gev[g]) cudaEventDestroy(ctx->gev[g]);
     for (int g = 0; g < 2; ++g)
         if (ctx->ev_run[g]) cudaEventDestroy(ctx->ev_run[g]);
-    void* bptrs[] = {ctx->bb.u4, ctx->bb.part, ctx->bb.vir, ctx->bb.bar, ctx->bb.abortf, ctx->cta_rep,
+    void* bptrs[] = {ctx->bb.u4, ctx->bb.part, ctx->bb.vir, ctx->bb.bar, ctx->bb.abortf, ctx->bb.xs, ctx->bb.vs, ctx->bb.ws, ctx->cta_rep,
                      ctx->cr_boxes};
     for (void* p : bptrs)
         if (p) cudaFree(p);
@@ -768,6 +768,7 @@ ne_status ne_ctx_clone(ne_ctx* src, int max_atoms, int max_replicas, ne_ctx** ou
     if (s) return s;
     c->tpa = src->tpa;
     c->cluster_c = src->cluster_c;
+    c->bb.spin_limit = src->bb.spin_limit;
     s = ne_ctx_set_theta(c, src->theta, nullptr);
     if (!s && cudaDeviceSynchronize() != cudaSuccess) s = NE_ECUDA;
     if (s) {
@@ -819,6 +820,13 @@ ne_status ne_ctx_set_runner(ne_ctx* ctx, int runner)
     if (!ctx) return NE_EINVAL;
     if (runner < 0 || runner > 2) return fail(ctx, NE_EINVAL, "runner must be 0 (automatic), 1 (cluster) or 2 (brick)");
     ctx->runner = runner;
+    return NE_OK;
+}
+
+ne_status ne_ctx_set_wait_limit(ne_ctx* ctx, unsigned polls)
+{
+    if (!ctx) return NE_EINVAL;
+    ctx->bb.spin_limit = polls ? polls : NE_SPIN_LIMIT;
     return NE_OK;
 }
 
@@ -1643,11 +1651,19 @@ static ne_status build_plan(ne_ctx* ctx, const ne_md_params* md, const ne_crysta
         if (!P.brick)
             return fail(ctx, NE_ENOMEM, "brick runner: the batch needs more CTAs than the device holds at once");
         // exchange buffers, sized for the context (once)
-        if (!ctx->bb.u4) {
-            const size_t N = (size_t)ctx->max_atoms;
-            NE_CU(cudaMalloc((void**)&ctx->bb.u4, sizeof(float4) * 2 * N));
-            NE_CU(cudaMalloc((void**)&ctx->bb.bar, sizeof(unsigned) * NE_BAR_STRIDE * (size_t)ctx->max_rep));
-            NE_CU(cudaMalloc((void**)&ctx->bb.abortf, sizeof(int)));
+        {
+            const size_t N = (size_t)ctx->max_atoms, R = (size_t)ctx->max_rep;
+            cudaError_t e = cudaSuccess;
+            auto need = [&](auto** p, size_t bytes) {
+                if (e == cudaSuccess && !*p) e = cudaMalloc((void**)p, bytes);
+            };
+            need(&ctx->bb.u4, sizeof(float4) * 2 * N);
+            need(&ctx->bb.bar, sizeof(unsigned) * NE_BAR_STRIDE * R);
+            need(&ctx->bb.abortf, sizeof(int));
+            need(&ctx->bb.xs, sizeof(double) * 3 * N);
+            need(&ctx->bb.vs, sizeof(float) * 3 * N);
+            need(&ctx->bb.ws, sizeof(double) * 5 * R);
+            NE_CU(e);
         }
         if (P.n_cta > ctx->bb_ctas) {
             if (ctx->bb.part) cudaFree(ctx->bb.part);
@@ -1828,7 +1844,7 @@ static ne_status crystal_segment_impl(ne_ctx* ctx, const ne_md_params* md, const
         NE_CU(ne::launch_brick(P.tpa, ctx->xrep, n_rep, ctx->cta_rep, P.n_cta, P.smem, ctx->st_vec, ctx->st_dist, x_dev,
                                v_dev, W_dev, ctx->status, S, step_begin, n_steps, ctx->tab, ctx->work, P.k_lo,
                                ctx->lam_tab + step_begin, Wcum_dev, ctx->bb, n_tot, st, P.npt, ctx->cr_boxes));
-        ++ctx->cr_launches;
+        ctx->cr_launches += 2;  // k_brick, k_brick_commit
         NE_CU(cudaEventRecord(ctx->ev_run[1], st));
         ctx->run_timed = true;
         if (P.npt) {  // ne_ctx_boxes reads the boxes this call reached

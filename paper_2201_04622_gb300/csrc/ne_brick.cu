@@ -26,9 +26,11 @@
 // the replica forms the same scale factors (the same sums in the same order,
 // the same Philox normal) before its integration.  A barrier is an arrival count
 // in global memory; every CTA of the launch is resident at once (cooperative
-// launch), and every wait is bounded: after BAR_SPIN_LIMIT polls a CTA records
+// launch), and every wait is bounded: after bb.spin_limit polls a CTA records
 // NE_ETIMEOUT, raises the abort word and leaves, and the others leave at the
-// barrier they wait at.
+// barrier they wait at.  What the replicas reached is left in buffers of the
+// context, and a second kernel (k_brick_commit) takes it over when every CTA is
+// done: all replicas without an error, or, if a wait gave up, none.
 //
 // The neighbours' (u, F') are plain loads through L1: a barrier's acquire orders
 // them after the other CTAs' writes (and drops the SM's L1 lines), and a CTA's
@@ -71,7 +73,6 @@ constexpr int NSV = 2 * ND_ + NF_;  // floats of the sums: (hi, lo) per energy, 
 constexpr int NPART = NSV + 1;      // and max |u|
 constexpr int T_UX = 2 * ND_ + (P_UX - ND_), T_XX = 2 * ND_ + (P_XX - ND_);
 constexpr int NRED = (int)NP_ + 1;
-constexpr unsigned BAR_SPIN_LIMIT = 1u << 22;  // polls, each an L2 round trip: a few seconds at most
 constexpr double XSCALE = 4294967296.0;        // fixed point: 2^32 per Angstrom
 
 struct dfl {
@@ -118,8 +119,8 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
 // replica the slowest one's time and two more L2 round trips.  Returns false
 // when a wait gave up, here or, as the abort word says, in another CTA: the
 // caller leaves.
-__device__ bool replica_barrier(unsigned* bar, unsigned n, unsigned& target, int* status, int widx, int* abortf,
-                                int* s_flag)
+__device__ bool replica_barrier(unsigned* bar, unsigned n, unsigned& target, int* status, int widx,
+                                const ne::BrickBufs& bb, int* s_flag)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -130,11 +131,11 @@ __device__ bool replica_barrier(unsigned* bar, unsigned n, unsigned& target, int
         unsigned spins = 0;
         while ((int)(ld_acquire(bar) - target) < 0) {
             ++spins;
-            if (spins > BAR_SPIN_LIMIT || ((spins & 63u) == 0u && ld_acquire((const unsigned*)abortf) != 0u)) {
+            if (spins > bb.spin_limit || ((spins & 63u) == 0u && ld_acquire((const unsigned*)bb.abortf) != 0u)) {
                 ok = 0;
                 ne_set_status(status, ST_ETIMEOUT);
                 ne_set_status(status + 1 + widx, ST_ETIMEOUT);
-                atomicExch(abortf, 1);
+                atomicExch(bb.abortf, 1);
                 break;
             }
         }
@@ -158,10 +159,10 @@ __device__ __forceinline__ void warp_df3(dfl (&v)[3])
 template <int TPA, bool NPT>
 __global__ void __launch_bounds__(BTHREADS, 1)
     k_brick(const XRep* __restrict__ reps, const int* __restrict__ cta_rep, const float4* __restrict__ st_vec,
-            const float* __restrict__ st_dist, double* __restrict__ xg, double* __restrict__ vg,
-            double* __restrict__ Wg, int* status, Sched S, long long s_begin, long long n_steps, Tables tab,
+            const float* __restrict__ st_dist, const double* __restrict__ xg, const double* __restrict__ vg,
+            const double* __restrict__ Wg, int* status, Sched S, long long s_begin, long long n_steps, Tables tab,
             unsigned long long* work, int k_lo, const double* __restrict__ lam_tab, double* __restrict__ wcum,
-            ne::BrickBufs bb, long long n_tot, double* __restrict__ boxes_out)
+            ne::BrickBufs bb, long long n_tot)
 {
     constexpr int SLOTS = BTHREADS / TPA;
     static_assert(BTHREADS % TPA == 0 && SLOTS % 32 == 0, "whole warps of one pair lane");
@@ -393,7 +394,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         cta_partials(pd, pf, um, (int)(s_begin & 1));
     }
     unsigned target = 0;
-    bool alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);
+    bool alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb, s_flag);
 
     unsigned n_cand = 0, n_pair = 0;
     const float rc2 = tab.rc2f, rmin2 = tab.rmin2f, inv_h = tab.inv_h_rf;
@@ -616,7 +617,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             ((float*)&u_cur[tsu])[3] = dF;
             if (!isfinite(emb)) bad |= ST_ENAN;
         }
-        alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // F' visible everywhere
+        alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb, s_flag);  // F' visible everywhere
         if (!alive) break;
 
         // ---- pass 2: embedding forces over the visits of pass 1, f'(r)/r from TMEM
@@ -732,7 +733,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                             bb.vir[(size_t)blockIdx.x * 6 + 2 * a3 + 1] = t[a3].lo;
                         }
                 }
-                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // virials visible
+                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb, s_flag);  // virials visible
                 if (!alive) break;
                 if (w == 0) {
                     const double lam = lam_tab[it + 1];
@@ -844,7 +845,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             }
             if (!fin) {
                 cta_partials(pd, pf, dead ? 1e30f : un, p ^ 1);
-                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);  // u of s + 1 visible
+                alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb, s_flag);  // u of s + 1 visible
             }
         }
     }
@@ -863,27 +864,49 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             atomicAdd(&work[1], (unsigned long long)n_pair);
         }
     }
-    if (!alive) return;  // a wait gave up: the call reports NE_ETIMEOUT
-    // every CTA's error bits for its replica are in the status word after
-    // this barrier; a replica that raised none writes its state back
-    alive = replica_barrier(bar, (unsigned)C, target, status, R_.widx, bb.abortf, s_flag);
-    if (!alive) return;
-    if (threadIdx.x == 0) s_flag[1] = atomicOr(status + 1 + R_.widx, 0) | (int)ld_acquire((const unsigned*)bb.abortf);
-    __syncthreads();
-    if (s_flag[1] == 0) {
-        if (own)
-            for (int c = 0; c < 3; ++c) {
-                // the site of the atom in the (scaled) box
-                const long long site = NPT ? __double2ll_rn(s_b->mu_tot[c] * (double)site_fix(c)) : site_fix(c);
-                xg[gi + c] = (double)(xr[c] + site) / XSCALE;
-                vg[gi + c] = (double)v[c];
-            }
-        if (wthread) {
-            Wg[2 * R_.widx] = s_work[0];
-            Wg[2 * R_.widx + 1] = s_work[1];
-            if (NPT && boxes_out)
-                for (int c = 0; c < 3; ++c) boxes_out[3 * R_.widx + c] = s_b->mu_tot[c] * R_.box0[c];
+    if (!alive) return;  // a wait gave up: the call reports NE_ETIMEOUT and changes nothing
+    if (own)
+        for (int c = 0; c < 3; ++c) {
+            // the site of the atom in the (scaled) box
+            const long long site = NPT ? __double2ll_rn(s_b->mu_tot[c] * (double)site_fix(c)) : site_fix(c);
+            bb.xs[gi + c] = (double)(xr[c] + site) / XSCALE;
+            bb.vs[gi + c] = v[c];
         }
+    if (wthread) {
+        double* const ws = bb.ws + 5 * (size_t)R_.widx;
+        ws[0] = s_work[0];
+        ws[1] = s_work[1];
+        if (NPT)
+            for (int c = 0; c < 3; ++c) ws[2 + c] = s_b->mu_tot[c] * R_.box0[c];
+    }
+}
+
+// The state that the replicas reached into the caller's arrays, after the last
+// CTA has ended: a replica's only if it raised no error, none if a wait gave up
+// (every replica then has NE_ETIMEOUT).  Within the runner itself the CTAs of
+// replicas that no longer wait for one another could not tell alike whether
+// another one's wait gives up.
+__global__ void __launch_bounds__(256)
+    k_brick_commit(const XRep* __restrict__ reps, const int* __restrict__ cta_rep, ne::BrickBufs bb,
+                   double* __restrict__ x, double* __restrict__ v, double* __restrict__ W, int* status,
+                   double* __restrict__ boxes_out)
+{
+    const XRep& R = reps[cta_rep[blockIdx.x]];
+    const int rank = (int)blockIdx.x - R.cta0;
+    if (*bb.abortf) {
+        if (rank == 0 && threadIdx.x == 0) ne_set_status(status + 1 + R.widx, ST_ETIMEOUT);
+        return;
+    }
+    if (status[1 + R.widx]) return;
+    const size_t o = 3 * (size_t)R.off;
+    for (int q = rank * 256 + threadIdx.x; q < 3 * R.n; q += R.ncta * 256) {
+        x[o + q] = bb.xs[o + q];
+        v[o + q] = (double)bb.vs[o + q];
+    }
+    if (rank == 0 && threadIdx.x < 5) {
+        const double t = bb.ws[5 * (size_t)R.widx + threadIdx.x];
+        if (threadIdx.x < 2) W[2 * R.widx + threadIdx.x] = t;
+        else if (boxes_out) boxes_out[3 * R.widx + threadIdx.x - 2] = t;
     }
 }
 
@@ -905,13 +928,12 @@ template <int TPA, bool NPT>
 cudaError_t brick_launch(cudaLaunchConfig_t& cfg, const XRep* reps, const int* cta_rep, const float4* st_vec,
                          const float* st_dist, double* x, double* v, double* W, int* status, const Sched& S,
                          long long s_begin, long long n_steps, const Tables& tab, unsigned long long* work, int k_lo,
-                         const double* lam_tab, double* wcum, const ne::BrickBufs& bb, long long n_tot,
-                         double* boxes_out)
+                         const double* lam_tab, double* wcum, const ne::BrickBufs& bb, long long n_tot)
 {
     cudaError_t e = brick_attributes<TPA, NPT>(cfg.dynamicSmemBytes);
     if (e == cudaSuccess)
         e = cudaLaunchKernelEx(&cfg, k_brick<TPA, NPT>, reps, cta_rep, st_vec, st_dist, x, v, W, status, S, s_begin,
-                               n_steps, tab, work, k_lo, lam_tab, wcum, bb, n_tot, boxes_out);
+                               n_steps, tab, work, k_lo, lam_tab, wcum, bb, n_tot);
     return e;
 }
 
@@ -984,16 +1006,19 @@ cudaError_t launch_brick(int tpa, const XRep* reps, int n_rep, const int* cta_re
     cfg.attrs = attr;
     cfg.numAttrs = 1;
 #define NE_BRICK_ARGS cfg, reps, cta_rep, st_vec, st_dist, x, v, W, status, S, s_begin, n_steps, tab, work, k_lo, \
-                      lam_tab, wcum, bb, n_tot, boxes_out
+                      lam_tab, wcum, bb, n_tot
     switch (tpa) {
-    case 1: return npt ? brick_launch<1, true>(NE_BRICK_ARGS) : brick_launch<1, false>(NE_BRICK_ARGS);
-    case 2: return npt ? brick_launch<2, true>(NE_BRICK_ARGS) : brick_launch<2, false>(NE_BRICK_ARGS);
-    case 3: return npt ? brick_launch<3, true>(NE_BRICK_ARGS) : brick_launch<3, false>(NE_BRICK_ARGS);
-    case 4: return npt ? brick_launch<4, true>(NE_BRICK_ARGS) : brick_launch<4, false>(NE_BRICK_ARGS);
-    case 8: return npt ? brick_launch<8, true>(NE_BRICK_ARGS) : brick_launch<8, false>(NE_BRICK_ARGS);
+    case 1: e = npt ? brick_launch<1, true>(NE_BRICK_ARGS) : brick_launch<1, false>(NE_BRICK_ARGS); break;
+    case 2: e = npt ? brick_launch<2, true>(NE_BRICK_ARGS) : brick_launch<2, false>(NE_BRICK_ARGS); break;
+    case 3: e = npt ? brick_launch<3, true>(NE_BRICK_ARGS) : brick_launch<3, false>(NE_BRICK_ARGS); break;
+    case 4: e = npt ? brick_launch<4, true>(NE_BRICK_ARGS) : brick_launch<4, false>(NE_BRICK_ARGS); break;
+    case 8: e = npt ? brick_launch<8, true>(NE_BRICK_ARGS) : brick_launch<8, false>(NE_BRICK_ARGS); break;
     default: return cudaErrorInvalidValue;
     }
 #undef NE_BRICK_ARGS
+    if (e != cudaSuccess) return e;
+    k_brick_commit<<<n_cta, 256, 0, st>>>(reps, cta_rep, bb, x, v, W, status, npt ? boxes_out : nullptr);
+    return cudaGetLastError();
 }
 
 }  // namespace ne

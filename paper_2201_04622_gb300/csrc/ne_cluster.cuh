@@ -318,7 +318,12 @@ struct BrickBufs {
     float* vir;      // [n_cta][6] per-CTA diagonal virial (hi, lo per axis; barostat only)
     unsigned* bar;   // [replicas][NE_BAR_STRIDE] barrier arrivals, a cache line each
     int* abortf;     // a bounded wait gave up: every CTA leaves
+    double* xs;      // [N][3] positions that the call reached, until they are taken over
+    float* vs;       // [N][3] velocities
+    double* ws;      // [replicas][5] works and box
+    unsigned spin_limit;  // polls, each an L2 round trip, after which a wait gives up
 };
+#define NE_SPIN_LIMIT (1u << 22)  // a few seconds
 cudaError_t launch_brick(int tpa, const XRep* reps, int n_rep, const int* cta_rep, int n_cta, size_t smem, const float4* st_vec,
                          const float* st_dist, double* x, double* v, double* W, int* status, const Sched& S,
                          long long s_begin, long long n_steps, const Tables& tab, unsigned long long* work,
