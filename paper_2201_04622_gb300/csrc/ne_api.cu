@@ -277,8 +277,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
             R.invL[d] = 1.0 / R.L[d];
             R.Lf[d] = (float)R.L[d];
             R.iLf[d] = (float)R.invL[d];
-            // (the margin covers the FP32 binning)
-            R.nc[d] = geometry ? (int)std::min(std::floor(shrink * R.L[d] / (rl + 1e-3)), 1024.0) : 0;
+            R.nc[d] = geometry ? (int)std::min(std::floor(shrink * R.L[d] / rl), 1024.0) : 0;
         }
         // cells of edge >= r_c + skin; fewer (larger) cells when the box is
         // sparse, so the cell count stays below 2n + 27
@@ -313,6 +312,7 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
         R.replica = m.replica;
         if (m.replica >= (1u << 28)) return fail(ctx, NE_EINVAL, "replica id must be < 2^28");
         R.npt = m.npt;
+        ne_bin64(R, rl);
         R.P0 = m.P0;
         R.mp = m.npt ? m.beta_T / m.tau_p : 0.0;
         npt_any |= m.npt;

@@ -72,6 +72,7 @@ struct RepDev {
     int off, n, tile0, ntile;
     int grp0;        // first of its groups of GROUP_TILES tiles
     int nc[3];       // cells per axis; 0 = all pairs
+    int bin64;       // cells found in FP64 (see ne_bin64)
     int cell_off;
     int dof;
     unsigned long long seed;
@@ -91,6 +92,16 @@ struct RepDev {
     double inv_w;    // 1 / n, or 1 / M with species tables
     double ms[NE_MAX_SPECIES_DEV], ks[NE_MAX_SPECIES_DEV], c2s[NE_MAX_SPECIES_DEV], hdts[NE_MAX_SPECIES_DEV];
 };
+
+// The list build finds a position's cell in FP32, to 3e-7 of the box edge, which
+// cells of an edge above r_c + skin + 1e-3 A have room for up to 2000 A.  A replica
+// with smaller cells (down to r_c + skin, where an edge is a near multiple of it or
+// a barostat contracts the box) or a longer edge has its atoms binned in FP64.
+inline void ne_bin64(RepDev& R, double rl)
+{
+    R.bin64 = R.npt != 0;
+    for (int d = 0; d < 3; ++d) R.bin64 |= R.nc[d] > 0 && (R.L[d] < (rl + 1e-3) * R.nc[d] || R.L[d] > 2000.0);
+}
 
 // Schedule of a run, shared by the replicas of one launch.
 enum { SCHED_SWITCH = 0, SCHED_FIXED = 1 };

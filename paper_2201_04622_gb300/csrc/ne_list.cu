@@ -117,8 +117,8 @@ __device__ void sort_cells(const DevBatch& B, int rep, bool scatter, int* s_warp
 // (176 and 253 us).  Whole calls, before and with this build: energy and forces of
 // 70,304 atoms in FP64 1232 -> 973 us, energy and gradients of 65,536 atoms 1504
 // -> 1091 us, the 200-step spring fit of 2000 atoms at 1400 K 17.0 -> 13.6 ms.
-// The image index and the cell in FP32 (the cells are 1e-3 A wider than r_c +
-// skin) took another 8 us of FP64 out.
+// The image index and, where the cells are wide enough (bin64), the cell in FP32
+// took another 8 us of FP64 out.
 __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force, int from_sites)
 {
     __shared__ int s_warp[32];
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_nl_cells(DevBatch B, int force
         } else {
             int c3[3];
             for (int d = 0; d < 3; ++d) {
-                const int q = (int)(wf[d] * P.iLf[d] * (float)P.nc[d]);
+                const int q = P.bin64 ? (int)(w[d] * P.invL[d] * P.nc[d]) : (int)(wf[d] * P.iLf[d] * (float)P.nc[d]);
                 c3[d] = min(max(q, 0), P.nc[d] - 1);
             }
             const int c = (c3[0] * P.nc[1] + c3[1]) * P.nc[2] + c3[2];

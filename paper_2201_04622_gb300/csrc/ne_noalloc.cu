@@ -164,13 +164,14 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
         R.invL[d] = 1.0 / box[d];
         R.Lf[d] = (float)R.L[d];
         R.iLf[d] = (float)R.invL[d];
-        R.nc[d] = (int)std::min(std::floor(box[d] / (rc + 1e-3)), 1024.0);  // the margin covers the FP32 binning
+        R.nc[d] = (int)std::min(std::floor(box[d] / rc), 1024.0);
     }
     while ((long long)R.nc[0] * R.nc[1] * R.nc[2] > 2ll * n + 27) {
         int d = R.nc[0] >= R.nc[1] && R.nc[0] >= R.nc[2] ? 0 : (R.nc[1] >= R.nc[2] ? 1 : 2);
         R.nc[d] -= 1;
     }
     if (R.nc[0] < 3 || R.nc[1] < 3 || R.nc[2] < 3) R.nc[0] = R.nc[1] = R.nc[2] = 0;
+    ne_bin64(R, rc);
     R.m = 1.0;
     R.c1 = 1.0;
     R.rlist2 = rc * rc;
