@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(STEP_THREADS)
     const long long s = __ldcg(step_base) + j;  // from L2: the last chunk's end advanced it
     const double* T = B.tot + (size_t)rep * NTOT;
     const bool draw = do_open || !do_close;  // a step follows: its normals
+    const bool prep = !do_open && !do_close;
     // the normals of the coming step, which depend on nothing that a kernel of
     // the chain writes, while pass 2 drains
     R z = 0;
@@ -262,6 +263,9 @@ __global__ void __launch_bounds__(STEP_THREADS)
         }
     }
     if (bad) ne_set_status(B.status, bad);
+    // the list of the sites is built: the first step's list kernel has nothing
+    // to do (pass 1 clears the mark of a build inside the run)
+    if (prep && threadIdx.x == 0 && tile == P.tile0) B.building[rep] = 0;
     if (do_open && threadIdx.x == STEP_THREADS - 32 && tile == P.tile0)
         step_work(B, S, T, rep, s, s_lam[0], s_lam[1]);
     // the tile's partials: UX.. and the normals per component, U2, U_E and KE
