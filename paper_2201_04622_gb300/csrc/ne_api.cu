@@ -368,7 +368,8 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
     B.xi64 = ctx->xi64;
     B.nbr = ctx->nbr;
     B.ncnt = ctx->ncnt;
-    B.sl = ctx->sl;
+    // mixed: neighbour and f'(r)/r in the buffer that FP64 has f'(r)/r in
+    B.sl = md[0].prec == NE_MIXED ? (int*)ctx->gs : ctx->sl;
     B.scnt = ctx->scnt;
     B.cellof = ctx->cellof;
     B.cslot = ctx->cslot;
@@ -673,7 +674,7 @@ ne_status ne_ctx_create(const ne_eam_params* eam, int max_atoms, int max_replica
     A(dalloc(&ctx->xi32, 3 * N));
     A(dalloc(&ctx->nbr, N * NE_NMAX));
     A(dalloc(&ctx->ncnt, N));
-    A(dalloc(&ctx->sl, 2 * N * NE_SMAX));
+    A(dalloc(&ctx->sl, N * NE_SMAX));
     A(dalloc(&ctx->scnt, N));
     A(dalloc(&ctx->cellof, N));
     A(dalloc(&ctx->cslot, N));

@@ -15,8 +15,9 @@
 //   nbr, ncnt           candidate list within r_c + skin: int [N][NE_NMAX] (neighbour and its
 //                       image), count [N]
 //   sl, gs, scnt        the step's pairs inside r_c: neighbour and its image, and f'(r)/r of
-//                       each -- (int, float bits) pairs [N][NE_SMAX] in sl (mixed), int
-//                       [N][NE_SMAX] in sl and double [N][NE_SMAX] in gs (FP64); count [N]
+//                       each -- int [N][NE_SMAX] and double [N][NE_SMAX] (FP64), or (int,
+//                       float bits) pairs [N][NE_SMAX] in sl, which then is gs's buffer (mixed);
+//                       count [N]
 //   partA / partB       partial sums of the pair blocks (pass 1 and 2) and of the
 //                       step kernel's tiles, quantity-major
 //   tot                 per-replica totals formed by the last block of pass 2
