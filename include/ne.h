@@ -152,7 +152,10 @@ ne_status ne_ctx_set_theta(ne_ctx* ctx, const double* theta_dev, void* stream);
 ne_status ne_ctx_get_theta(ne_ctx* ctx, double* theta_dev, void* stream);
 
 /* Tuning of the pair kernels: threads per atom (1, 2, 4 or 8).  Without this
- * call they are chosen by the batch's size (8 to 32). */
+ * call they are chosen by the atoms of the whole batch (32 up to 4096, 16 up to
+ * 16,384, else 8).  The order of an atom's sums follows the choice, so a
+ * replica's results agree to rounding whatever batch it is in, and bit for bit
+ * in batches of either side of those limits only with a choice made here. */
 ne_status ne_ctx_set_tuning(ne_ctx* ctx, int threads_per_atom);
 
 /* CTAs per thread-block cluster of ne_crystal_run_segment (a scheduling
