@@ -192,6 +192,7 @@ void fill_tables(ne_ctx* ctx)
     t.nk = p.n_knots;
     t.h_r = p.r_c / (p.n_knots - 1);
     t.inv_h_r = (p.n_knots - 1) / p.r_c;
+    ne_split_inv_h(t, p.n_knots - 1, p.r_c);
     t.h_rho = p.rho_max / (p.n_knots - 1);
     t.inv_h_rho = (p.n_knots - 1) / p.rho_max;
     t.r_c = p.r_c;

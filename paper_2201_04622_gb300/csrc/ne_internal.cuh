@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 // 32-byte aligned quadruple of doubles (one spline interval in FP64)
 struct __align__(32) ned4 {
     double x, y, z, w;
@@ -124,10 +126,22 @@ struct Tables {
     const ned4* F64;
     int nk;
     double h_r, inv_h_r, h_rho, inv_h_rho;
+    double ih_hi, ih_k, ih_c;  // 1 / h_r = ih_hi (1 + ih_k), ih_hi of 29 bits; (1 + ih_k) / 2
     double r_c, rho_max;
     float inv_h_rf, rcf, rc2f, rmin2f, inv_h_rhof;
     float rho_maxf, ihr_lo;  // inv_h_rho = inv_h_rhof + ihr_lo to double-float precision
 };
+
+// the factors of 1 / h_r = n / r_c, from the rounded quotient and its residue
+inline void ne_split_inv_h(Tables& t, int n, double r_c)
+{
+    const double q = n / r_c;
+    int ex;
+    const double m = std::frexp(q, &ex);
+    t.ih_hi = std::ldexp(std::nearbyint(std::ldexp(m, 29)), ex - 29);
+    t.ih_k = ((q - t.ih_hi) + std::fma(-q, r_c, (double)n) / r_c) / t.ih_hi;
+    t.ih_c = 0.5 + 0.5 * t.ih_k;
+}
 
 struct DevBatch {
     int n_rep, n_tot, n_tiles;

@@ -231,6 +231,7 @@ extern "C" ne_status ne_eam_energy_forces_noalloc(const ne_eam_params* eam, ne_p
     t.nk = nk;
     t.h_r = rc / (nk - 1);
     t.inv_h_r = (nk - 1) / rc;
+    ne_split_inv_h(t, nk - 1, rc);
     t.h_rho = eam->rho_max / (nk - 1);
     t.inv_h_rho = (nk - 1) / eam->rho_max;
     t.r_c = rc;
