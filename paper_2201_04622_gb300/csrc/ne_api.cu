@@ -405,8 +405,9 @@ ne_status setup_batch(ne_ctx* ctx, int n_rep, const int* off, const double* boxe
 ne_status finish(ne_ctx* ctx, cudaStream_t st)
 {
     NE_CU(cudaGetLastError());
-    // the status word goes straight to pinned host memory
-    ne::launch_status_out(ctx->status, ctx->status_host, st);
+    // the status word goes straight to pinned host memory (which holds the last
+    // call's until then: a launch that failed must not pass for it)
+    NE_CU(ne::launch_status_out(ctx->status, ctx->status_host, st));
     NE_CU(cudaStreamSynchronize(st));
     const int bits = *(volatile int*)ctx->status_host;
     ctx->last_bits = bits;

@@ -490,7 +490,7 @@ constexpr int SETUP_REPS = 6;    // replicas a set-up launch takes (their table 
 constexpr int SETUP_MAX = 24;    // replicas up to which the set-up goes by launches
 void launch_setup(const RepDev* reps, int n_rep, RepDev* rep, int* tile_rep, unsigned* tile_done, int* flags,
                   int* status, double* tot, cudaStream_t st);
-void launch_status_out(const int* status, int* host, cudaStream_t st);  // host: pinned
+cudaError_t launch_status_out(const int* status, int* host, cudaStream_t st);  // host: pinned
 void launch_set_step(long long* step_base, long long s, cudaStream_t st);
 void launch_advance(long long* step_base, long long by, cudaStream_t st);
 void launch_noise(unsigned long long seed, unsigned replica, int stream, long long step, int n, int mixed,

@@ -656,7 +656,10 @@ void launch_setup(const RepDev* reps, int n_rep, RepDev* rep, int* tile_rep, uns
     }
 }
 
-void launch_status_out(const int* status, int* host, cudaStream_t st) { ne_launch(k_status_out, 1, 1, 0, st, status, host); }
+cudaError_t launch_status_out(const int* status, int* host, cudaStream_t st)
+{
+    return ne_launch(k_status_out, 1, 1, 0, st, status, host);
+}
 
 void launch_init_velocities(const DevBatch& B, int fix_cm, cudaStream_t st)
 {
