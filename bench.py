@@ -445,10 +445,10 @@ def run_ours(args):
                 # ncu DRAM read + write of one launch of this kernel on this
                 # workload (k_cluster on fl2, a 200-step launch: 2.26 MB read, 0
                 # written; k_brick on rs16, a 200-step launch: 1.85 MB read,
-                # 0.19 MB written); the replicas live on chip or in L2, so the
+                # 0.25 MB written); the replicas live on chip or in L2, so the
                 # figure does not grow with the steps; null elsewhere
                 "traffic": (2.26e6 if args.workload == "fl2" and runner_kind == "cluster" else
-                            2.04e6 if args.workload == "rs16" and runner_kind == "brick" else None),
+                            2.10e6 if args.workload == "rs16" and runner_kind == "brick" else None),
                 "kernel_ms": kern_ms, "us_per_step": kern_ms * 1e3 / K,
                 "peak_note": "%d SMs x %d FP32 lanes x %.0f MHz (median SM clock sampled around the "
                              "timed region)" % (n_sm, FP32_LANES_PER_SM, sm_hz / 1e6),

@@ -16,7 +16,10 @@ from . import ne
 def tune(ctx, mds, offsets, x, v, x0, boxes, W, step_begin=0, n_steps=100,
          threads_per_atom=(1, 2, 4, 8), skins=None):
     """Return (best, table): best = dict(tpa, skin, ms_per_step); table = all
-    candidates.  The state (x, v, W) is restored after every trial."""
+    candidates.  The state (x, v, W) is restored after every trial.  The 32
+    threads per atom that batches up to 4096 atoms have without ne_ctx_set_tuning
+    are not among the candidates (2000 atoms, mixed: 21.9 us a step against 30.4
+    with 8)."""
     rc = ne.ctx_cutoff(ctx)
     if rc is None:
         raise ValueError("context not created through this binding: its cutoff is unknown")

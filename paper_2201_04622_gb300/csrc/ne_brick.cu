@@ -38,8 +38,8 @@
 // hit L1.  The spline window in shared memory starts at 1 A, which leaves L1
 // room for them.  Four bcc 16^3, a step: 29.4 us with every neighbour from L2
 // (long-scoreboard and barrier stalls 5.2 and 5.1 an issue), u and F' apart and
-// barriers of the whole launch; 23.7 us now (2.7 and 3.8).  bcc 32^3: 69.7 and
-// 59.4 us.
+// barriers of the whole launch; 23 us now (2.7 and 3.7).  bcc 32^3: 69.7 and 59.4
+// us, 46 spread over 128 CTAs (its plan's rule is in ne_api.cu).
 //
 // Threads: TPA threads per atom (8, 4, 3, 2 or 1, the largest at which the
 // batch's CTAs fit the device at one CTA per SM); thread t works on slot

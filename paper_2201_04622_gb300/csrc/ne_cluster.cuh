@@ -220,8 +220,9 @@ __device__ __forceinline__ void ne_baro_box(ne_baro_smem& b, const XRep& R, doub
     b.noise = sqrt(2.0 * R.kT * R.mp * dt / V);
 }
 
-// The step's scale factors from the diagonal virial W (double-float per axis,
-// the same in every lane), by lanes 0 .. 2 of one warp; i: the step's place in z
+// The step's scale factors from the diagonal virial W (the same in every lane;
+// double-float per axis, and so added over the axes: 48 bits of sums that FP32
+// pairs leave good to 24), by lanes 0 .. 2 of one warp; i: the step's place in z
 __device__ __forceinline__ void ne_baro_step(ne_baro_smem& b, const XRep& R, const dff (&W)[3], double lam, double dt,
                                              double r_c, int i)
 {

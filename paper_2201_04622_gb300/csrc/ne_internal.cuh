@@ -189,7 +189,7 @@ struct DevBatch {
     double* trace;     // nullable, [rows][8], single replica
     int trace_stride, trace_rows;
     int* flags;        // [n_rep] list rebuild requested (set by the step kernel)
-    int* building;     // [n_rep] rebuild in progress (set by the binning, cleared by pass 1)
+    int* building;     // [n_rep] rebuild in progress (set by the binning, cleared by pass 1 or a run's set-up step)
     unsigned long long* rebuilds;  // count of replica list builds
     int* status;
     Tables tab;
@@ -311,7 +311,7 @@ __device__ __forceinline__ float ne_normal32(uint4 w, int c)
 }
 
 // exp(x) - 1: the Taylor sum for the small arguments of a barostat step
-// (|x| < 1/64: the eighth term is below 2^-60 of the first), else expm1
+// (|x| < 1/64: the eighth term is below 2^-57 of the first), else expm1
 __device__ __forceinline__ double ne_baro_expm1(double x)
 {
     if (fabs(x) >= 0.015625) return expm1(x);
@@ -372,7 +372,9 @@ __device__ __forceinline__ dff dff_warp_sum(dff v)
 // Called by all 32 lanes.  Partials are doubles on the FP64 path and
 // double-float pairs, sixteen loads in flight, on the mixed one (serial FP64
 // adds of a 65,536-atom replica's 2048 partials, 15 quantities in the one
-// finishing block, cost 13 us).
+// finishing block, cost 13 us).  A choice of fewer bits: such a sum of 16 to 2048
+// partials is off by up to 3.4e-15 of it (an FP64 one by 1.5e-16), under terms that
+// FP32 pairs leave at 1e-8 of it; the works are FP64.
 __device__ __forceinline__ double ne_warp_part_sum(const double* part, int nt)
 {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -487,7 +489,10 @@ void launch_pass2(const DevBatch& B, bool mixed, cudaStream_t st);
 void launch_step(const DevBatch& B, const Sched& S, bool mixed, const long long* step_base,
                  int j, int do_close, int do_open, cudaStream_t st);
 constexpr int SETUP_REPS = 6;    // replicas a set-up launch takes (their table is its argument: 4 KB)
-constexpr int SETUP_MAX = 24;    // replicas up to which the set-up goes by launches
+// Replicas up to which the set-up goes by launches, above by copies and clears.  A
+// run of no steps in us by the one and the other: 1 replica 30, 35; 6 38, 45; 12 51,
+// 53; 24 72, 70; 36 94, 86; 72 164, 134
+constexpr int SETUP_MAX = 24;
 void launch_setup(const RepDev* reps, int n_rep, RepDev* rep, int* tile_rep, unsigned* tile_done, int* flags,
                   int* status, double* tot, cudaStream_t st);
 cudaError_t launch_status_out(const int* status, int* host, cudaStream_t st);  // host: pinned

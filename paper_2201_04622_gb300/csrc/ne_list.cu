@@ -1,7 +1,8 @@
 // ne_list.cu -- neighbour-list build of the multi-kernel path.
 //
 // Rebuild of the candidate list of every replica whose flag is set (or of all
-// replicas, when forced), in two launches that return at once when there is
+// replicas, when forced), in two launches (three with a replica above
+// SORT_IN_BLOCK atoms, four of them forced) that return at once when there is
 // nothing to do:
 //   k_nl_cells  reference positions (the lattice sites at the start of a run,
 //               the current positions after an atom strayed more than
@@ -9,7 +10,9 @@
 //               One thread per atom over all SMs; the block that finishes a
 //               replica's last tile forms its cell starts and writes the atoms
 //               sorted by cell, each cell's by index, so the order does not
-//               depend on the atomics;
+//               depend on the atomics.  Replicas above SORT_IN_BLOCK are
+//               sorted, and in a forced build scattered, by launches over all
+//               SMs (k_nl_sort, k_nl_scatter);
 //   k_nl_list   for each atom the atoms of the 27 surrounding cells (all atoms
 //               when the box holds < 3 cells per axis) within r_c + skin,
 //               minimum image, FP32 distances with a 1e-3 A margin so that
@@ -328,7 +331,9 @@ void launch_nl_build(const DevBatch& B, int force, int from_sites, cudaStream_t 
     if (B.n_max > SORT_IN_BLOCK)
         ne_launch(k_nl_sort, (B.n_tiles + 3) / 4, 256, 0, st, B);
     // a warp an atom up to 8192 atoms (a quarter of a million threads, one
-    // wave), eight lanes above: fewer idle lanes at the ends of the short runs
+    // wave), eight lanes above: fewer idle lanes at the ends of the short runs.
+    // Whole mixed energy calls in us with 32 and with 8: 2000 atoms 63-66, 76; 4056
+    // 72, 82; 8192 90, 96; 12,288 109, 102; 16,000 124, 114; 35,152 154, 123
     if (B.n_tot <= 8192)
         ne_launch(k_nl_list<32>, grid(B.n_tiles * (NE_TILE * 32 / LIST_THREADS)), LIST_THREADS, 0, st, B);
     else
